@@ -344,7 +344,7 @@ int wec_load(wec_tank *tank, const void *buf, size_t n);
  * Neumann whatever beta holds there and the top face Dirichlet p = 0 (ghost -p_c,
  * i.e. 2 beta_top p_c).  Preconditioner: one multigrid V(mg_pre, mg_post) cycle
  * (red-black Gauss-Seidel, 2x2 sum restriction, piecewise-constant prolongation,
- * coarse faces = mean of the two fine faces, dense LU on the coarsest level).
+ * coarse faces = mean of the two fine faces, direct solve on the coarsest level).
  * nx, ny >= 2. */
 int wec_poisson_create(int nx, int ny, const wec_solver_opts *opts, void *cuda_stream,
                        wec_poisson **out);
@@ -373,7 +373,7 @@ int wec_poisson_solve(wec_poisson *P, const double *b, double *x, double rtol, i
  * Preconditioner: one V(mg_pre, mg_post) cycle with red-black Gauss-Seidel
  * (colour (i+j+k) mod 2), 2x2x2 sum restriction, piecewise-constant
  * prolongation, coarse face = half the sum of the four fine faces it covers,
- * dense LU on the coarsest level; coarsening halves all three sizes while all
+ * direct solve on the coarsest level; coarsening halves all three sizes while all
  * are even and >= 4, and must end at <= 512 cells.  WEC_PREC_MIXED runs the
  * V-cycle in FP32 (FP32 copies of the hierarchy) inside the FP64 FGMRES.
  * nx, ny >= 2, nz >= 2; every face array below 2^31 entries; otherwise
@@ -519,24 +519,23 @@ double wec_wave_number_fenton_kd(double omega, double depth, double g);
 int wec_jonswap(double Hs, double Tp, double gamma, int ncomp, double *amp, double *omega);
 
 /* ---- process-wide options ------------------------------------------------ */
-/* "mg_fused" (default 1): the multigrid V-cycle runs as one shared-memory tile
+/* "mg_fused" (default 1): the 2D multigrid V-cycle runs as one shared-memory tile
  * kernel per fine level for pre-smoothing + residual + restriction, one for
- * prolongation + post-smoothing, and one single-CTA kernel, staged in shared
- * memory, for the levels of at most 4096 cells; 0 launches one kernel per colour
+ * prolongation + post-smoothing, and one thread-block cluster for the coarse levels
+ * (the first that fits in its shared memory, down); 0 launches one kernel per colour
  * pass, restriction and prolongation.  Both compute the same values up to
  * rounding.  "mg_autotune" (default 1): when a solver is created, time the fused
- * kernels' tile shapes (64x16, 32x16, 32x8, 16x8) on each level and keep the
- * fastest, then time whole V-cycles with the single-CTA kernel starting at the
- * smallest admissible level or one or two levels coarser and keep the fastest;
- * 0 uses 64x16 everywhere and the smallest admissible level.  Tuning results
- * are kept per (grid, precision, mg_pre, mg_post) for the life of the process:
- * later solvers of the same shape reuse them and compute the same bits.
- * "mg_bottom_shift" (default -1 = autotuned): start the single-CTA kernel this
- * many levels below the smallest admissible one (0..8, capped at the coarsest).
- * "mg3_bottom" (default 1): the 3D V-cycle runs its levels of at most 8192
- * cells, down to the coarsest, in one 1024-thread CTA (iterates and right-hand
- * sides in shared memory); 0 launches them level by level.  Both compute the same
- * bits.
+ * kernels' tile shapes (64x16, 32x16, 32x8, 16x8) on each level above the cluster's
+ * and keep the fastest; 0 uses 64x16 everywhere.  Tuning results are kept per (grid,
+ * precision, mg_pre, mg_post) for the life of the process: later solvers of the
+ * same shape reuse them (a tile's shape does not change the bits).
+ * "mg_bottom_shift" (default -1, as 0): start the cluster kernel this many levels
+ * below the first that fits (0..8, capped at the coarsest).
+ * "mg3_bottom" (default 1): the 3D V-cycle runs its coarse levels in one
+ * thread-block cluster (iterates and coefficients in shared memory); 0 launches
+ * them level by level.  Both compute the same bits.  (In both, and in the 2D
+ * cluster kernel, the levels of at most 512 cells are one fixed linear map, formed
+ * with the hierarchy and applied as a matrix.)
  * "tank3_split_momentum" (default 1): the 3D momentum system per component as
  * two kernels (transport terms, then viscous terms and assembly); 0: one
  * kernel.  Both form the same terms: the same bits with double-float stencils,
@@ -549,7 +548,7 @@ int wec_set_option(const char *name, int value);
 /* Fused multigrid tile shape (interior cells) per level of the tank's solver, as
  * chosen by the autotuner when the tank was created ("mg_autotune" option; the
  * coarsest level's entry is meaningless; 0 x 0 marks a level run inside the
- * single-CTA kernel).  *nlev receives the number of levels; at most max entries
+ * cluster kernel).  *nlev receives the number of levels; at most max entries
  * are written. */
 int wec_tank_mg_tiles(const wec_tank *tank, int *tile_x, int *tile_y, int max, int *nlev);
 

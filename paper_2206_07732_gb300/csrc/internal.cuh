@@ -14,8 +14,8 @@ namespace wec {
 constexpr double kPi = 3.14159265358979323846;
 constexpr int kMaxLevels = 24;
 constexpr int kMaxRestart = 32;
-constexpr int kInvMax = 32;         // coarsest levels up to this size also get an explicit inverse
 constexpr int kMaxCoarse = 512;      // cells on the coarsest multigrid level
+constexpr int kDense = 512;          // cells of the finest level whose part of the V-cycle is applied as a matrix
 constexpr int kRedBlocks = 304;      // partial-sum blocks of the step's reductions (2 x 152 SMs)
 constexpr int kRedThreads = 256;
 constexpr int kKrylovBlocks = 912;   // max CTAs of the Krylov reduction kernels (6 x 152 SMs)
@@ -37,7 +37,8 @@ inline int nblk(long long n, int t) { return (int)((n + t - 1) / t); }
 // completed and its writes are visible -- the same ordering as plain stream
 // order -- while the launch itself (launch_k) may be processed before that
 // kernel ends.  No kernel triggers its dependents early: measured, an early
-// trigger let waiting grids take SM slots and slowed the step by 6 %.
+// trigger let waiting grids take SM slots and slowed the step by 6 % (in the
+// solver's single-wave kernels alone: a 2D solve by 6 %).
 __device__ __forceinline__ void pdl_entry()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -116,10 +117,12 @@ struct wec_poisson {
     wec::Level<double> L64[wec::kMaxLevels];
     wec::Level<float> L32[wec::kMaxLevels];
     int ncoarse = 0;
-    double *lu64 = nullptr;
-    float *lu32 = nullptr;
-    double *inv64 = nullptr;  // explicit inverse of the coarsest operator (at most kInvMax cells)
+    double *inv64 = nullptr;  // explicit inverse of the coarsest operator
     float *inv32 = nullptr;
+    void *band = nullptr;     // scratch of its factorisation
+    int dense = 0;            // first level of at most kDense cells: the V-cycle from there down is applied as a matrix
+    double *dense64 = nullptr;  // that matrix, where the level is not the coarsest
+    float *dense32 = nullptr;
     // FGMRES workspace (FP64 outer iteration)
     double *V = nullptr;        // (m+1) x n
     double *Z = nullptr;        // m x n preconditioned vectors (FP64 in both precisions)
@@ -138,8 +141,8 @@ struct wec_poisson {
     double *kdf_d0 = nullptr;   // the diagonal as float pairs
     int tile64[wec::kMaxLevels] = {}, tile32[wec::kMaxLevels] = {};  // fused tile shape per level (autotuned)
     bool tuned = false;
-    int bottom_shift = 0;       // bottom kernel starts this many levels below the smallest admissible one (autotuned)
-    int bottom_level = -1;      // the level the bottom kernel starts at (set by the last fused V-cycle)
+    int bottom_shift = 0;       // the cluster kernel starts this many levels below the first admissible one
+    int bottom_level = -1;      // the level the cluster kernel starts at (set by the last fused V-cycle)
     wec::KState *ks = nullptr;  // device
     wec::KState *ksh = nullptr; // pinned host mirror
     size_t bytes = 0;
@@ -152,7 +155,7 @@ int poisson_init(wec_poisson *P, int nx, int ny, int prec, int restart, int nu1,
                  cudaStream_t st, int nz = 1);
 void poisson_free(wec_poisson *P);
 // Level-0 coefficients already in P->L64[0].bu / bv (/ bw in 3D) (device): build coarse levels,
-// FP32 copies and the coarse LU (enqueued on st).
+// FP32 copies, the coarsest inverse and the dense level's matrix (enqueued on st).
 int poisson_build(wec_poisson *P, cudaStream_t st);
 // Host-polled FGMRES solve on P->st.
 int poisson_solve(wec_poisson *P, const double *b, double *x, double rtol, int maxit, int *iters,
@@ -167,7 +170,7 @@ int solve_result(wec_poisson *P, int *iters, double *relres);
 int poisson_apply(wec_poisson *P, const double *x, double *y);
 void set_mg_fused(bool on);
 void set_mg_autotune(bool on);
-void set_mg_bottom_shift(int shift);  // -1: autotune
+void set_mg_bottom_shift(int shift);  // -1: as 0
 void set_tank3_split_momentum(bool on);
 void set_mg3_bottom(bool on);
 void poisson_tiles(const wec_poisson *P, int *tx, int *ty, int max);

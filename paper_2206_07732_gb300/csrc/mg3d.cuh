@@ -1,14 +1,15 @@
 // Multigrid level kernels of the three-dimensional pressure operator (included
-// by solver.cu inside its anonymous namespace; uses at_sel, k_lu_solve).
+// by solver.cu inside its anonymous namespace; uses at_sel, mg_coarse.cuh, mg_cluster.cuh).
 //
 // Operator and layouts as in poisson_op.cuh (diag3_at / offsum3_at).  Red-black
 // Gauss-Seidel with colour (i + j + k) mod 2, restriction = sum of the eight
 // children's residuals, piecewise-constant prolongation, coarse face = half the
-// sum of the four fine faces it covers, dense LU on the coarsest level.  Every
-// smoothed level has nx, ny, nz even.
+// sum of the four fine faces it covers, a direct solve on the coarsest level.  Every
+// smoothed level has nx, ny, nz even.  From the level of at most kDense cells
+// down the V-cycle is applied as a matrix (mg_cluster.cuh), here too.
 //
 // Cell layouts.  FP64 levels keep x, b and 1/d in the natural order (x fastest).
-// FP32 levels above the coarsest keep x and 1/d -- and b below level 0, whose
+// FP32 levels above the dense one keep x and 1/d -- and b below level 0, whose
 // b is written by the Krylov kernels -- colour-packed: the cells of colour 0,
 // then those of colour 1, each block row by row with i / 2 fastest (pk3).  A
 // one-colour pass then reads and writes only its own colour's x, 1/d and b, in
@@ -102,17 +103,7 @@ __global__ void __launch_bounds__(256) k3_rbgs(int nx, int ny, int nz, const T *
 // the natural order and in OT -- its own cell and the other-colour cell beside
 // it in the row (i ^ 1), whose pass came before -- instead of its packed x
 // (nothing reads that after it), so no separate pass reads it again.
-// (OT: the result's type, FP64, FP32 or float pairs)
-template <typename OT>
-__device__ __forceinline__ OT widen_out(float v)
-{
-    if constexpr (std::is_same<OT, double>::value)
-        return f2d_exact(v);
-    else if constexpr (std::is_same<OT, float>::value)
-        return v;
-    else
-        return OT(v, 0.f);
-}
+// (OT: the result's type, FP64 or FP32)
 // Z1: the black pass of the first pre-smoothing sweep with its red pass folded
 // in (offsum3_pk_z; the red values are not stored: with two or more sweeps the
 // next red pass replaces them before anything reads them).
@@ -325,177 +316,7 @@ __global__ void k3_invdiag(Level3Diag<T> D)
     D.id[l][ix3((D.pk >> l) & 1u, nx, ny, D.nz[l], i, j, k)] = T(1) / diag3_at(D.bx[l], D.by[l], D.bz[l], nx, ny, D.nz[l], i, j, k);
 }
 
-// Dense operator of the coarsest level (n <= kMaxCoarse cells) into A (n x n,
-// zeroed here), then its LU without pivoting (a symmetric M-matrix), one block.
-template <typename T>
-__global__ void k3_lu_factor(int nx, int ny, int nz, const T *__restrict__ bx, const T *__restrict__ by,
-                             const T *__restrict__ bz, T *A)
-{
-    pdl_entry();
-    const int n = nx * ny * nz, pl = nx * ny;
-    for (long long q = threadIdx.x; q < (long long)n * n; q += blockDim.x) A[q] = T(0);
-    __syncthreads();
-    for (int c = threadIdx.x; c < n; c += blockDim.x) {
-        const int r = c / nx, i = c - r * nx, k = r / ny, j = r - k * ny;
-        const int fx = r * (nx + 1) + i, fy = (r + k) * nx + i;
-        T *row = A + (long long)c * n;
-        row[c] = diag3_at(bx, by, bz, nx, ny, nz, i, j, k);
-        if (i > 0) row[c - 1] = -bx[fx];
-        if (i < nx - 1) row[c + 1] = -bx[fx + 1];
-        if (j > 0) row[c - nx] = -by[fy];
-        if (j < ny - 1) row[c + nx] = -by[fy + nx];
-        if (k > 0) row[c - pl] = -bz[c];
-        if (k < nz - 1) row[c + pl] = -bz[c + pl];
-    }
-    __syncthreads();
-    for (int p = 0; p < n; ++p) {
-        const T piv = A[(long long)p * n + p];
-        for (int r = p + 1 + threadIdx.x; r < n; r += blockDim.x) {
-            const T f = A[(long long)r * n + p] / piv;
-            A[(long long)r * n + p] = f;
-            for (int c = p + 1; c < n; ++c) A[(long long)r * n + c] -= f * A[(long long)p * n + c];
-        }
-        __syncthreads();
-    }
-}
-
-// The coarse levels lb .. nlev-1 of a 3D V-cycle in one CTA: the same passes
-// in the same order and per-cell arithmetic as the per-level kernels (so the
-// same bits), each level's iterate and right-hand side in shared memory, the
-// faces and 1/d read through L1 from the hierarchy.  Below a few thousand cells
-// a per-level launch costs ~6 us whatever its size; here a level costs its
-// passes' barriers.  b of level lb is read from bg, its x written to xg.  In
-// shared memory every level is in the natural order; with pk set, the levels
-// above the coarsest are colour-packed in global memory (1/d, bg, xg).
-constexpr int kBottom3Max = 8192;   // cells of the first level run in the CTA
-constexpr int kBottom3Levels = 8;
-constexpr int kBottom3Smem = 227 * 1024;  // dynamic shared memory opted in for k3_bottom
-template <typename T>
-struct Bot3 {
-    int lb, nlev, nu1, nu2, ncoarse, pk;
-    int nx[kBottom3Levels], ny[kBottom3Levels], nz[kBottom3Levels];
-    const T *bx[kBottom3Levels], *by[kBottom3Levels], *bz[kBottom3Levels], *id[kBottom3Levels];
-    const T *lu;
-};
-
-template <typename T>
-__global__ void __launch_bounds__(1024) k3_bottom(Bot3<T> B, const T *__restrict__ bg, T *__restrict__ xg)
-{
-    pdl_entry();
-    extern __shared__ __align__(16) unsigned char k3b_smem[];
-    T *const sm = reinterpret_cast<T *>(k3b_smem);
-    const int nt = blockDim.x, tid = threadIdx.x;
-    const int L = B.nlev - B.lb;  // levels in the CTA (local index 0 = level lb)
-    int off[kBottom3Levels];
-    {
-        int o = 0;
-        for (int q = 0; q < L; ++q) {
-            off[q] = o;
-            o += 2 * B.nx[q] * B.ny[q] * B.nz[q];
-        }
-    }
-    auto X = [&](int q) { return sm + off[q]; };
-    auto Bv = [&](int q) { return sm + off[q] + B.nx[q] * B.ny[q] * B.nz[q]; };
-    const bool pk0 = B.pk && L > 1;  // level lb colour-packed in global memory
-    // natural index of the t-th cell of level lb's global arrays
-    auto nat0 = [&](int t) {
-        if (!pk0) return t;
-        const int nx = B.nx[0], ny = B.ny[0], half = nx >> 1, nh = half * ny * B.nz[0];
-        const int col = t >= nh ? 1 : 0, u = t - col * nh, r = u / half, ih = u - r * half;
-        const int k = r / ny, j = r - k * ny;
-        return r * nx + 2 * ih + ((j + k + col) & 1);
-    };
-    {
-        const int n0 = B.nx[0] * B.ny[0] * B.nz[0];
-        for (int t = tid; t < n0; t += nt) Bv(0)[nat0(t)] = bg[t];
-    }
-    __syncthreads();
-    // one colour of a red-black sweep on local level q (first: from x = 0)
-    auto pass = [&](int q, int color, bool first) {
-        const int nx = B.nx[q], ny = B.ny[q], nz = B.nz[q], half = nx >> 1, nh = half * ny * nz;
-        const bool pq = B.pk && q < L - 1;  // 1/d of this level colour-packed
-        T *x = X(q);
-        const T *b = Bv(q);
-        for (int t = tid; t < nh; t += nt) {
-            const int r = t / half, ih = t - r * half;
-            const int k = r / ny, j = r - k * ny;
-            const int i = 2 * ih + ((j + k + color) & 1);
-            const int c = r * nx + i;
-            const T id = B.id[q][pq ? color * nh + t : c];
-            if (first) {
-                x[c] = (b[c] + T(0)) * id;
-                x[c ^ 1] = T(0);
-            } else {
-                x[c] = (b[c] + offsum3_at(B.bx[q], B.by[q], B.bz[q], x, nx, ny, nz, i, j, k)) * id;
-            }
-        }
-        __syncthreads();
-    };
-    for (int q = 0; q + 1 < L; ++q) {
-        for (int s = 0; s < B.nu1; ++s) {
-            pass(q, 0, s == 0);
-            pass(q, 1, false);
-        }
-        // residual of the eight children into the coarse right-hand side
-        const int nx = B.nx[q], ny = B.ny[q], nz = B.nz[q];
-        const int cx = nx >> 1, cy = ny >> 1, cz = nz >> 1;
-        const T *x = X(q), *b = Bv(q);
-        T *bc = Bv(q + 1);
-        for (int t = tid; t < cx * cy * cz; t += nt) {
-            const int R = t / cx, I = t - R * cx, K = R / cy, J = R - K * cy;
-            T s = T(0);
-            for (int dk = 0; dk < 2; ++dk)
-                for (int dj = 0; dj < 2; ++dj)
-                    for (int di = 0; di < 2; ++di) {
-                        const int i = 2 * I + di, j = 2 * J + dj, k = 2 * K + dk, c = (k * ny + j) * nx + i;
-                        const T d = diag3_at(B.bx[q], B.by[q], B.bz[q], nx, ny, nz, i, j, k);
-                        const T ax = fma3(d, x[c], -offsum3_at(B.bx[q], B.by[q], B.bz[q], x, nx, ny, nz, i, j, k));
-                        s += b[c] - ax;
-                    }
-            bc[t] = s;
-        }
-        __syncthreads();
-    }
-    // coarsest level: the dense LU factors, one warp (the arithmetic of k_lu_solve)
-    if (tid < 32) {
-        const int n = B.ncoarse, lane = tid;
-        const T *A = B.lu, *b = Bv(L - 1);
-        T *x = X(L - 1);
-        for (int r = 0; r < n; ++r) {
-            T s = T(0);
-            for (int c = lane; c < r; c += 32) s += A[(long long)r * n + c] * x[c];
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0) x[r] = b[r] - s;
-            __syncwarp();
-        }
-        for (int r = n - 1; r >= 0; --r) {
-            T s = T(0);
-            for (int c = r + 1 + lane; c < n; c += 32) s += A[(long long)r * n + c] * x[c];
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0) x[r] = (x[r] - s) / A[(long long)r * n + r];
-            __syncwarp();
-        }
-    }
-    __syncthreads();
-    for (int q = L - 2; q >= 0; --q) {
-        const int nx = B.nx[q], ny = B.ny[q], nz = B.nz[q];
-        T *x = X(q);
-        const T *xc = X(q + 1);
-        for (int c = tid; c < nx * ny * nz; c += nt) {
-            const int r = c / nx, i = c - r * nx, k = r / ny, j = r - k * ny;
-            x[c] += xc[((k >> 1) * (ny >> 1) + (j >> 1)) * (nx >> 1) + (i >> 1)];
-        }
-        __syncthreads();
-        for (int s = 0; s < B.nu2; ++s) {
-            pass(q, 0, false);
-            pass(q, 1, false);
-        }
-    }
-    const int n0 = B.nx[0] * B.ny[0] * B.nz[0];
-    for (int t = tid; t < n0; t += nt) xg[t] = X(0)[nat0(t)];
-}
-
-// out (natural order: FP64, FP32 or float pairs) = x of an FP32 level (colour-packed if pk)
+// out (natural order: FP64 or FP32) = x of an FP32 level (colour-packed if pk)
 template <typename TO>
 __global__ void __launch_bounds__(256) k3_unpack(int nx, int ny, int nz, const float *__restrict__ x, int pk, TO *out,
                                                  const int *outsel)
@@ -506,11 +327,11 @@ __global__ void __launch_bounds__(256) k3_unpack(int nx, int ny, int nz, const f
     out = at_sel(out, outsel, (long long)nx * ny * nz);
     const int r = c / nx, i = c - r * nx, k = r / ny, j = r - k * ny;
     const float v = x[ix3(pk, nx, ny, nz, i, j, k)];
-    if constexpr (std::is_same<TO, float>::value) out[c] = v; else out[c] = widen_out<TO>(v);
+    out[c] = widen_out<TO>(v);
 }
 
 // x0 = M^{-1} b0, one V-cycle over the 3D levels L (precision T).  FP32: x0
-// is the level-0 iterate (colour-packed unless level 0 is the coarsest), b0 in
+// is the level-0 iterate (colour-packed unless level 0 is the dense level), b0 in
 // the natural order; xout (nullable): where the last level-0 pass also writes
 // the result in FP64 (osel: its column).  Returns whether it did.
 template <typename T, typename OT = double>
@@ -520,8 +341,8 @@ bool vcycle3_unfused(wec_poisson *P, Level<T> *L, const T *b0, T *x0, const int 
     bool wrote = false;
     const int TB = 256;
     const double ts = sizeof(T);
-    constexpr bool PK = std::is_same<T, float>::value;  // levels above the coarsest colour-packed
-    auto packed = [&](int l) { return PK && l < P->nlev - 1 ? 1 : 0; };
+    constexpr bool PK = std::is_same<T, float>::value;  // levels above the dense one colour-packed
+    auto packed = [&](int l) { return PK && l < P->dense ? 1 : 0; };
     // (the colour-packed kernels take the level-0 vectors unselected: bsel, and
     // xsel when x0 is the FP32 iterate, are null for an FP32 V-cycle)
     // a row of w cells over nb blocks of tx threads (a multiple of 32, at most
@@ -550,16 +371,13 @@ bool vcycle3_unfused(wec_poisson *P, Level<T> *L, const T *b0, T *x0, const int 
                      first, bs, xs);
         }
     };
-    // the coarse levels from lb down run in one CTA (option "mg3_bottom")
+    // the coarse levels from lb down run in one cluster (option "mg3_bottom")
     int lb = P->nlev;
-    if (g_mg3_bottom) {
-        lb = 1;
-        while (lb < P->nlev - 1 && (long long)L[lb].nx * L[lb].ny * L[lb].nz > kBottom3Max) ++lb;
-        size_t sm = 0;
-        for (int l = lb; l < P->nlev; ++l) sm += 2 * sizeof(T) * (size_t)L[l].nx * L[l].ny * L[l].nz;
-        if (P->nlev - lb > kBottom3Levels || lb >= P->nlev || sm > (size_t)kBottom3Smem) lb = P->nlev;
-    }
-    for (int l = 0; l < P->nlev; ++l) {
+    const int end = P->dense;  // from there down the V-cycle is a matrix
+    ClPlan<T> M;
+    size_t smem = 0;
+    if (g_mg3_bottom) lb = cluster_first(P, L, 0, M, smem);
+    for (int l = 0; l <= end; ++l) {
         Level<T> &A = L[l];
         const T *b = l == 0 ? b0 : A.b;
         T *x = l == 0 ? x0 : A.x;
@@ -567,38 +385,25 @@ bool vcycle3_unfused(wec_poisson *P, Level<T> *L, const T *b0, T *x0, const int 
         const double n = (double)A.nx * A.ny * A.nz;
         const double nf = (A.nx + 1.0) * A.ny * A.nz + A.nx * (A.ny + 1.0) * A.nz + A.nx * A.ny * (A.nz + 1.0);
         if (l == lb) {
-            Bot3<T> Bt{};
-            Bt.lb = lb;
-            Bt.nlev = P->nlev;
-            Bt.nu1 = P->nu1;
-            Bt.nu2 = P->nu2;
-            Bt.ncoarse = P->ncoarse;
-            Bt.pk = PK ? 1 : 0;
-            if constexpr (sizeof(T) == 8) Bt.lu = (const T *)P->lu64; else Bt.lu = (const T *)P->lu32;
-            size_t smem = 0;
-            double bytes = 0.0;
-            for (int q = 0; q < P->nlev - lb; ++q) {
-                const Level<T> &C = L[lb + q];
-                Bt.nx[q] = C.nx;
-                Bt.ny[q] = C.ny;
-                Bt.nz[q] = C.nz;
-                Bt.bx[q] = C.bu;
-                Bt.by[q] = C.bv;
-                Bt.bz[q] = C.bw;
-                Bt.id[q] = C.id;
-                const double nq = (double)C.nx * C.ny * C.nz;
-                smem += (size_t)(2 * nq) * sizeof(T);
-                bytes += (nq + (C.nx + 1.0) * C.ny * C.nz + C.nx * (C.ny + 1.0) * C.nz + C.nx * C.ny * (C.nz + 1.0)) * ts;
+            WEC_PROF("mg_cluster", lb, cluster_bytes(P, L, lb), st);
+            M.bpk = lb > 0 ? packed(lb) : 0;
+            M.opk = lb > 0 || (PK && !xout) ? packed(lb) : 0;
+            if (lb > 0) {
+                launch_cluster<T, 3, T>(M, smem, 1, b, nullptr, A.x, nullptr, st);
+            } else if constexpr (PK) {
+                if (xout) {
+                    launch_cluster<T, 3, OT>(M, smem, 1, b, bs, xout, osel, st);
+                    return true;
+                }
+            } else {
+                launch_cluster<T, 3, T>(M, smem, 1, b, bs, x, xs, st);
             }
-            WEC_PROF("mg3_bottom", lb, bytes + 2.0 * n * ts, st);
-            launch_k(k3_bottom<T>, 1, 1024, smem, st, Bt, (const T *)A.b, A.x);
             break;
         }
-        if (l == P->nlev - 1) {
-            T *lu = nullptr;
-            if constexpr (sizeof(T) == 8) lu = (T *)P->lu64; else lu = (T *)P->lu32;
-            WEC_PROF("mg_lu_solve", l, (n * n + 2 * n) * ts, st);
-            launch_k(k_lu_solve<T>, 1, 32, 0, st, (int)n, lu, b, x, bs, xs);
+        if (l == end) {
+            WEC_PROF("mg_coarse_solve", l, (n * n + 2 * n) * ts, st);
+            launch_k(k_coarse_solve<T>, nblk((long long)n, 8), 256, 0, st, (int)n,
+                     end < P->nlev - 1 ? dense_mat<T>(P) : coarse_inv<T>(P), b, x, bs, xs);
             break;
         }
         for (int q = 0; q < P->nu1; ++q)
@@ -630,8 +435,8 @@ bool vcycle3_unfused(wec_poisson *P, Level<T> *L, const T *b0, T *x0, const int 
             }
         }
     }
-    // ascent: from the level above the coarsest, or above the levels the CTA finished
-    for (int l = (lb < P->nlev ? lb : P->nlev - 1) - 1; l >= 0; --l) {
+    // ascent: from the level above the dense one, or above the levels the cluster finished
+    for (int l = (lb < P->nlev ? lb : end) - 1; l >= 0; --l) {
         Level<T> &A = L[l];
         const T *b = l == 0 ? b0 : A.b;
         T *x = l == 0 ? x0 : A.x;
@@ -675,18 +480,12 @@ void vcycle3_t(wec_poisson *P, Level<T> *L, const T *b0, TO *x0, const int *bsel
         static_assert(std::is_same<TO, double>::value, "an FP64 V-cycle delivers FP64");
         vcycle3_unfused<T>(P, L, b0, x0, bsel, xsel, st);
     } else {
-        // the natural-order result (FP64, FP32 or float pairs) is written by the
-        // last level-0 pass where there is one
-        if constexpr (std::is_same<TO, float>::value) {
-            if (x0 == L[0].x) {
-                vcycle3_unfused<T>(P, L, b0, L[0].x, bsel, nullptr, st);
-                return;
-            }
-        }
+        // the natural-order result (FP64 or FP32) is written by the last level-0
+        // pass, or the cluster kernel, where there is one
         if (vcycle3_unfused<T, TO>(P, L, b0, L[0].x, bsel, nullptr, st, x0, xsel)) return;
         const long long n = (long long)L[0].nx * L[0].ny * L[0].nz;
         WEC_PROF("convert", 0, (4.0 + sizeof(TO)) * n, st);
         launch_k(k3_unpack<TO>, nblk(n, 256), 256, 0, st, L[0].nx, L[0].ny, L[0].nz, (const float *)L[0].x,
-                 P->nlev > 1 ? 1 : 0, x0, xsel);
+                 P->dense > 0 ? 1 : 0, x0, xsel);
     }
 }

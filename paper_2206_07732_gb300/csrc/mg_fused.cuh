@@ -10,9 +10,8 @@
 //               neighbour), so after 2 nu1 passes the tile and one ring around
 //               it are exact, which is what the residual needs.  Halo cells are
 //               recomputed redundantly.
-//   k_mg_bottom one CTA for all levels of at most kBottomCells cells, staged in
-//               shared memory, down to the dense LU of the coarsest level and
-//               back up, with __syncthreads() between colour passes.
+//   k_mg_cluster (mg_cluster.cuh) the coarse levels, down to the coarsest level's
+//               solve and back up.
 //   k_mg_post   per fine level: prolongation + correction and nu2 sweeps, same
 //               tiling.
 // A cell update is x = (b + sum_f beta_f x_nb) * (1 / d) with the reciprocal of
@@ -32,9 +31,6 @@ namespace {
 constexpr int kNumTiles = 4;
 constexpr int kTileX[kNumTiles] = {64, 32, 32, 16};
 constexpr int kTileY[kNumTiles] = {16, 16, 8, 8};
-constexpr int kBottomCells = 4096;      // levels up to this size run inside one CTA (shared memory)
-constexpr int kBottomSmemMax = 200 * 1024;
-constexpr int kBottomThreads = 1024;
 
 // q = k / d for 0 <= k < 2^16, 2 <= d < 2^16 by one multiply-high with m = magic_u16(d):
 // with m = floor(2^32 / d) + 1 the error term k (m - 2^32 / d) / 2^32 < 2^-16 < 1 / d.
@@ -219,210 +215,6 @@ __global__ void __launch_bounds__(256) k_mg_post(int nx, int ny, const T *__rest
     for (int k = threadIdx.x; k < kTX * kTY; k += blockDim.x) {
         int li = H + k % kTX, lj = H + k / kTX, gi = t.gx0 + li, gj = t.gy0 + lj;
         if (gi < nx && gj < ny) x[gj * nx + gi] = TO(t.x[lj * t.ex + li]);
-    }
-}
-
-template <typename T>
-struct BottomLevels {
-    int lb, nlev, nu1, nu2;
-    int nx[kMaxLevels], ny[kMaxLevels];
-    const T *bu[kMaxLevels], *bv[kMaxLevels];
-    T *x[kMaxLevels], *b[kMaxLevels];
-    const T *id[kMaxLevels];
-    const T *lu;
-    const T *inv;  // explicit inverse of the coarsest operator, or nullptr (use lu)
-    double *x0d;  // when set (lb = 0, FP32 levels): level-0 result stored widened here instead of x[0]
-};
-
-// The coarsest level's explicit inverse (n <= kInvMax), or else its LU, is
-// staged in shared memory when it takes at most 16 KB (n <= 64 cells in FP32, 45
-// in FP64); a larger LU is read from global.
-template <typename T>
-__host__ __device__ inline bool lu_staged(const BottomLevels<T> &L)
-{
-    const long long n = (long long)L.nx[L.nlev - 1] * L.ny[L.nlev - 1];
-    return L.inv || n * n * (long long)sizeof(T) <= 16 * 1024;
-}
-
-template <typename T>
-__host__ __device__ inline long long level_elems(const BottomLevels<T> &L, int l)
-{
-    return 3LL * L.nx[l] * L.ny[l] + (long long)(L.nx[l] + 1) * L.ny[l] + (long long)L.nx[l] * (L.ny[l] + 1);
-}
-
-// Shared-memory elements the bottom kernel stages for levels lb.. (x, b, 1/d,
-// bu, bv each) and, when staged, the coarsest LU.
-template <typename T>
-__host__ __device__ inline long long bottom_elems(const BottomLevels<T> &L, int lb)
-{
-    long long e = 0;
-    for (int l = lb; l < L.nlev; ++l) e += level_elems(L, l);
-    if (lu_staged(L)) {
-        const long long n = (long long)L.nx[L.nlev - 1] * L.ny[L.nlev - 1];
-        e += n * n;
-    }
-    return e;
-}
-
-// One colour pass of a level held in shared memory by the whole CTA (nx even).
-// first: from x = 0 (the other colour is set to zero alongside).
-template <typename T>
-__device__ void sm_pass(int nx, int ny, const T *bu, const T *bv, const T *id, T *x, const T *b, int color,
-                        bool first)
-{
-    const int half = nx >> 1;
-    const unsigned mh = magic_u16(half);
-    for (int k = threadIdx.x; k < half * ny; k += blockDim.x) {
-        const int j = div_u16(k, mh);
-        const int i = 2 * (k - j * half) + ((j & 1) ^ color);
-        const int c = j * nx + i;
-        if (first) {
-            x[c] = b[c] * id[c];
-            x[c + (i & 1 ? -1 : 1)] = T(0);
-        } else {
-            x[c] = (b[c] + offsum_at(bu, bv, x, nx, ny, i, j)) * id[c];
-        }
-    }
-    __syncthreads();
-}
-
-// Levels lb .. nlev-1 of the V-cycle in one CTA, all staged in shared memory:
-// load b of level lb and every level's coefficients, smooth / restrict down to
-// the dense LU of the coarsest level, prolong / smooth back up, store x of level lb.
-template <typename T>
-__global__ void __launch_bounds__(kBottomThreads) k_mg_bottom(BottomLevels<T> L, const int *bsel,
-                                                               const int *xsel)
-{
-    pdl_entry();
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ long long off[kMaxLevels + 1];
-    const int lb = L.lb, last = L.nlev - 1;
-    if (threadIdx.x == 0) {
-        long long o = 0;
-        for (int l = lb; l < L.nlev; ++l) {
-            off[l] = o;
-            o += level_elems(L, l);
-        }
-        off[kMaxLevels] = o;  // the staged LU
-    }
-    __syncthreads();
-    T *sm = reinterpret_cast<T *>(smem_raw);
-    auto X = [&](int l) { return sm + off[l]; };
-    auto B = [&](int l) { return sm + off[l] + (long long)L.nx[l] * L.ny[l]; };
-    auto ID = [&](int l) { return sm + off[l] + 2LL * L.nx[l] * L.ny[l]; };
-    auto BU = [&](int l) { return sm + off[l] + 3LL * L.nx[l] * L.ny[l]; };
-    auto BV = [&](int l) { return sm + off[l] + 3LL * L.nx[l] * L.ny[l] + (long long)(L.nx[l] + 1) * L.ny[l]; };
-    // stage b of level lb, every level's coefficients and the LU, all copies in flight at once
-    {
-        const long long n = (long long)L.nx[lb] * L.ny[lb];
-        const T *bg = lb == 0 ? at_sel((const T *)L.b[lb], bsel, n) : L.b[lb];
-        T *sb = B(lb);
-        for (int k = threadIdx.x; k < n; k += blockDim.x) cp_async_el(sb + k, bg + k);
-    }
-    for (int l = lb; l < L.nlev; ++l) {
-        const int nx = L.nx[l], ny = L.ny[l];
-        T *su = BU(l), *sv = BV(l);
-        const T *gu = L.bu[l], *gv = L.bv[l];
-        for (int k = threadIdx.x; k < (nx + 1) * ny; k += blockDim.x) cp_async_el(su + k, gu + k);
-        for (int k = threadIdx.x; k < nx * (ny + 1); k += blockDim.x) cp_async_el(sv + k, gv + k);
-        T *sid = ID(l);
-        const T *gid = L.id[l];
-        for (int k = threadIdx.x; k < nx * ny; k += blockDim.x) cp_async_el(sid + k, gid + k);
-    }
-    // the coarsest level's explicit inverse, or its LU when that is staged
-    const int nlu = L.nx[last] * L.ny[last];
-    const T *csrc = L.inv ? L.inv : L.lu;
-    const bool c_sm = lu_staged(L);
-    const T *lu = c_sm ? sm + off[kMaxLevels] : L.lu;
-    if (c_sm)
-        for (int k = threadIdx.x; k < nlu * nlu; k += blockDim.x) cp_async_el(sm + off[kMaxLevels] + k, csrc + k);
-    cp_async_wait_all();
-    __syncthreads();
-    for (int l = lb; l < last; ++l) {
-        const int nx = L.nx[l], ny = L.ny[l];
-        T *x = X(l), *b = B(l), *su = BU(l), *sv = BV(l), *id = ID(l);
-        for (int q = 0; q < L.nu1; ++q) {
-            sm_pass(nx, ny, su, sv, id, x, b, 0, q == 0);
-            sm_pass(nx, ny, su, sv, id, x, b, 1, false);
-        }
-        const int ncx = nx >> 1, ncy = ny >> 1;
-        const unsigned mc = magic_u16(ncx);
-        T *bc = B(l + 1);
-        for (int k = threadIdx.x; k < ncx * ncy; k += blockDim.x) {
-            const int J = div_u16(k, mc), I = k - J * ncx;
-            T r[4];
-            int qq = 0;
-            for (int dj = 0; dj < 2; ++dj)
-                for (int di = 0; di < 2; ++di) {
-                    int i = 2 * I + di, j = 2 * J + dj, c = j * nx + i;
-                    T d = diag_at(su, sv, nx, ny, i, j);
-                    T ax = d * x[c] - offsum_at(su, sv, x, nx, ny, i, j);
-                    r[qq++] = b[c] - ax;
-                }
-            bc[k] = ((r[0] + r[1]) + r[2]) + r[3];
-        }
-        __syncthreads();
-    }
-    if (L.inv) {
-        // x = A^{-1} b: one warp per row, lanes over columns, fixed shuffle tree
-        const int n = nlu;
-        T *x = X(last);
-        const T *b = B(last);
-        const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-        for (int r = w; r < n; r += kBottomThreads / 32) {
-            T s = lane < n ? lu[r * n + lane] * b[lane] : T(0);
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0) x[r] = s;
-        }
-        __syncthreads();
-    } else {
-        const int n = nlu;
-        T *x = X(last);
-        const T *b = B(last);
-        if (threadIdx.x < 32) {
-            const int lane = threadIdx.x;
-            for (int r = 0; r < n; ++r) {
-                T s = T(0);
-                for (int c = lane; c < r; c += 32) s += lu[(long long)r * n + c] * x[c];
-                for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-                if (lane == 0) x[r] = b[r] - s;
-                __syncwarp();
-            }
-            for (int r = n - 1; r >= 0; --r) {
-                T s = T(0);
-                for (int c = r + 1 + lane; c < n; c += 32) s += lu[(long long)r * n + c] * x[c];
-                for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-                if (lane == 0) x[r] = (x[r] - s) / lu[(long long)r * n + r];
-                __syncwarp();
-            }
-        }
-        __syncthreads();
-    }
-    for (int l = last - 1; l >= lb; --l) {
-        const int nx = L.nx[l], ny = L.ny[l];
-        T *x = X(l), *b = B(l), *su = BU(l), *sv = BV(l), *id = ID(l);
-        const T *xc = X(l + 1);
-        const unsigned mx = magic_u16(nx);
-        for (int k = threadIdx.x; k < nx * ny; k += blockDim.x) {
-            const int j = div_u16(k, mx), i = k - j * nx;
-            x[k] += xc[(j >> 1) * (nx >> 1) + (i >> 1)];
-        }
-        __syncthreads();
-        for (int q = 0; q < L.nu2; ++q) {
-            sm_pass(nx, ny, su, sv, id, x, b, 0, false);
-            sm_pass(nx, ny, su, sv, id, x, b, 1, false);
-        }
-    }
-    {
-        const long long n = (long long)L.nx[lb] * L.ny[lb];
-        const T *x = X(lb);
-        if (lb == 0 && L.x0d) {
-            double *xg = at_sel(L.x0d, xsel, n);
-            for (int k = threadIdx.x; k < n; k += blockDim.x) xg[k] = double(x[k]);
-        } else {
-            T *xg = lb == 0 ? at_sel(L.x[lb], xsel, n) : L.x[lb];
-            for (int k = threadIdx.x; k < n; k += blockDim.x) xg[k] = x[k];
-        }
     }
 }
 

@@ -7,7 +7,7 @@
 // left/right/bottom walls Neumann, the top face Dirichlet p = 0 (ghost -p_c).
 // Multigrid: red-black Gauss-Seidel, sum-of-four restriction of the residual,
 // piecewise-constant prolongation, coarse face coefficient = mean of the two
-// fine faces it covers, dense LU on the coarsest level (<= 512 cells).
+// fine faces it covers, direct solve on the coarsest level (<= 512 cells).
 // Mixed precision: the V-cycle runs in FP32 on FP32 copies of the hierarchy;
 // the Krylov basis, Hessenberg, residuals and the solution stay FP64.
 #include <algorithm>
@@ -179,60 +179,6 @@ __global__ void k_convert(long long n, const TI *__restrict__ in, TO *__restrict
         out[c] = TO(in[c]);
 }
 
-// Dense LU of the coarsest operator (no pivoting: A is a symmetric M-matrix).
-// One block; the matrix lives in global memory (n <= 512).  inv (n <= kInvMax,
-// else nullptr): also A^{-1}, column t by thread t from the two triangular solves.
-template <typename T>
-__global__ void k_lu_factor(int nx, int ny, const T *__restrict__ bu, const T *__restrict__ bv, T *A, T *inv)
-{
-    pdl_entry();
-    // small systems (n <= 64) are built, factored and inverted in shared memory
-    constexpr int kSmallN = 64;
-    __shared__ T Ms[kSmallN * kSmallN];
-    __shared__ T Is[kInvMax * kInvMax];
-    const int n = nx * ny;
-    const bool small = n <= kSmallN;
-    T *M = small ? Ms : A;
-    for (long long q = threadIdx.x; q < (long long)n * n; q += blockDim.x) M[q] = T(0);
-    __syncthreads();
-    for (int r = threadIdx.x; r < n; r += blockDim.x) {
-        int i = r % nx, j = r / nx;
-        M[(long long)r * n + r] = diag_at(bu, bv, nx, ny, i, j);
-        if (i > 0) M[(long long)r * n + r - 1] = -bu[j * (nx + 1) + i];
-        if (i < nx - 1) M[(long long)r * n + r + 1] = -bu[j * (nx + 1) + i + 1];
-        if (j > 0) M[(long long)r * n + r - nx] = -bv[j * nx + i];
-        if (j < ny - 1) M[(long long)r * n + r + nx] = -bv[(j + 1) * nx + i];
-    }
-    __syncthreads();
-    for (int k = 0; k < n; ++k) {
-        T piv = M[(long long)k * n + k];
-        for (int r = k + 1 + threadIdx.x; r < n; r += blockDim.x) {
-            T f = M[(long long)r * n + k] / piv;
-            M[(long long)r * n + k] = f;
-            for (int c = k + 1; c < n; ++c) M[(long long)r * n + c] -= f * M[(long long)k * n + c];
-        }
-        __syncthreads();
-    }
-    if (small)
-        for (int q = threadIdx.x; q < n * n; q += blockDim.x) A[q] = M[q];
-    if (!inv) return;  // inv is given only for n <= kInvMax
-    const int t = threadIdx.x;
-    if (t < n) {
-        for (int r = 0; r < n; ++r) {  // L y = e_t (unit lower), y in column t of Is
-            T s = r == t ? T(1) : T(0);
-            for (int c = 0; c < r; ++c) s -= M[(long long)r * n + c] * Is[c * n + t];
-            Is[r * n + t] = s;
-        }
-        for (int r = n - 1; r >= 0; --r) {  // U x = y
-            T s = Is[r * n + t];
-            for (int c = r + 1; c < n; ++c) s -= M[(long long)r * n + c] * Is[c * n + t];
-            Is[r * n + t] = s / M[(long long)r * n + r];
-        }
-    }
-    __syncthreads();
-    for (int q = threadIdx.x; q < n * n; q += blockDim.x) inv[q] = Is[q];
-}
-
 // 1/d of every cell of levels 0..nlev-1 (one launch; thread per cell of the
 // concatenated levels, level found from the prefix offsets).
 template <typename T>
@@ -256,31 +202,6 @@ __global__ void k_invdiag(LevelDiag<T> D)
     D.id[l][c] = T(1) / diag_at(D.bu[l], D.bv[l], nx, D.ny[l], i, j);
 }
 
-// x = U^{-1} L^{-1} b, one warp.
-template <typename T>
-__global__ void k_lu_solve(int n, const T *__restrict__ A, const T *__restrict__ b, T *__restrict__ x,
-                           const int *bsel, const int *xsel)
-{
-    pdl_entry();
-    int lane = threadIdx.x;
-    b = at_sel(b, bsel, n);
-    x = at_sel(x, xsel, n);
-    for (int r = 0; r < n; ++r) {
-        T s = T(0);
-        for (int c = lane; c < r; c += 32) s += A[(long long)r * n + c] * x[c];
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) x[r] = b[r] - s;
-        __syncwarp();
-    }
-    for (int r = n - 1; r >= 0; --r) {
-        T s = T(0);
-        for (int c = r + 1 + lane; c < n; c += 32) s += A[(long long)r * n + c] * x[c];
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) x[r] = (x[r] - s) / A[(long long)r * n + r];
-        __syncwarp();
-    }
-}
-
 }  // namespace
 }  // namespace wec
 
@@ -290,8 +211,20 @@ namespace wec {
 namespace {
 
 bool g_mg_fused = true;  // fused V-cycle kernels (wec_set_option "mg_fused")
-bool g_mg3_bottom = true;  // the 3D coarse levels in one CTA (wec_set_option "mg3_bottom")
+bool g_mg3_bottom = true;  // the 3D coarse levels in one cluster (wec_set_option "mg3_bottom")
 
+// an FP32 value in the result's type (FP64 and FP32 V-cycles: OT = T too)
+template <typename OT, typename T>
+__device__ __forceinline__ OT widen_out(T v)
+{
+    if constexpr (std::is_same<OT, T>::value)
+        return v;
+    else
+        return f2d_exact(v);
+}
+
+#include "mg_coarse.cuh"
+#include "mg_cluster.cuh"
 #include "mg3d.cuh"
 
 // --------------------------------------------------- Krylov (FP64 outer) ----
@@ -875,10 +808,9 @@ void vcycle_unfused(wec_poisson *P, Level<T> *L, const T *b0, T *x0, const int *
         const int *bs = l == 0 ? bsel : nullptr, *xs = l == 0 ? xsel : nullptr;
         const double n = (double)A.nx * A.ny, nf = (double)(A.nx + 1) * A.ny + (double)A.nx * (A.ny + 1);
         if (l == P->nlev - 1) {
-            T *lu = nullptr;
-            if constexpr (sizeof(T) == 8) lu = (T *)P->lu64; else lu = (T *)P->lu32;
-            WEC_PROF("mg_lu_solve", l, (n * n + 2 * n) * ts, st);
-            launch_k(k_lu_solve<T>, 1, 32, 0, st, A.nx * A.ny, lu, b, x, bs, xs);
+            const int nc = A.nx * A.ny;
+            WEC_PROF("mg_coarse_solve", l, (n * n + 2 * n) * ts, st);
+            launch_k(k_coarse_solve<T>, nblk(nc, 8), 256, 0, st, nc, coarse_inv<T>(P), b, x, bs, xs);
             break;
         }
         int nh = (A.nx >> 1) * A.ny;
@@ -984,8 +916,8 @@ void launch_post(int tile, const Level<T> &A, const T *b, TO *x, const T *xc, in
     }
 }
 
-// Fused V-cycle: per fine level one pre and one post kernel, one CTA for the
-// levels of at most kBottomCells cells.  The level-0 result x0 is stored in TO.
+// Fused V-cycle: per fine level one pre and one post kernel, one cluster for the
+// coarse levels.  The level-0 result x0 is stored in TO.
 template <typename T, typename TO>
 void vcycle_fused(wec_poisson *P, Level<T> *L, const T *b0, TO *x0, const int *bsel, const int *xsel,
                   cudaStream_t st)
@@ -993,39 +925,9 @@ void vcycle_fused(wec_poisson *P, Level<T> *L, const T *b0, TO *x0, const int *b
     const double ts = sizeof(T);
     const int H = 2 * std::max(P->nu1, P->nu2);
     const int *tiles = sizeof(T) == 8 ? P->tile64 : P->tile32;
-    BottomLevels<T> B;
-    B.nlev = P->nlev;
-    B.nu1 = P->nu1;
-    B.nu2 = P->nu2;
-    if constexpr (sizeof(T) == 8) {
-        B.lu = (const T *)P->lu64;
-        B.inv = (const T *)P->inv64;
-    } else {
-        B.lu = (const T *)P->lu32;
-        B.inv = (const T *)P->inv32;
-    }
-    for (int l = 0; l < P->nlev; ++l) {
-        B.nx[l] = L[l].nx;
-        B.ny[l] = L[l].ny;
-        B.bu[l] = L[l].bu;
-        B.bv[l] = L[l].bv;
-        B.id[l] = L[l].id;
-        B.x[l] = l == 0 ? nullptr : L[l].x;
-        B.b[l] = l == 0 ? (T *)b0 : L[l].b;
-    }
-    if constexpr (std::is_same<T, TO>::value) {
-        B.x[0] = x0;
-        B.x0d = nullptr;
-    } else {
-        B.x0d = x0;  // FP32 levels, FP64 level-0 result
-    }
-    // first level small enough, whose staging (with all coarser levels) fits in shared memory
-    int lb = 0;
-    while (lb < P->nlev - 1 &&
-           ((long long)L[lb].nx * L[lb].ny > kBottomCells || bottom_elems(B, lb) * (long long)sizeof(T) > kBottomSmemMax))
-        ++lb;
-    lb = std::min(lb + P->bottom_shift, P->nlev - 1);  // autotuned: coarser levels may run faster in one CTA
-    B.lb = lb;
+    ClPlan<T> M;
+    size_t smem = 0;
+    const int lb = cluster_first(P, L, std::max(P->bottom_shift, 0), M, smem);
     P->bottom_level = lb;
     for (int l = 0; l < lb; ++l) {
         Level<T> &A = L[l];
@@ -1034,13 +936,11 @@ void vcycle_fused(wec_poisson *P, Level<T> *L, const T *b0, TO *x0, const int *b
         launch_pre<T>(tiles[l], A, l == 0 ? b0 : A.b, L[l + 1].b, P->nu1, H, l == 0 ? bsel : nullptr, st);
     }
     {
-        // algorithmic bytes: b and x of level lb, every level's coefficients, the LU
-        const double nb = (double)L[lb].nx * L[lb].ny, nc = (double)L[P->nlev - 1].nx * L[P->nlev - 1].ny;
-        double bytes = (2.0 * nb + nc * nc) * ts;
-        for (int l = lb; l < P->nlev; ++l) bytes += ((L[l].nx + 1.0) * L[l].ny + L[l].nx * (L[l].ny + 1.0)) * ts;
-        const size_t smem_b = (size_t)bottom_elems(B, lb) * sizeof(T);
-        WEC_PROF("mg_bottom", lb, bytes, st);
-        launch_k(k_mg_bottom<T>, 1, kBottomThreads, smem_b, st, B, bsel, xsel);
+        WEC_PROF("mg_cluster", lb, cluster_bytes(P, L, lb), st);
+        if (lb == 0)
+            launch_cluster<T, 2, TO>(M, smem, 1, b0, bsel, x0, xsel, st);
+        else
+            launch_cluster<T, 2, T>(M, smem, 1, (const T *)L[lb].b, nullptr, L[lb].x, nullptr, st);
     }
     for (int l = lb - 1; l >= 0; --l) {
         Level<T> &A = L[l];
@@ -1054,9 +954,9 @@ void vcycle_fused(wec_poisson *P, Level<T> *L, const T *b0, TO *x0, const int *b
 }
 
 bool g_mg_autotune = true;     // wec_set_option "mg_autotune"
-int g_mg_bottom_shift = -1;    // wec_set_option "mg_bottom_shift" (-1: autotune)
+int g_mg_bottom_shift = -1;    // wec_set_option "mg_bottom_shift" (-1: the smallest admissible level)
 
-// Autotuner of the fused level kernels: on each non-coarsest level, time the
+// Autotuner of the fused level kernels: on each level above the cluster kernel's, time the
 // pre + post pair of every tile shape (3 runs each, CUDA events on the solver's
 // stream) and keep the fastest.  Runs once per solver, on placeholder
 // coefficients (all 1), before anything is captured.
@@ -1068,7 +968,7 @@ int autotune_levels(wec_poisson *P, Level<T> *L, int *tiles, cudaStream_t st)
     WEC_CK(cudaEventCreate(&e0));
     WEC_CK(cudaEventCreate(&e1));
     int rc = WEC_OK;
-    for (int l = 0; l + 1 < P->nlev && rc == WEC_OK; ++l) {
+    for (int l = 0; l < P->bottom_level && rc == WEC_OK; ++l) {
         Level<T> &A = L[l];
         const long long n = (long long)A.nx * A.ny;
         T *b = l == 0 ? (T *)P->w : A.b;  // scratch stand-ins for the level-0 vectors
@@ -1104,47 +1004,6 @@ int autotune_levels(wec_poisson *P, Level<T> *L, int *tiles, cudaStream_t st)
     return rc;
 }
 
-// Where the single-CTA bottom starts: time whole fused V-cycles with the bottom
-// at the smallest admissible level and up to two levels coarser (tiled kernels
-// above it), keep the fastest.  Runs after the tile shapes are tuned.
-template <typename T>
-int autotune_bottom(wec_poisson *P, Level<T> *L, cudaStream_t st)
-{
-    cudaEvent_t e0, e1;
-    WEC_CK(cudaEventCreate(&e0));
-    WEC_CK(cudaEventCreate(&e1));
-    // level-0 stand-ins in V (at least 2 n doubles; overwritten at the start of every solve)
-    const long long n0 = (long long)L[0].nx * L[0].ny;
-    T *b = (T *)P->V, *x = (T *)P->V + n0;
-    float best = 1e30f;
-    int best_shift = 0;
-    for (int shift = 0; shift <= 2; ++shift) {
-        P->bottom_shift = shift;
-        vcycle_fused<T, T>(P, L, b, x, nullptr, nullptr, st);  // sets bottom_level
-        if (shift > 0 && P->bottom_level >= P->nlev - 1) break;
-        float tmin = 1e30f;
-        for (int r = 0; r < 4; ++r) {
-            cudaEventRecord(e0, st);
-            vcycle_fused<T, T>(P, L, b, x, nullptr, nullptr, st);
-            cudaEventRecord(e1, st);
-            if (cudaEventSynchronize(e1) != cudaSuccess) break;
-            float ms = 0.f;
-            cudaEventElapsedTime(&ms, e0, e1);
-            tmin = std::min(tmin, ms);
-        }
-        if (tmin < best) {
-            best = tmin;
-            best_shift = shift;
-        }
-    }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    P->bottom_shift = best_shift;
-    vcycle_fused<T, T>(P, L, b, x, nullptr, nullptr, st);  // records the chosen bottom level
-    const cudaError_t ce = cudaGetLastError();
-    return ce == cudaSuccess ? WEC_OK : cuda_fail(ce, "autotune_bottom");
-}
-
 template <typename T>
 __global__ void k_fill(long long n, T *a, T v)
 {
@@ -1155,11 +1014,9 @@ __global__ void k_fill(long long n, T *a, T v)
 
 // Tuning results per (nx, ny, precision, nu1, nu2), shared by every solver of
 // the process: the first solver of a shape times the candidates, later ones
-// reuse its choices, so equal tanks run the same kernels and give the same bits
-// (the bottom split changes rounding; timings alone would not repeat).
+// reuse its choices.
 struct TuneResult {
     int tile[kMaxLevels];
-    int bottom_shift, bottom_level;
 };
 std::mutex g_tune_mu;
 std::map<std::tuple<int, int, int, int, int>, TuneResult> g_tune_cache;
@@ -1168,15 +1025,20 @@ int poisson_autotune(wec_poisson *P, cudaStream_t st)
 {
     for (int l = 0; l < kMaxLevels; ++l) P->tile64[l] = P->tile32[l] = 0;
     P->bottom_shift = g_mg_bottom_shift > 0 ? g_mg_bottom_shift : 0;
-    if (!g_mg_autotune || P->nlev < 2) return WEC_OK;
+    {  // the levels from here on are the cluster kernel's
+        size_t smem = 0;
+        ClPlan<double> M64;
+        ClPlan<float> M32;
+        P->bottom_level = P->prec == WEC_PREC_FP64 ? cluster_first(P, P->L64, P->bottom_shift, M64, smem)
+                                                   : cluster_first(P, P->L32, P->bottom_shift, M32, smem);
+    }
+    if (!g_mg_autotune || P->bottom_level < 1) return WEC_OK;
     std::lock_guard<std::mutex> lk(g_tune_mu);
     const auto key = std::make_tuple(P->nx, P->ny, P->prec, P->nu1, P->nu2);
     int *tiles = P->prec == WEC_PREC_FP64 ? P->tile64 : P->tile32;
     auto hit = g_tune_cache.find(key);
     if (hit != g_tune_cache.end()) {
         for (int l = 0; l < kMaxLevels; ++l) tiles[l] = hit->second.tile[l];
-        P->bottom_shift = g_mg_bottom_shift >= 0 ? g_mg_bottom_shift : hit->second.bottom_shift;
-        P->bottom_level = g_mg_bottom_shift >= 0 ? -1 : hit->second.bottom_level;
         P->tuned = true;
         return WEC_OK;
     }
@@ -1190,23 +1052,15 @@ int poisson_autotune(wec_poisson *P, cudaStream_t st)
             launch_k(k_fill<float>, nblk(nv, 256), 256, 0, st, nv, P->L32[l].bv, 1.0f);
         }
     }
-    // the placeholder operator's hierarchy, diagonals and coarsest factors, so the
+    // the placeholder operator's hierarchy, diagonals and coarsest inverse, so the
     // trial V-cycles run on finite values
     if (int e = poisson_build(P, st)) return e;
     int e = P->prec == WEC_PREC_FP64 ? autotune_levels<double>(P, P->L64, P->tile64, st)
                                      : autotune_levels<float>(P, P->L32, P->tile32, st);
-    if (!e && g_mg_bottom_shift < 0)
-        e = P->prec == WEC_PREC_FP64 ? autotune_bottom<double>(P, P->L64, st) : autotune_bottom<float>(P, P->L32, st);
     if (e) return e;
-    if (g_mg_bottom_shift < 0) {  // a forced split is not a tuning result
-        TuneResult r;
-        for (int l = 0; l < kMaxLevels; ++l) r.tile[l] = tiles[l];
-        r.bottom_shift = P->bottom_shift;
-        r.bottom_level = P->bottom_level;
-        g_tune_cache[key] = r;
-    } else {
-        P->bottom_shift = g_mg_bottom_shift;
-    }
+    TuneResult r;
+    for (int l = 0; l < kMaxLevels; ++l) r.tile[l] = tiles[l];
+    g_tune_cache[key] = r;
     P->have_coef = false;  // the real operator must still be set
     P->tuned = true;
     WEC_CK(cudaStreamSynchronize(st));
@@ -1471,10 +1325,9 @@ int poisson_init(wec_poisson *P, int nx, int ny, int prec, int restart, int nu1,
     if (!attrs_done) {
         // shared-memory tiles of the fused level kernels exceed the 48 KB default (H <= 8)
         if (int e = set_tile_attrs()) return e;
-        WEC_CK(cudaFuncSetAttribute(k_mg_bottom<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBottomSmemMax));
-        WEC_CK(cudaFuncSetAttribute(k_mg_bottom<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBottomSmemMax));
-        WEC_CK(cudaFuncSetAttribute(k3_bottom<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBottom3Smem));
-        WEC_CK(cudaFuncSetAttribute(k3_bottom<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBottom3Smem));
+        if (int e = set_cluster_attrs()) return e;
+        WEC_CK(cudaFuncSetAttribute(k_coarse_inverse<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCoarseSmem));
+        WEC_CK(cudaFuncSetAttribute(k_coarse_inverse<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCoarseSmem));
         if (int e = set_kgrid_max()) return e;
         attrs_done = true;
     }
@@ -1550,13 +1403,25 @@ int poisson_init(wec_poisson *P, int nx, int ny, int prec, int restart, int nu1,
             P->bytes += (nu + nv + nw + 2 * nc) * 4;
         }
     }
-    WEC_CK(cudaMalloc(&P->lu64, (size_t)P->ncoarse * P->ncoarse * 8));
-    if (prec == WEC_PREC_MIXED) WEC_CK(cudaMalloc(&P->lu32, (size_t)P->ncoarse * P->ncoarse * 4));
-    if (P->ncoarse <= kInvMax) {
+    const size_t ninv = (size_t)P->ncoarse * P->ncoarse;
+    for (P->dense = nl - 1; P->dense > 0; --P->dense) {
+        const Level<double> &A = P->L64[P->dense - 1];
+        if ((long long)A.nx * A.ny * A.nz > kDense) break;
+    }
+    if (P->dense < nl - 1) {
+        const Level<double> &A = P->L64[P->dense];
+        const size_t nd = (size_t)A.nx * A.ny * A.nz;
         if (prec == WEC_PREC_FP64)
-            WEC_CK(cudaMalloc(&P->inv64, (size_t)P->ncoarse * P->ncoarse * 8));
+            WEC_CK(cudaMalloc(&P->dense64, nd * nd * 8));
         else
-            WEC_CK(cudaMalloc(&P->inv32, (size_t)P->ncoarse * P->ncoarse * 4));
+            WEC_CK(cudaMalloc(&P->dense32, nd * nd * 4));
+    }
+    if (prec == WEC_PREC_FP64) {
+        WEC_CK(cudaMalloc(&P->inv64, ninv * 8));
+        WEC_CK(cudaMalloc(&P->band, coarse_band_elems(coarse_op(P->L64[nl - 1])) * 8));
+    } else {
+        WEC_CK(cudaMalloc(&P->inv32, ninv * 4));
+        WEC_CK(cudaMalloc(&P->band, coarse_band_elems(coarse_op(P->L32[nl - 1])) * 4));
     }
     size_t n = (size_t)nx * ny * nz;
     int m = restart;
@@ -1598,8 +1463,9 @@ void poisson_free(wec_poisson *P)
         cudaFree(P->L64[l].xp); cudaFree(P->L32[l].xp);
         cudaFree(P->L64[l].id); cudaFree(P->L32[l].id);
     }
-    cudaFree(P->lu64); cudaFree(P->lu32);
+    cudaFree(P->band);
     cudaFree(P->inv64); cudaFree(P->inv32);
+    cudaFree(P->dense64); cudaFree(P->dense32);
     cudaFree(P->V); cudaFree(P->Z); cudaFree(P->w); cudaFree(P->d0); cudaFree(P->part); cudaFree(P->dots); cudaFree(P->hess);
     for (double *&q : P->kdf_face) {
         cudaFree(q);
@@ -1639,8 +1505,8 @@ int build_invdiag3(wec_poisson *P, Level<T> *L, cudaStream_t st)
     Level3Diag<T> D;
     D.nlev = P->nlev;
     D.off[0] = 0;
-    // FP32 levels above the coarsest are colour-packed (mg3d.cuh)
-    D.pk = std::is_same<T, float>::value ? (1u << (P->nlev - 1)) - 1u : 0u;
+    // FP32 levels above the dense one are colour-packed (mg3d.cuh)
+    D.pk = std::is_same<T, float>::value ? (1u << P->dense) - 1u : 0u;
     for (int l = 0; l < P->nlev; ++l) {
         D.nx[l] = L[l].nx;
         D.ny[l] = L[l].ny;
@@ -1658,8 +1524,27 @@ int build_invdiag3(wec_poisson *P, Level<T> *L, cudaStream_t st)
     return WEC_OK;
 }
 
+// the inverse of the coarsest operator
 template <typename T>
-int build_hierarchy3(wec_poisson *P, Level<T> *L, T *lu, cudaStream_t st)
+void build_coarse(wec_poisson *P, const Level<T> *L, cudaStream_t st)
+{
+    const double n = P->ncoarse;
+    WEC_PROF("mg_coarse_inverse", P->nlev - 1, sizeof(T) * n * n, st);
+    launch_coarse_inverse(L[P->nlev - 1], coarse_inv<T>(P), (T *)P->band, st);
+}
+
+// the dense level's matrix
+template <typename T, int D>
+void build_dense(wec_poisson *P, const Level<T> *L, cudaStream_t st)
+{
+    if (P->dense == P->nlev - 1) return;
+    const double n = (double)L[P->dense].nx * L[P->dense].ny * L[P->dense].nz;
+    WEC_PROF("mg_dense", P->dense, sizeof(T) * n * n, st);
+    launch_dense<T, D>(P, L, st);
+}
+
+template <typename T>
+int build_hierarchy3(wec_poisson *P, Level<T> *L, cudaStream_t st)
 {
     for (int l = 0; l + 1 < P->nlev; ++l) {
         Level<T> &F = L[l], &C = L[l + 1];
@@ -1667,11 +1552,10 @@ int build_hierarchy3(wec_poisson *P, Level<T> *L, T *lu, cudaStream_t st)
         WEC_PROF("mg_coarsen", l, 5.0 * sizeof(T) * cnt, st);
         launch_k(k3_coarsen<T>, nblk(cnt, 256), 256, 0, st, F.nx, F.ny, F.nz, F.bu, F.bv, F.bw, C.bu, C.bv, C.bw);
     }
-    Level<T> &Lc = L[P->nlev - 1];
-    const double nn = (double)Lc.nx * Lc.ny * Lc.nz;
-    WEC_PROF("mg_lu_factor", P->nlev - 1, sizeof(T) * nn * nn, st);
-    launch_k(k3_lu_factor<T>, 1, 256, 0, st, Lc.nx, Lc.ny, Lc.nz, Lc.bu, Lc.bv, Lc.bw, lu);
-    return build_invdiag3<T>(P, L, st);
+    build_coarse(P, L, st);
+    if (int e = build_invdiag3<T>(P, L, st)) return e;
+    build_dense<T, 3>(P, L, st);
+    return WEC_OK;
 }
 
 int poisson_build3(wec_poisson *P, cudaStream_t st)
@@ -1706,9 +1590,9 @@ int poisson_build3(wec_poisson *P, cudaStream_t st)
                 launch_k(k_convert<float, double>, nblk(nf[q], 256), 256, 0, st, nf[q], src[q], dst[q], nullptr);
             }
         }
-        e = build_hierarchy3<float>(P, P->L32, P->lu32, st);
+        e = build_hierarchy3<float>(P, P->L32, st);
     } else {
-        e = build_hierarchy3<double>(P, P->L64, P->lu64, st);
+        e = build_hierarchy3<double>(P, P->L64, st);
     }
     if (e) return e;
     WEC_CK(cudaGetLastError());
@@ -1726,7 +1610,7 @@ int poisson_build(wec_poisson *P, cudaStream_t st)
     }
     if (P->prec == WEC_PREC_MIXED) {
         // the V-cycle is FP32 throughout: level 0 converted once, coarse levels
-        // and the coarsest LU formed in FP32 (the FP64 operator is level 0 only)
+        // and the coarsest inverse formed in FP32 (the FP64 operator is level 0 only)
         Level<double> &A = P->L64[0];
         Level<float> &F = P->L32[0];
         const long long nu = (long long)(A.nx + 1) * A.ny, nv = (long long)A.nx * (A.ny + 1);
@@ -1744,11 +1628,9 @@ int poisson_build(wec_poisson *P, cudaStream_t st)
             WEC_PROF("mg_coarsen", l, 12.0 * cnt, st);
             launch_k(k_coarsen<float>, nblk(cnt, 256), 256, 0, st, Fl.nx, Fl.ny, Fl.bu, Fl.bv, C.bu, C.bv);
         }
-        Level<float> &Lf = P->L32[P->nlev - 1];
-        const double nn = (double)Lf.nx * Lf.ny;
-        WEC_PROF("mg_lu_factor", P->nlev - 1, 4.0 * nn * nn, st);
-        launch_k(k_lu_factor<float>, 1, 256, 0, st, Lf.nx, Lf.ny, Lf.bu, Lf.bv, P->lu32, P->inv32);
+        build_coarse(P, P->L32, st);
         if (int e = build_invdiag<float>(P, P->L32, st)) return e;
+        build_dense<float, 2>(P, P->L32, st);
     } else {
         for (int l = 0; l + 1 < P->nlev; ++l) {
             Level<double> &F = P->L64[l], &C = P->L64[l + 1];
@@ -1756,11 +1638,9 @@ int poisson_build(wec_poisson *P, cudaStream_t st)
             WEC_PROF("mg_coarsen", l, 24.0 * cnt, st);
             launch_k(k_coarsen<double>, nblk(cnt, 256), 256, 0, st, F.nx, F.ny, F.bu, F.bv, C.bu, C.bv);
         }
-        Level<double> &Lc = P->L64[P->nlev - 1];
-        const double nn = (double)Lc.nx * Lc.ny;
-        WEC_PROF("mg_lu_factor", P->nlev - 1, 8.0 * nn * nn, st);
-        launch_k(k_lu_factor<double>, 1, 256, 0, st, Lc.nx, Lc.ny, Lc.bu, Lc.bv, P->lu64, P->inv64);
+        build_coarse(P, P->L64, st);
         if (int e = build_invdiag<double>(P, P->L64, st)) return e;
+        build_dense<double, 2>(P, P->L64, st);
     }
     WEC_CK(cudaGetLastError());
     P->have_coef = true;
