@@ -129,8 +129,9 @@ struct wec_poisson {
     double *w = nullptr;        // n
     double *d0 = nullptr;       // n: diagonal of the FP64 level-0 operator
     double *part = nullptr;     // (kMaxRestart+2) x (kKrylovBlocks / 8) cluster partial sums
-    double *dots = nullptr;     // h1, h2 of the two Gram-Schmidt passes
-    double *hess = nullptr;     // (m+1) x m Hessenberg, then cs, sn, g, y
+    double *dots = nullptr;     // h1: the new vector's dot products with the basis
+    double *gram = nullptr;     // Gram matrix of the normalised basis (off-diagonal part)
+    double *hess = nullptr;     // (m+1) x m Hessenberg, then cs, sn, g, sc, y
     double *cs = nullptr, *sn = nullptr, *g = nullptr, *y = nullptr;
     double *sc = nullptr;       // m+1: 1 / ||u_k|| of the unnormalised basis vectors u_k (V's columns)
     // Arnoldi arithmetic in float pairs (3D, WEC_PREC_MIXED_DF): V then holds pairs

@@ -457,21 +457,6 @@ __device__ __forceinline__ void set_cond(unsigned long long h, int use, unsigned
     if (use) cudaGraphSetConditional((cudaGraphConditionalHandle)h, v);
 }
 
-__global__ void k_ks_init(KState *ks, double rtol, int maxit, int m)
-{
-    pdl_entry();
-    ks->rtol = rtol;
-    ks->maxit = maxit;
-    ks->m = m;
-    ks->its = 0;
-    ks->status = 0;
-    ks->done = 0;
-    ks->j = 0;
-    ks->jd = 0;
-    ks->cycle_end = 0;
-    ks->ncycles = 0;
-}
-
 // The level-0 operator seen by the Krylov kernels: D = 2 (bx, by = beta_u,
 // beta_v; nz = 1) or D = 3 (beta_x, beta_y, beta_z); FP64, or float pairs (VT =
 // df64) for the pair-arithmetic Arnoldi step.
@@ -486,7 +471,7 @@ template <int D, typename VT>
 __device__ __forceinline__ VT op_offsum(const OpT<VT> &o, const VT *__restrict__ x, long long c)
 {
     if constexpr (D == 2) {
-        const int j = (int)(c / o.nx), i = (int)(c - (long long)j * o.nx);
+        const int cc = (int)c, j = cc / o.nx, i = cc - j * o.nx;  // (2D grids: nx ny < 2^31)
         return offsum_at(o.bx, o.by, x, o.nx, o.ny, i, j);
     } else {
         const int cc = (int)c, r = cc / o.nx, i = cc - r * o.nx, k = r / o.ny, j = r - k * o.ny;
@@ -505,9 +490,9 @@ __global__ void k_diag0(int nx, int ny, const double *__restrict__ bu, const dou
     d[c] = diag_at(bu, bv, nx, ny, i, j);
 }
 
-// bn = ||b||_2, tol = rtol bn.
+// A new solve's state, bn = ||b||_2 and tol = rtol bn.
 __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(KT, 4)
-    k_bnorm(long long n, const double *__restrict__ b, double *part, KState *ks)
+    k_bnorm(long long n, const double *__restrict__ b, double *part, KState *ks, double rtol, int maxit, int m)
 {
     pdl_entry();
     __shared__ double sh[KT / 32];
@@ -523,7 +508,17 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(KT, 4)
     if (threadIdx.x == 0) {
         double bn = sqrt(t);
         ks->bn = bn;
-        ks->tol = ks->rtol * bn;
+        ks->tol = rtol * bn;
+        ks->rtol = rtol;
+        ks->maxit = maxit;
+        ks->m = m;
+        ks->its = 0;
+        ks->status = 0;
+        ks->done = 0;
+        ks->j = 0;
+        ks->jd = 0;
+        ks->cycle_end = 0;
+        ks->ncycles = 0;
         ks->cnt[0] = 0;
     }
 }
@@ -648,125 +643,178 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(KT, kb_blocks(KB))
     if (threadIdx.x == 0) ks->cnt[2] = 0;
 }
 
-// First Gram-Schmidt update w -= sum_k h1_k v_k = w - sum_k (h1_k s_k) u_k, then
-// h2_k = v_k . w.
+// The CTA's partials of the orthogonalised vector a = w - sum_k hs_k u_k: u_k . a
+// (k < nk) into bsm[k] and a . a into bsm[nk], in the pass that writes a.  V_k[c]
+// is read once where K values fit the registers (K <= 16).
+template <int K, typename VT>
+__device__ __forceinline__ void block_orth_k(VT *V, long long n, int nk, const VT *hs, float *__restrict__ b32,
+                                             double (*sh)[KMAXV], double *bsm)
+{
+    constexpr bool HOLD = K <= 16;
+    constexpr int P2 = K >= 32 ? 5 : K >= 16 ? 4 : K >= 8 ? 3 : K >= 4 ? 2 : K >= 2 ? 1 : 0;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    VT *const w = V + (long long)nk * n;
+    VT av[K], an = VT(0.0);
+#pragma unroll
+    for (int q = 0; q < K; ++q) av[q] = VT(0.0);
+    for (long long c = blockIdx.x * (long long)KT + threadIdx.x; c < n; c += (long long)gridDim.x * KT) {
+        VT v[HOLD ? K : 1];
+        VT a = w[c];
+        if constexpr (HOLD) {
+#pragma unroll
+            for (int q = 0; q < K; ++q) v[q] = q < nk ? V[(long long)q * n + c] : VT(0.0);
+#pragma unroll
+            for (int q = 0; q < K; ++q)
+                if (q < nk) a -= hs[q] * v[q];
+        } else {
+            for (int q = 0; q < nk; ++q) a -= hs[q] * V[(long long)q * n + c];
+        }
+        w[c] = a;
+        if (b32) b32[c] = vt_float(a);
+#pragma unroll
+        for (int q = 0; q < K; ++q)
+            if (q < nk) av[q] += (HOLD ? v[HOLD ? q : 0] : V[(long long)q * n + c]) * a;
+        an += a * a;
+    }
+    double a[K];
+#pragma unroll
+    for (int q = 0; q < K; ++q) a[q] = vt_double(av[q]);
+    warp_reduce_scatter<K>(a, lane);
+    if ((lane & ((32 >> P2) - 1)) == 0) {
+        const int k = lane >> (5 - P2);
+        if (k < nk) sh[warp][k] = a[0];
+    }
+    const double s = warp_sum(vt_double(an));
+    if (lane == 0) sh[warp][nk] = s;
+    __syncthreads();
+    if (threadIdx.x <= nk) {
+        double r = 0.0;
+        for (int q = 0; q < KT / 32; ++q) r += sh[q][threadIdx.x];
+        bsm[threadIdx.x] = r;
+    }
+}
+
+// Classical Gram-Schmidt, twice, in one pass over the basis.  With h1_k = v_k . w
+// the second pass's coefficients v_k . (w - sum_l h1_l v_l) are h1_k - sum_l G_kl
+// h1_l, G_kl = v_k . v_l the basis's Gram matrix: every earlier call measured its
+// new column (the dot products below, of the vector as it was stored), so the
+// second pass's dot products need no pass of their own.  w -= sum_k (h1_k + h2_k)
+// v_k leaves u_{j+1} in column j+1 (and its FP32 copy b32 for the next mixed
+// V-cycle), h_{j+1,j} = ||w||, s_{j+1} = 1 / h_{j+1,j}, and column j+1 of G.  The
+// last cluster applies the Givens rotations to column j, counts the iteration,
+// decides whether the cycle ends (converged estimate, iteration cap, breakdown, or
+// full basis), advances j otherwise, and sets the IF condition.
+// Bound by the FP64 pipe (FP64) or HBM (float pairs over HBM-sized vectors).  Two
+// kernels, one per pass, read the basis twice: 531 us together at 512x256x256 in
+// float pairs where this one takes 318.
 template <int KB, typename VT = double>
-__global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(KT, KB <= 4 ? 4 : KB <= 8 ? 3 : 2)
-    k_orth_dots(long long n, VT *V, const double *__restrict__ sc, const double *__restrict__ h1, double *part,
-                double *h2, KState *ks)
+__global__ void __cluster_dims__(kCl, 1, 1)
+    __launch_bounds__(KT, KB <= 4 ? (std::is_same<VT, double>::value ? 4 : 5) : KB <= 8 ? 3 : 2)
+    k_orth(long long n, VT *V, double *sc, float *__restrict__ b32, const double *__restrict__ h1, double *G, double *part,
+           KState *ks, double *H, double *cs, double *sn, double *g, unsigned long long hif, int use)
 {
     pdl_entry();
     __shared__ double sh[KT / 32][KMAXV];
     __shared__ double bsm[KMAXV];
     __shared__ VT hs[KMAXV];
-    const int j = ks->j, nk = j + 1;
-    VT *w = V + (long long)(j + 1) * n;
-    if (threadIdx.x < nk) hs[threadIdx.x] = VT(h1[threadIdx.x] * sc[threadIdx.x]);
-    __syncthreads();
-    // the update and the second dots in one pass over the basis (V_k[c] read once)
-    block_dots<KB>(
-        V, n, 0, nk,
-        [&](long long c, const auto &v, int, int) {
-            constexpr int KH = std::extent<std::remove_reference_t<decltype(v)>>::value;
-            VT a = w[c];
-            if (nk <= KH) {
-#pragma unroll
-                for (int k = 0; k < KH; ++k)
-                    if (k < nk) a -= hs[k] * v[k];
-            } else {
-                for (int k = 0; k < nk; ++k) a -= hs[k] * V[(long long)k * n + c];
-            }
-            w[c] = a;
-            return a;
-        },
-        sh, bsm);
-    cluster_partials(bsm, nk, part);
-    if (!last_cluster(&ks->cnt[2])) return;
-    final_partials(part, nk, gridDim.x / kCl, h2);
-    __syncthreads();
-    if (threadIdx.x < nk) h2[threadIdx.x] *= sc[threadIdx.x];
-    if (threadIdx.x == 0) ks->cnt[2] = 0;
-}
-
-// Second update w -= sum_k (h2_k s_k) u_k, which leaves u_{j+1} = w in column j+1
-// (and its FP32 copy b32 for the next mixed V-cycle), h_{j+1,j} = ||w||, s_{j+1} =
-// 1 / h_{j+1,j}; the last cluster applies the Givens rotations to column j,
-// counts the iteration, decides whether the cycle ends (converged estimate,
-// iteration cap, breakdown, or full basis), advances j otherwise, and sets the
-// IF condition.
-template <typename VT = double>
-__global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(KT, std::is_same<VT, double>::value ? 4 : 6)
-    k_orth_norm(long long n, VT *V, double *sc, float *__restrict__ b32, const double *__restrict__ h1,
-                const double *__restrict__ h2, double *part, KState *ks, double *H, double *cs, double *sn,
-                double *g, unsigned long long hif, int use)
-{
-    pdl_entry();
-    __shared__ double sh[KT / 32];
-    __shared__ double bsm[1];
-    __shared__ VT hs[KMAXV];
-    const int j = ks->j;
-    VT *w = V + (long long)(j + 1) * n;
-    if (threadIdx.x <= j) hs[threadIdx.x] = VT(h2[threadIdx.x] * sc[threadIdx.x]);
-    __syncthreads();
-    VT av2 = VT(0.0);
-    for (long long c = blockIdx.x * (long long)KT + threadIdx.x; c < n; c += (long long)gridDim.x * KT) {
-        VT a = w[c];
-#pragma unroll 4
-        for (int k = 0; k <= j; ++k) a -= hs[k] * V[(long long)k * n + c];
-        w[c] = a;
-        if (b32) b32[c] = vt_float(a);
-        av2 += a * a;
+    __shared__ double hh[KMAXV];  // h1 + h2, then the rotated column
+    const int j = ks->j, nk = j + 1, lane = threadIdx.x & 31;
+    // a warp per row of G
+    for (int k = threadIdx.x >> 5; k < nk; k += KT / 32) {
+        double d = lane < nk && lane != k ? G[k * KMAXV + lane] * h1[lane] : 0.0;
+        for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+        if (lane == 0) {
+            const double h = h1[k] - d;
+            hh[k] = h;
+            hs[k] = VT(h * sc[k]);
+        }
     }
-    double a2 = block_sum(vt_double(av2), sh);
-    if (threadIdx.x == 0) bsm[0] = a2;
-    cluster_partials(bsm, 1, part);
+    __syncthreads();
+    if (nk <= 1) {
+        block_orth_k<1>(V, n, nk, hs, b32, sh, bsm);
+    } else if (nk <= 2) {
+        block_orth_k<2>(V, n, nk, hs, b32, sh, bsm);
+    } else if (nk <= 4 || KB <= 4) {  // (KB <= 4: nk <= 4)
+        block_orth_k<4>(V, n, nk, hs, b32, sh, bsm);
+    } else if constexpr (KB <= 8) {
+        block_orth_k<8>(V, n, nk, hs, b32, sh, bsm);
+    } else {
+        if (nk <= 8)
+            block_orth_k<8>(V, n, nk, hs, b32, sh, bsm);
+        else if (nk <= 16)
+            block_orth_k<16>(V, n, nk, hs, b32, sh, bsm);
+        else
+            block_orth_k<32>(V, n, nk, hs, b32, sh, bsm);
+    }
+    cluster_partials(bsm, nk + 1, part);
     if (!last_cluster(&ks->cnt[2])) return;
-    double t = final_sum(part, gridDim.x / kCl, sh);
-    if (threadIdx.x != 0) return;
     const int m = ks->m;
-    for (int k = 0; k <= j; ++k) H[k * m + j] = (0.0 + h1[k]) + h2[k];
-    double hn = sqrt(t);
-    H[(j + 1) * m + j] = hn;
-    for (int k = 0; k < j; ++k) {
-        double p = H[k * m + j], q = H[(k + 1) * m + j];
-        H[k * m + j] = cs[k] * p + sn[k] * q;
-        H[(k + 1) * m + j] = -sn[k] * p + cs[k] * q;
+    // the rotations so far beside the sums (one round trip to L2 for both)
+    double *const c0 = sh[0], *const s0 = sh[1];
+    if (threadIdx.x < j) {
+        c0[threadIdx.x] = cs[threadIdx.x];
+        s0[threadIdx.x] = sn[threadIdx.x];
     }
-    double p = H[j * m + j], q = H[(j + 1) * m + j];
-    double den = sqrt(p * p + q * q);
-    cs[j] = p / den;
-    sn[j] = q / den;
-    H[j * m + j] = den;
-    H[(j + 1) * m + j] = 0.0;
-    g[j + 1] = -sn[j] * g[j];
-    g[j] = cs[j] * g[j];
-    ks->its += 1;
-    ks->jd = j + 1;
-    ks->hn = hn;
-    ks->ihn = hn != 0.0 ? 1.0 / hn : 0.0;
-    sc[j + 1] = ks->ihn;
-    double est = fabs(g[j + 1]);
-    int ce = est <= ks->tol || ks->its >= ks->maxit || hn == 0.0 || j + 1 == m || !isfinite(est);
-    if (!isfinite(est)) ks->status = WEC_ERR_NONFINITE;
-    ks->cycle_end = ce;
-    if (!ce) ks->j = j + 1;  // every CTA read j at its start
-    ks->cnt[2] = 0;
-    set_cond(hif, use, (unsigned)ce);
+    final_partials(part, nk + 1, gridDim.x / kCl, bsm);
+    __syncthreads();
+    const double hn = sqrt(bsm[nk]), ihn = hn != 0.0 ? 1.0 / hn : 0.0;
+    if (threadIdx.x < nk) {
+        const double gk = bsm[threadIdx.x] * sc[threadIdx.x] * ihn;
+        G[threadIdx.x * KMAXV + nk] = gk;
+        G[nk * KMAXV + threadIdx.x] = gk;
+    }
+    if (threadIdx.x == 0) {
+        for (int k = 0; k < j; ++k) {
+            const double p = hh[k], q = hh[k + 1];
+            hh[k] = c0[k] * p + s0[k] * q;
+            hh[k + 1] = -s0[k] * p + c0[k] * q;
+        }
+        const double p = hh[j], q = hn;
+        const double den = sqrt(p * p + q * q);
+        const double cj = p / den, sj = q / den, gj = g[j];
+        hh[j] = den;
+        cs[j] = cj;
+        sn[j] = sj;
+        g[j + 1] = -sj * gj;
+        g[j] = cj * gj;
+        const int its = ks->its + 1;
+        ks->its = its;
+        ks->jd = j + 1;
+        ks->hn = hn;
+        ks->ihn = ihn;
+        sc[j + 1] = ihn;
+        const double est = fabs(sj * gj);
+        const int ce = est <= ks->tol || its >= ks->maxit || hn == 0.0 || j + 1 == m || !isfinite(est);
+        if (!isfinite(est)) ks->status = WEC_ERR_NONFINITE;
+        ks->cycle_end = ce;
+        if (!ce) ks->j = j + 1;  // every CTA read j at its start
+        ks->cnt[2] = 0;
+        set_cond(hif, use, (unsigned)ce);
+    }
+    __syncthreads();
+    if (threadIdx.x <= j) H[threadIdx.x * m + j] = hh[threadIdx.x];
 }
 
-// y from the triangular system, then y_k s_k: the preconditioned vectors are
-// stored for the unnormalised basis (z'_k = z_k / s_k), so x += sum_k (y_k s_k) z'_k.
-__global__ void k_backsolve(int m, const double *__restrict__ H, const double *__restrict__ g, double *__restrict__ y,
-                            const double *__restrict__ sc, const KState *ks)
+// y from the triangular system H y = g (one warp, a row per lane, column by column
+// in shared memory), then y_k s_k: the preconditioned vectors are stored for the
+// unnormalised basis (z'_k = z_k / s_k), so x += sum_k (y_k s_k) z'_k.
+__global__ void __launch_bounds__(256)
+    k_backsolve(int m, const double *__restrict__ H, const double *__restrict__ g, double *__restrict__ y,
+                const double *__restrict__ sc, const KState *ks)
 {
     pdl_entry();
-    const int jd = ks->jd;
-    for (int k = jd - 1; k >= 0; --k) {
-        double s = g[k];
-        for (int l = k + 1; l < jd; ++l) s -= H[k * m + l] * y[l];
-        y[k] = s / H[k * m + k];
+    __shared__ double Hs[kMaxRestart * kMaxRestart];
+    const int jd = ks->jd, k = threadIdx.x;
+    for (int q = threadIdx.x; q < jd * jd; q += blockDim.x) Hs[q] = H[(q / jd) * m + q % jd];
+    __syncthreads();
+    if (k >= 32) return;
+    double v = k < jd ? g[k] : 0.0;
+    for (int l = jd - 1; l >= 0; --l) {
+        if (k == l) v /= Hs[l * jd + l];
+        const double yl = __shfl_sync(0xffffffffu, v, l);
+        if (k < l) v -= Hs[k * jd + l] * yl;
     }
-    for (int k = 0; k < jd; ++k) y[k] *= sc[k];
+    if (k < jd) y[k] = v * sc[k];
 }
 
 template <typename VT = double>
@@ -1091,12 +1139,12 @@ void vcycle_t(wec_poisson *P, Level<T> *L, const T *b0, TO *x0, const int *bsel,
 // scheduler places whole clusters inside a GPC, so the count comes from the
 // occupancy query, not from SMs x CTAs per SM.  Set once by poisson_init.
 // the largest grid (CTAs) of each Krylov reduction kernel: its resident
-// clusters, at most kKrylovBlocks; res[d3], mv[d3][restart <= 8], od[restart <= 8]
+// clusters, at most kKrylovBlocks; res[d3], mv[d3][restart <= 8], on[restart <= 8]
 struct KGrids {
-    int bnorm = kCl, on = kCl, res[2] = {kCl, kCl}, mv[2][2] = {{kCl, kCl}, {kCl, kCl}}, od[2] = {kCl, kCl};
-    // the float-pair Arnoldi kernels (3D): residual, matvec[restart <= 8], orth dots[restart <= 8], orth norm
-    int res_df = kCl, mv_df[2] = {kCl, kCl}, od_df[2] = {kCl, kCl}, on_df = kCl;
-    int mv_df4 = kCl, od_df4 = kCl;  // their variants for at most 4 basis vectors (more CTAs per SM)
+    int bnorm = kCl, res[2] = {kCl, kCl}, mv[2][2] = {{kCl, kCl}, {kCl, kCl}}, on[2] = {kCl, kCl};
+    // the float-pair Arnoldi kernels (3D): residual, matvec[restart <= 8], orthogonalisation[restart <= 8]
+    int res_df = kCl, mv_df[2] = {kCl, kCl}, on_df[2] = {kCl, kCl};
+    int mv_df4 = kCl, on_df4 = kCl;  // their variants for at most 4 basis vectors (more CTAs per SM)
 };
 KGrids g_kg;
 
@@ -1128,33 +1176,31 @@ int set_kgrid_max()
     };
     KGrids &k = g_kg;
     int e = r(k_bnorm, k.bnorm);
-    if (!e) e = r(k_orth_norm<double>, k.on);
     if (!e) e = r(k_residual_norm<2>, k.res[0]);
     if (!e) e = r(k_residual_norm<3>, k.res[1]);
     if (!e) e = r(k_matvec_dots<2, 32>, k.mv[0][0]);
     if (!e) e = r(k_matvec_dots<2, 8>, k.mv[0][1]);
     if (!e) e = r(k_matvec_dots<3, 32>, k.mv[1][0]);
     if (!e) e = r(k_matvec_dots<3, 8>, k.mv[1][1]);
-    if (!e) e = r(k_orth_dots<32>, k.od[0]);
-    if (!e) e = r(k_orth_dots<8>, k.od[1]);
+    if (!e) e = r(k_orth<32>, k.on[0]);
+    if (!e) e = r(k_orth<8>, k.on[1]);
     if (!e) e = r(k_residual_norm<3, df64>, k.res_df);
     if (!e) e = r(k_matvec_dots<3, 32, df64, float>, k.mv_df[0]);
     if (!e) e = r(k_matvec_dots<3, 8, df64, float>, k.mv_df[1]);
     if (!e) e = r(k_matvec_dots<3, 4, df64, float>, k.mv_df4, kKrylovBlocks);
-    if (!e) e = r(k_orth_dots<4, df64>, k.od_df4, kKrylovBlocks);
-    if (!e) e = r(k_orth_dots<32, df64>, k.od_df[0]);
-    if (!e) e = r(k_orth_dots<8, df64>, k.od_df[1]);
-    if (!e) e = r(k_orth_norm<df64>, k.on_df, kKrylovBlocks);
+    if (!e) e = r(k_orth<4, df64>, k.on_df4, kKrylovBlocks);
+    if (!e) e = r(k_orth<32, df64>, k.on_df[0]);
+    if (!e) e = r(k_orth<8, df64>, k.on_df[1]);
     return e;
 }
 
 // Reduction kernels: a multiple of the cluster size, at most one wave of the
-// kernel's resident clusters (gmax).  Vectors that stay in L2 (up to 2^22
-// cells) take at most 2 CTAs per SM: those passes are latency-bound and half
-// the partials shorten the final reduction.
+// kernel's resident clusters (gmax).  Vectors of up to 2^20 cells take at most 2
+// CTAs per SM: those passes are latency-bound and half the partials shorten the
+// final reduction.
 int kgrid(long long n, int gmax)
 {
-    if (n <= (1ll << 22)) gmax = std::min(gmax, 2 * 152);
+    if (n <= (1ll << 20)) gmax = std::min(gmax, 2 * 152);
     const long long g = std::min<long long>(nblk(n, KT), gmax);
     return (int)((g + kCl - 1) / kCl * kCl);
 }
@@ -1205,12 +1251,8 @@ void enqueue_begin(wec_poisson *P, const double *b, double *x, double rtol, int 
     const double nf = nfaces(P);
     float *b32 = P->prec == WEC_PREC_MIXED ? P->L32[0].b : nullptr;
     {
-        WEC_PROF("scalar", -1, 64.0, st);
-        launch_k(k_ks_init, 1, 1, 0, st, P->ks, rtol, maxit, P->restart);
-    }
-    {
         WEC_PROF("krylov_norm", -1, 8.0 * n, st);
-        launch_k(k_bnorm, kgrid(n, g_kg.bnorm), KT, 0, st, n, b, P->part, P->ks);
+        launch_k(k_bnorm, kgrid(n, g_kg.bnorm), KT, 0, st, n, b, P->part, P->ks, rtol, maxit, P->restart);
     }
     WEC_PROF("krylov_residual", -1, 8.0 * (4.0 * n + nf) + (b32 ? 4.0 * n : 0.0), st);
     launch_residual_norm(P, b, x, b32, 0, hw, use, st);
@@ -1228,8 +1270,8 @@ void enqueue_body(wec_poisson *P, unsigned long long hif, int use, cudaStream_t 
     const double nf = nfaces(P);
     const int m = P->restart, d3 = P->nz > 1 ? 1 : 0, kb8 = m <= 8 ? 1 : 0;
     const bool mixed = P->prec == WEC_PREC_MIXED;
-    double *h1 = P->dots, *h2 = P->dots + (kMaxRestart + 2);
-    // the mixed V-cycle reads u_j in FP32, written beside it by k_residual_norm / k_orth_norm
+    double *h1 = P->dots;
+    // the mixed V-cycle reads u_j in FP32, written beside it by k_residual_norm / k_orth
     if (P->kdf) {  // (3D, FP32 V-cycles) the float-pair Arnoldi step
         vcycle3_t<float, float>(P, P->L32, P->L32[0].b, (float *)P->Z, nullptr, &P->ks->j, st);
         const bool k4 = jh >= 0 && jh + 1 <= 4;
@@ -1241,15 +1283,10 @@ void enqueue_body(wec_poisson *P, unsigned long long hif, int use, cudaStream_t 
             launch_k(kern, kgrid(n, k4 ? g_kg.mv_df4 : g_kg.mv_df[kb8]), KT, 0, st, op0df(P),
                      (const df64 *)P->kdf_d0, (const float *)P->Z, (df64 *)P->V, P->sc, P->part, h1, P->ks);
         }
-        {
-            WEC_PROF("krylov_orth_dots", -1, 8.0 * n * (m + 2), st);
-            auto kern = k4 ? k_orth_dots<4, df64> : kb8 ? k_orth_dots<8, df64> : k_orth_dots<32, df64>;
-            launch_k(kern, kgrid(n, k4 ? g_kg.od_df4 : g_kg.od_df[kb8]), KT, 0, st, n, (df64 *)P->V, P->sc, h1,
-                     P->part, h2, P->ks);
-        }
-        WEC_PROF("krylov_orth_norm", -1, 8.0 * n * (m + 2) + 4.0 * n, st);
-        launch_k(k_orth_norm<df64>, kgrid(n, g_kg.on_df), KT, 0, st, n, (df64 *)P->V, P->sc, P->L32[0].b, h1, h2,
-                 P->part, P->ks, P->hess, P->cs, P->sn, P->g, hif, use);
+        WEC_PROF("krylov_orth", -1, 8.0 * n * (m + 2) + 4.0 * n, st);
+        auto kern = k4 ? k_orth<4, df64> : kb8 ? k_orth<8, df64> : k_orth<32, df64>;
+        launch_k(kern, kgrid(n, k4 ? g_kg.on_df4 : g_kg.on_df[kb8]), KT, 0, st, n, (df64 *)P->V, P->sc, P->L32[0].b, h1,
+                 P->gram, P->part, P->ks, P->hess, P->cs, P->sn, P->g, hif, use);
         return;
     }
     if (!mixed)
@@ -1262,14 +1299,9 @@ void enqueue_body(wec_poisson *P, unsigned long long hif, int use, cudaStream_t 
                        : (kb8 ? k_matvec_dots<2, 8> : k_matvec_dots<2, 32>);
         launch_k(kern, kgrid(n, g_kg.mv[d3][kb8]), KT, 0, st, op0(P), P->d0, P->Z, P->V, P->sc, P->part, h1, P->ks);
     }
-    {
-        WEC_PROF("krylov_orth_dots", -1, 8.0 * n * (m + 2), st);
-        launch_k(kb8 ? k_orth_dots<8> : k_orth_dots<32>, kgrid(n, g_kg.od[kb8]), KT, 0, st, n, P->V, P->sc, h1,
-                 P->part, h2, P->ks);
-    }
-    WEC_PROF("krylov_orth_norm", -1, 8.0 * n * (m + 2) + (mixed ? 4.0 * n : 0.0), st);
-    launch_k(k_orth_norm<double>, kgrid(n, g_kg.on), KT, 0, st, n, P->V, P->sc, mixed ? P->L32[0].b : nullptr, h1, h2, P->part, P->ks,
-             P->hess, P->cs, P->sn, P->g, hif, use);
+    WEC_PROF("krylov_orth", -1, 8.0 * n * (m + 2) + (mixed ? 4.0 * n : 0.0), st);
+    launch_k(kb8 ? k_orth<8> : k_orth<32>, kgrid(n, g_kg.on[kb8]), KT, 0, st, n, P->V, P->sc,
+             mixed ? P->L32[0].b : nullptr, h1, P->gram, P->part, P->ks, P->hess, P->cs, P->sn, P->g, hif, use);
 }
 
 // End of a cycle: y from the triangular system, x += Z y, true residual, then
@@ -1282,7 +1314,7 @@ void enqueue_close(wec_poisson *P, const double *b, double *x, unsigned long lon
     const bool mixed = P->prec == WEC_PREC_MIXED;
     {
         WEC_PROF("scalar", -1, 8.0 * m * m, st);
-        launch_k(k_backsolve, 1, 1, 0, st, m, P->hess, P->g, P->y, P->sc, P->ks);
+        launch_k(k_backsolve, 1, 256, 0, st, m, P->hess, P->g, P->y, P->sc, P->ks);
     }
     {
         WEC_PROF("krylov_update_x", -1, 16.0 * n + (P->kdf ? 4.0 : 8.0) * n * m, st);
@@ -1437,15 +1469,17 @@ int poisson_init(wec_poisson *P, int nx, int ny, int prec, int restart, int nu1,
     }
     // reduction partials: one per cluster and quantity
     WEC_CK(cudaMalloc(&P->part, (size_t)(kMaxRestart + 2) * (kKrylovBlocks / kCl) * 8));
-    WEC_CK(cudaMalloc(&P->dots, 2 * (kMaxRestart + 2) * 8));
-    size_t nh = (size_t)(m + 1) * m + 3 * (m + 1) + m + 8 + (m + 1);
+    WEC_CK(cudaMalloc(&P->dots, (kMaxRestart + 2) * 8));
+    WEC_CK(cudaMalloc(&P->gram, KMAXV * KMAXV * 8));
+    WEC_CK(cudaMemset(P->gram, 0, KMAXV * KMAXV * 8));
+    size_t nh = (size_t)(m + 1) * m + 5 * (m + 1);
     WEC_CK(cudaMalloc(&P->hess, nh * 8));
     WEC_CK(cudaMemset(P->hess, 0, nh * 8));
     P->cs = P->hess + (m + 1) * m;
     P->sn = P->cs + (m + 1);
     P->g = P->sn + (m + 1);
-    P->y = P->g + (m + 1);
-    P->sc = P->y + m + 8;
+    P->sc = P->g + (m + 1);
+    P->y = P->sc + (m + 1);
     WEC_CK(cudaMalloc(&P->ks, sizeof(KState)));
     WEC_CK(cudaMemset(P->ks, 0, sizeof(KState)));
     WEC_CK(cudaMallocHost(&P->ksh, sizeof(KState)));
@@ -1466,7 +1500,7 @@ void poisson_free(wec_poisson *P)
     cudaFree(P->band);
     cudaFree(P->inv64); cudaFree(P->inv32);
     cudaFree(P->dense64); cudaFree(P->dense32);
-    cudaFree(P->V); cudaFree(P->Z); cudaFree(P->w); cudaFree(P->d0); cudaFree(P->part); cudaFree(P->dots); cudaFree(P->hess);
+    cudaFree(P->V); cudaFree(P->Z); cudaFree(P->w); cudaFree(P->d0); cudaFree(P->part); cudaFree(P->dots); cudaFree(P->gram); cudaFree(P->hess);
     for (double *&q : P->kdf_face) {
         cudaFree(q);
         q = nullptr;
