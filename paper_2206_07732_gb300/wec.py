@@ -305,7 +305,7 @@ class Tank:
 
     def get(self, f):
         f = FIELD_NAMES.get(f, f)
-        a = np.zeros(self.shape(f))
+        a = np.empty(self.shape(f))  # (every value is written)
         _check(load().wec_get_field(self.h, f, _ptr(a), a.size))
         return a
 
@@ -689,7 +689,9 @@ class Tank3:
     __del__ = close
 
     def get(self, fid):
-        a = np.zeros(self.shapes[fid])
+        # not zeroed first: the copy fills every value, and into the untouched pages
+        # that zeros() hands out it runs at 1 to 2 GB/s (16 MB: 14 ms, empty 0.7 ms)
+        a = np.empty(self.shapes[fid])
         _check(load().wec_tank3_get_field(self.h, fid, _ptr(a), a.size))
         return a
 
