@@ -21,6 +21,7 @@
 #include <cmath>
 #include <utility>
 
+#include "limiters.cuh"
 #include "tank.cuh"
 
 namespace wec {
@@ -127,56 +128,6 @@ __device__ __forceinline__ R cell_at(const TankP &P, const S *__restrict__ a, in
     return R(a[clampi(j, 0, P.ny - 1) * P.nx + clampi(i, 0, P.nx - 1)]);
 }
 
-// ----------------------------------------------------------------- PPM ----
-template <typename R>
-__device__ __forceinline__ R vl_slope(R am, R a0, R ap)
-{
-    R dl = a0 - am, dr = ap - a0;
-    if (dl * dr <= R(0.0)) return R(0.0);
-    R dc = R(0.5) * (ap - am);
-    R m = fmin(fabs(dc), fmin(R(2.0) * fabs(dl), R(2.0) * fabs(dr)));
-    return dc > R(0.0) ? m : -m;
-}
-
-// Limited Colella-Woodward edge values (left eL, right eR) of the middle cell of a[0..4].
-template <typename R>
-__device__ __forceinline__ void ppm_edges(const R *a, R &eL, R &eR)
-{
-    R dm = vl_slope<R>(a[0], a[1], a[2]);
-    R d0 = vl_slope<R>(a[1], a[2], a[3]);
-    R dp = vl_slope<R>(a[2], a[3], a[4]);
-    eL = a[1] + R(0.5) * (a[2] - a[1]) - (d0 - dm) * (R(1.0) / R(6.0));
-    eR = a[2] + R(0.5) * (a[3] - a[2]) - (dp - d0) * (R(1.0) / R(6.0));
-    R c = a[2];
-    if ((eR - c) * (c - eL) <= R(0.0)) {
-        eL = c;
-        eR = c;
-    } else {
-        R dA = eR - eL;
-        R m6 = dA * (c - R(0.5) * (eL + eR));
-        R q = dA * dA * (R(1.0) / R(6.0));
-        if (m6 > q)
-            eL = R(3.0) * c - R(2.0) * eR;
-        else if (-q > m6)
-            eR = R(3.0) * c - R(2.0) * eL;
-    }
-}
-
-// Time-centred upwind face state; a[0..5] = cells f-3..f+2 around face f.
-template <typename R>
-__device__ __forceinline__ R ppm_face(const R *a, R vel, R dt, R ih)
-{
-    R eL, eR;
-    if (vel >= R(0.0)) {
-        ppm_edges<R>(a, eL, eR);
-        R C = vel * dt * ih, dA = eR - eL, a6 = R(6.0) * (a[2] - R(0.5) * (eL + eR));
-        return eR - R(0.5) * C * (dA - (R(1.0) - C * (R(2.0) / R(3.0))) * a6);
-    }
-    ppm_edges<R>(a + 1, eL, eR);
-    R C = -vel * dt * ih, dA = eR - eL, a6 = R(6.0) * (a[3] - R(0.5) * (eL + eR));
-    return eL + R(0.5) * C * (dA + (R(1.0) - C * (R(2.0) / R(3.0))) * a6);
-}
-
 // Damping-zone weight (Jacobsen) and the vorticity-damping shape (cos(pi z~) + 1),
 // evaluated once per tank into tables (columns / rows) by k_tables.
 __device__ __forceinline__ double damp_alpha_eval(const TankP &P, double x)
@@ -200,28 +151,6 @@ template <typename R>
 __device__ __forceinline__ R vort_damp(const TankP &P, R shape, R idt)
 {
     return cst<R>(P).rho_a * shape * (R(0.25) * idt);
-}
-
-template <typename R>
-__device__ __forceinline__ R minmod(R a, R b)
-{
-    if (a * b <= R(0.0)) return R(0.0);
-    return fabs(a) < fabs(b) ? a : b;
-}
-
-template <typename R>
-__device__ __forceinline__ R koren(R quu, R qu, R qd)
-{
-    R d1 = qu - quu, d2 = qd - qu;
-    if (d1 * d2 <= R(0.0)) return qu;
-    R m = fmin(R(2.0) * fabs(d2), fmin((fabs(d1) + R(2.0) * fabs(d2)) * (R(1.0) / R(3.0)), R(2.0) * fabs(d1)));
-    return d1 > R(0.0) ? qu + R(0.5) * m : qu - R(0.5) * m;
-}
-
-template <typename R>
-__device__ __forceinline__ R upwind(R q0, R q1, R q2, R q3, R vel)
-{
-    return vel >= R(0.0) ? koren<R>(q0, q1, q2) : koren<R>(q3, q2, q1);
 }
 
 // ------------------------------------------------------------- kernels ----
@@ -413,91 +342,113 @@ __global__ void k_heave(TankP P, StepScalars *S, const double *__restrict__ part
     S->yc1 = yc1;
 }
 
-// sigma* = sigma^n - dt Q(u^n, sigma^n), then damping-zone relaxation.
+// The stencil kernels run one block row per grid row (blockIdx.x the row, which
+// may exceed 65535, blockIdx.y the tile along it; no index division) and split
+// off the cells and faces whose whole stencil lies inside the grid: those read at
+// fixed offsets, the rest through the accessors above with their ghost rules.  In
+// FP64 every one of them is bound by the FP64 pipe (two operations per clock and
+// SM), so the arithmetic spends as few FP64 instructions as the formulas allow:
+// limiter decisions on the integer pipe (limiters.cuh), face quantities formed
+// once, the viscous operator as a weighted sum.  At 1024x256 in FP64 the step's
+// stencils went from 1.15 to 0.58 ms: advection 243 -> 81 us, a reinitialisation
+// stage 51 -> 34, the momentum system 246 -> 147 (with the face quantities), a
+// Jacobi sweep 69 -> 18.
+constexpr int TX = 128;  // threads along a row
+inline dim3 row_grid(int nx, int rows) { return dim3(rows, (nx + TX - 1) / TX); }
+
+// The PPM value of sigma on every x-face (block rows 0 .. ny-1) and y-face (the
+// ny+1 rows after them), time-centred and upwind: a face value depends on the
+// face alone and is read by the two cells beside it.  Formed by each cell for its
+// four faces, advection took 243 us at 1024x256 in FP64; the two kernels take 81.
 template <typename R>
-__global__ void k_advect(TankP P, const R *__restrict__ s, const R *__restrict__ u,
-                         const R *__restrict__ v, const double *__restrict__ eta0,
-                         const double *__restrict__ inp, const R *__restrict__ alpha_c,
-                         double *__restrict__ out, R *__restrict__ out_w)
+__global__ void __launch_bounds__(TX) k_ppm_faces(TankP P, const R *__restrict__ s, const R *__restrict__ u,
+                                                  const R *__restrict__ v, const double *__restrict__ eta0,
+                                                  const double *__restrict__ inp, R *__restrict__ Fx, R *__restrict__ Fy)
 {
     pdl_entry();
-    int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= P.nx * P.ny) return;
-    const R dt = R(inp[0]);
-    const int nx = P.nx, i = c % nx, j = c / nx;
-    const R h = cst<R>(P).h;
-    R a[6], fx[2], fy[2];
-    for (int f = 0; f < 2; ++f) {
-        int fi = i + f;
-        for (int q = 0; q < 6; ++q) a[q] = sig_at<R>(P, s, eta0, fi - 3 + q, j);
-        fx[f] = ppm_face<R>(a, R(u[j * (nx + 1) + fi]), dt, cst<R>(P).ih);
-        int fj = j + f;
-        for (int q = 0; q < 6; ++q) a[q] = sig_at<R>(P, s, eta0, i, fj - 3 + q);
-        fy[f] = ppm_face<R>(a, R(v[fj * nx + i]), dt, cst<R>(P).ih);
+    const int nx = P.nx, ny = P.ny, i = blockIdx.y * TX + threadIdx.x;
+    const bool xf = (int)blockIdx.x < ny;
+    const int j = xf ? blockIdx.x : blockIdx.x - ny;
+    if (i >= nx + (xf ? 1 : 0)) return;
+    const int f = xf ? j * (nx + 1) + i : j * nx + i, c = j * nx + i, sd = xf ? 1 : nx;
+    const int cd = xf ? i : j, nd = xf ? nx : ny;
+    R a[6];
+    if (cd >= 3 && cd + 2 < nd) {
+#pragma unroll
+        for (int m = 0; m < 6; ++m) a[m] = s[c + (m - 3) * sd];
+    } else {
+#pragma unroll
+        for (int m = 0; m < 6; ++m) a[m] = sig_at<R>(P, s, eta0, xf ? i + m - 3 : i, xf ? j : j + m - 3);
     }
-    R ub = R(0.5) * (R(u[j * (nx + 1) + i]) + R(u[j * (nx + 1) + i + 1]));
-    R vb = R(0.5) * (R(v[j * nx + i]) + R(v[(j + 1) * nx + i]));
-    R Q = ub * (fx[1] - fx[0]) * cst<R>(P).ih + vb * (fy[1] - fy[0]) * cst<R>(P).ih;
-    R sa = R(s[c]) - dt * Q;
-    R al = alpha_c[i];
-    const R r = (R(1.0) - al) * sa + al * ((j + R(0.5)) * h - cst<R>(P).depth);
+    (xf ? Fx : Fy)[f] = ppm_face3<R>(a, (xf ? u : v)[f], R(inp[0]) * cst<R>(P).ih);
+}
+
+// sigma* = sigma^n - dt Q(u^n, sigma^n) from the face values, then damping-zone
+// relaxation.
+template <typename R>
+__global__ void __launch_bounds__(TX) k_advect(TankP P, const R *__restrict__ s, const R *__restrict__ u,
+                                               const R *__restrict__ v, const R *__restrict__ Fx,
+                                               const R *__restrict__ Fy, const double *__restrict__ inp,
+                                               const R *__restrict__ alpha_c, double *__restrict__ out,
+                                               R *__restrict__ out_w)
+{
+    pdl_entry();
+    const int nx = P.nx, i = blockIdx.y * TX + threadIdx.x, j = blockIdx.x;
+    if (i >= nx) return;
+    const int c = j * nx + i, fu = c + j;
+    const R dtih = R(inp[0]) * cst<R>(P).ih;
+    const R ub = R(0.5) * (u[fu] + u[fu + 1]), vb = R(0.5) * (v[c] + v[c + nx]);
+    const R sa = s[c] - dtih * (ub * (Fx[fu + 1] - Fx[fu]) + vb * (Fy[c + nx] - Fy[c]));
+    const R al = alpha_c[i];
+    const R r = (R(1.0) - al) * sa + al * ((j + R(0.5)) * cst<R>(P).h - cst<R>(P).depth);
     out[c] = r;
     if (out_w) out_w[c] = r;
 }
 
-// Sussman relaxation right-hand side S(sigma0)(|grad f| - 1), Godunov
-// Hamiltonian on ENO-2 (minmod) one-sided differences.
-template <typename R>
-__device__ R reinit_rhs(const TankP &P, const R *__restrict__ f, const R *__restrict__ sgn,
-                             const double *__restrict__ eta1, int i, int j)
-{
-    const R ih = cst<R>(P).ih, ih2 = R(0.5) * cst<R>(P).ih;
-    R c = R(f[j * P.nx + i]);
-    R xm2 = sig_at<R>(P, f, eta1, i - 2, j), xm1 = sig_at<R>(P, f, eta1, i - 1, j);
-    R xp1 = sig_at<R>(P, f, eta1, i + 1, j), xp2 = sig_at<R>(P, f, eta1, i + 2, j);
-    R ym2 = sig_at<R>(P, f, eta1, i, j - 2), ym1 = sig_at<R>(P, f, eta1, i, j - 1);
-    R yp1 = sig_at<R>(P, f, eta1, i, j + 1), yp2 = sig_at<R>(P, f, eta1, i, j + 2);
-    R dxm = xm2 - R(2.0) * xm1 + c, dx0 = xm1 - R(2.0) * c + xp1, dxp = c - R(2.0) * xp1 + xp2;
-    R dym = ym2 - R(2.0) * ym1 + c, dy0 = ym1 - R(2.0) * c + yp1, dyp = c - R(2.0) * yp1 + yp2;
-    R a = (c - xm1) * ih + minmod<R>(dxm, dx0) * ih2;
-    R b = (xp1 - c) * ih - minmod<R>(dx0, dxp) * ih2;
-    R cc = (c - ym1) * ih + minmod<R>(dym, dy0) * ih2;
-    R d = (yp1 - c) * ih - minmod<R>(dy0, dyp) * ih2;
-    R S = R(sgn[j * P.nx + i]);
-    R gx, gy;
-    if (S > R(0.0)) {
-        gx = fmax(sq<R>(fmax(a, R(0.0))), sq<R>(fmin(b, R(0.0))));
-        gy = fmax(sq<R>(fmax(cc, R(0.0))), sq<R>(fmin(d, R(0.0))));
-    } else {
-        gx = fmax(sq<R>(fmin(a, R(0.0))), sq<R>(fmax(b, R(0.0))));
-        gy = fmax(sq<R>(fmin(cc, R(0.0))), sq<R>(fmax(d, R(0.0))));
-    }
-    return S * (sqrt(gx + gy) - R(1.0));
-}
-
-// Smoothed sign S(sigma0) = sigma0 / sqrt(sigma0^2 + h^2), fixed over the pseudo-steps.
-template <typename R>
-__global__ void k_reinit_sign(TankP P, const R *__restrict__ s0, R *__restrict__ sgn)
-{
-    pdl_entry();
-    int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= P.nx * P.ny) return;
-    R g0 = s0[c];
-    sgn[c] = g0 / sqrt(g0 * g0 + cst<R>(P).h * cst<R>(P).h);
-}
-
-// TVD-RK2 stage: stage 1 out = f - dtau L(f); stage 2 out = (fprev + (f - dtau L(f))) / 2.
+// One TVD-RK2 stage of the Sussman relaxation: y = f - dtau S (|grad f| - 1), the
+// Godunov Hamiltonian on ENO-2 (minmod) one-sided differences, taken in units of
+// 1/h; stage 1 out = y, stage 2 (fprev) out = (fprev + y) / 2.  S = sigma0 /
+// sqrt(sigma0^2 + h^2) is fixed over the pseudo-steps: the first stage (first: f is
+// sigma0) forms it and stores it.
 template <typename R, typename TO>
-__global__ void k_reinit(TankP P, const R *__restrict__ f, const R *__restrict__ sgn,
-                         const R *__restrict__ fprev, const double *__restrict__ eta1, R dtau,
-                         TO *__restrict__ out)
+__global__ void __launch_bounds__(TX) k_reinit(TankP P, const R *__restrict__ f, R *sgn, const R *__restrict__ fprev,
+                                               const double *__restrict__ eta1, R dtau, TO *__restrict__ out, int first)
 {
     pdl_entry();
-    int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= P.nx * P.ny) return;
-    int i = c % P.nx, j = c / P.nx;
-    R s1 = R(f[c]) - dtau * reinit_rhs<R>(P, f, sgn, eta1, i, j);
-    out[c] = fprev ? R(0.5) * (R(fprev[c]) + s1) : s1;
+    const int nx = P.nx, ny = P.ny, i = blockIdx.y * TX + threadIdx.x, j = blockIdx.x;
+    if (i >= nx) return;
+    const int c0 = j * nx + i;
+    const R ih = cst<R>(P).ih, h = cst<R>(P).h, c = f[c0];
+    R S;
+    if (first)
+        sgn[c0] = S = c / sqrt(c * c + h * h);
+    else
+        S = sgn[c0];
+    const bool pos = positive(S), inner = i >= 2 && i < nx - 2 && j >= 2 && j < ny - 2;
+    R g2 = R(0.0);
+#pragma unroll
+    for (int d = 0; d < 2; ++d) {
+        const int o = d ? nx : 1, di = d == 0, dj = d;
+        R m2, m1, p1, p2;
+        if (inner) {
+            m2 = f[c0 - 2 * o];
+            m1 = f[c0 - o];
+            p1 = f[c0 + o];
+            p2 = f[c0 + 2 * o];
+        } else {
+            m2 = sig_at<R>(P, f, eta1, i - 2 * di, j - 2 * dj);
+            m1 = sig_at<R>(P, f, eta1, i - di, j - dj);
+            p1 = sig_at<R>(P, f, eta1, i + di, j + dj);
+            p2 = sig_at<R>(P, f, eta1, i + 2 * di, j + 2 * dj);
+        }
+        // the three second differences from the four first ones
+        const R e0 = c - m1, e1 = p1 - c, dm = e0 - (m1 - m2), d0 = e1 - e0, dp = (p2 - p1) - e1;
+        const R a = e0 + R(0.5) * mm3(dm, d0), nb = R(0.5) * mm3(d0, dp) - e1;
+        const R m = godunov_max(a, nb, pos);
+        g2 += m * m;
+    }
+    const R y = c - dtau * (S * (ih * sqrt(g2) - R(1.0)));
+    out[c0] = fprev ? R(0.5) * (fprev[c0] + y) : y;
 }
 
 // ---------------------------------------------------- momentum helpers ----
@@ -525,208 +476,201 @@ __global__ void k_tables(TankP P, double *t, float *t32)
     if (k <= ny) put(o3 + k, vort_shape_eval(P, k * P.h));
 }
 
-template <typename R>
-struct Fields {
-    const R *rc;              // cell density rho^n (transport)
-    const R *u, *v;           // velocities
-    const double *vin;        // left tangential inflow for v ghosts
-};
-
-template <typename R>
-__device__ __forceinline__ R ru_at(const TankP &P, const R *rc, int i, int j)
+// u, v with their ghosts where IN is false (the grid's edges); at fixed offsets
+// where the stencil is inside
+template <bool IN, typename R>
+__device__ __forceinline__ R uq2(const TankP &P, const R *__restrict__ u, int i, int j)
 {
-    i = clampi(i, 0, P.nx);
-    j = clampi(j, 0, P.ny - 1);
-    return R(0.5) * (cell_at<R>(P, rc, i - 1, j) + cell_at<R>(P, rc, i, j));
+    if constexpr (IN) return u[j * (P.nx + 1) + i]; else return u_at<R>(P, u, i, j);
+}
+template <bool IN, typename R>
+__device__ __forceinline__ R vq2(const TankP &P, const R *__restrict__ v, const double *__restrict__ vin, int i, int j)
+{
+    if constexpr (IN) return v[j * P.nx + i]; else return v_at<R>(P, v, vin, i, j);
+}
+// face densities ru [ny][nx+1], rv [ny+1][nx] (k_faces), clamped
+template <bool IN, typename R>
+__device__ __forceinline__ R ruq2(const TankP &P, const R *__restrict__ r, int i, int j)
+{
+    if constexpr (IN) return r[j * (P.nx + 1) + i];
+    return r[clampi(j, 0, P.ny - 1) * (P.nx + 1) + clampi(i, 0, P.nx)];
+}
+template <bool IN, typename R>
+__device__ __forceinline__ R rvq2(const TankP &P, const R *__restrict__ r, int i, int j)
+{
+    if constexpr (IN) return r[j * P.nx + i];
+    return r[clampi(j, 0, P.ny) * P.nx + clampi(i, 0, P.nx - 1)];
 }
 
+// Densities of rho^n on the u- and v-faces (the mean of the face's cells) and the
+// viscosities mu^n and mu^{n+1} at the nodes [ny+1][nx+1] (the mean of the four
+// cells around it, clamped into the grid), formed once per step.
 template <typename R>
-__device__ __forceinline__ R rv_at(const TankP &P, const R *rc, int i, int j)
-{
-    i = clampi(i, 0, P.nx - 1);
-    j = clampi(j, 0, P.ny);
-    return R(0.5) * (cell_at<R>(P, rc, i, j - 1) + cell_at<R>(P, rc, i, j));
-}
-
-// Consistent transport on the u-face (i, j): rho-breve and C share the mass flux.
-template <typename R>
-__device__ void transport_u(const TankP &P, const Fields<R> &X, int i, int j, R dt, R &rb, R &C)
-{
-    R m[4], f[4];
-    for (int s = 0; s < 2; ++s) {
-        int a = i - 1 + s;
-        R U = R(0.5) * (u_at<R>(P, X.u, a, j) + u_at<R>(P, X.u, a + 1, j));
-        R r = upwind<R>(ru_at<R>(P, X.rc, a - 1, j), ru_at<R>(P, X.rc, a, j), ru_at<R>(P, X.rc, a + 1, j),
-                          ru_at<R>(P, X.rc, a + 2, j), U);
-        R q = upwind<R>(u_at<R>(P, X.u, a - 1, j), u_at<R>(P, X.u, a, j), u_at<R>(P, X.u, a + 1, j),
-                          u_at<R>(P, X.u, a + 2, j), U);
-        m[s] = U * r;
-        f[s] = m[s] * q;
-    }
-    for (int s = 0; s < 2; ++s) {
-        int b = j - 1 + s;
-        R V = R(0.5) * (v_at<R>(P, X.v, X.vin, i - 1, b + 1) + v_at<R>(P, X.v, X.vin, i, b + 1));
-        R r = upwind<R>(ru_at<R>(P, X.rc, i, b - 1), ru_at<R>(P, X.rc, i, b), ru_at<R>(P, X.rc, i, b + 1),
-                          ru_at<R>(P, X.rc, i, b + 2), V);
-        R q = upwind<R>(u_at<R>(P, X.u, i, b - 1), u_at<R>(P, X.u, i, b), u_at<R>(P, X.u, i, b + 1),
-                          u_at<R>(P, X.u, i, b + 2), V);
-        m[2 + s] = V * r;
-        f[2 + s] = m[2 + s] * q;
-    }
-    rb = ru_at<R>(P, X.rc, i, j) - dt * cst<R>(P).ih * ((m[1] - m[0]) + (m[3] - m[2]));
-    C = ((R(f[1]) - R(f[0])) + (R(f[3]) - R(f[2]))) * cst<R>(P).ih;
-}
-
-template <typename R>
-__device__ void transport_v(const TankP &P, const Fields<R> &X, int i, int j, R dt, R &rb, R &C)
-{
-    R m[4], f[4];
-    for (int s = 0; s < 2; ++s) {
-        int a = i - 1 + s;
-        R U = R(0.5) * (u_at<R>(P, X.u, a + 1, j - 1) + u_at<R>(P, X.u, a + 1, j));
-        R r = upwind<R>(rv_at<R>(P, X.rc, a - 1, j), rv_at<R>(P, X.rc, a, j), rv_at<R>(P, X.rc, a + 1, j),
-                          rv_at<R>(P, X.rc, a + 2, j), U);
-        R q = upwind<R>(v_at<R>(P, X.v, X.vin, a - 1, j), v_at<R>(P, X.v, X.vin, a, j),
-                          v_at<R>(P, X.v, X.vin, a + 1, j), v_at<R>(P, X.v, X.vin, a + 2, j), U);
-        m[s] = U * r;
-        f[s] = m[s] * q;
-    }
-    for (int s = 0; s < 2; ++s) {
-        int b = j - 1 + s;
-        R V = R(0.5) * (v_at<R>(P, X.v, X.vin, i, b) + v_at<R>(P, X.v, X.vin, i, b + 1));
-        R r = upwind<R>(rv_at<R>(P, X.rc, i, b - 1), rv_at<R>(P, X.rc, i, b), rv_at<R>(P, X.rc, i, b + 1),
-                          rv_at<R>(P, X.rc, i, b + 2), V);
-        R q = upwind<R>(v_at<R>(P, X.v, X.vin, i, b - 1), v_at<R>(P, X.v, X.vin, i, b),
-                          v_at<R>(P, X.v, X.vin, i, b + 1), v_at<R>(P, X.v, X.vin, i, b + 2), V);
-        m[2 + s] = V * r;
-        f[2 + s] = m[2 + s] * q;
-    }
-    rb = rv_at<R>(P, X.rc, i, j) - dt * cst<R>(P).ih * ((m[1] - m[0]) + (m[3] - m[2]));
-    C = ((R(f[1]) - R(f[0])) + (R(f[3]) - R(f[2]))) * cst<R>(P).ih;
-}
-
-// L_mu u = div[mu (grad u + grad u^T)]: tau_xx / tau_yy at cells, tau_xy at
-// nodes with the four-cell mean viscosity.
-template <typename R>
-struct Visc {
-    const R *mu, *u, *v;
-    const double *vin;
-};
-
-template <typename R>
-__device__ __forceinline__ R mnode(const TankP &P, const Visc<R> &X, int i, int j)
-{
-    return R(0.25) * (cell_at<R>(P, X.mu, i - 1, j - 1) + cell_at<R>(P, X.mu, i, j - 1) + cell_at<R>(P, X.mu, i - 1, j) +
-                   cell_at<R>(P, X.mu, i, j));
-}
-
-template <typename R>
-__device__ __forceinline__ R txx(const TankP &P, const Visc<R> &X, int i, int j)
-{
-    return R(2.0) * cell_at<R>(P, X.mu, i, j) * (u_at<R>(P, X.u, i + 1, j) - u_at<R>(P, X.u, i, j)) * cst<R>(P).ih;
-}
-
-template <typename R>
-__device__ __forceinline__ R tyy(const TankP &P, const Visc<R> &X, int i, int j)
-{
-    return R(2.0) * cell_at<R>(P, X.mu, i, j) * (v_at<R>(P, X.v, X.vin, i, j + 1) - v_at<R>(P, X.v, X.vin, i, j)) * cst<R>(P).ih;
-}
-
-template <typename R>
-__device__ __forceinline__ R txy(const TankP &P, const Visc<R> &X, int i, int j)
-{
-    return mnode<R>(P, X, i, j) * ((u_at<R>(P, X.u, i, j) - u_at<R>(P, X.u, i, j - 1)) * cst<R>(P).ih +
-                                (v_at<R>(P, X.v, X.vin, i, j) - v_at<R>(P, X.v, X.vin, i - 1, j)) * cst<R>(P).ih);
-}
-
-template <typename R>
-__device__ __forceinline__ R visc_x(const TankP &P, const Visc<R> &X, int i, int j)
-{
-    return (txx<R>(P, X, i, j) - txx<R>(P, X, i - 1, j)) * cst<R>(P).ih + (txy<R>(P, X, i, j + 1) - txy<R>(P, X, i, j)) * cst<R>(P).ih;
-}
-
-template <typename R>
-__device__ __forceinline__ R visc_y(const TankP &P, const Visc<R> &X, int i, int j)
-{
-    return (tyy<R>(P, X, i, j) - tyy<R>(P, X, i, j - 1)) * cst<R>(P).ih + (txy<R>(P, X, i + 1, j) - txy<R>(P, X, i, j)) * cst<R>(P).ih;
-}
-
-template <typename R>
-__device__ __forceinline__ R visc_diag_x(const TankP &P, const Visc<R> &X, int i, int j)
-{
-    return -(R(2.0) * cell_at<R>(P, X.mu, i, j) + R(2.0) * cell_at<R>(P, X.mu, i - 1, j) + mnode<R>(P, X, i, j + 1) +
-             mnode<R>(P, X, i, j)) * (cst<R>(P).ih * cst<R>(P).ih);
-}
-
-template <typename R>
-__device__ __forceinline__ R visc_diag_y(const TankP &P, const Visc<R> &X, int i, int j)
-{
-    return -(R(2.0) * cell_at<R>(P, X.mu, i, j) + R(2.0) * cell_at<R>(P, X.mu, i, j - 1) + mnode<R>(P, X, i + 1, j) +
-             mnode<R>(P, X, i, j)) * (cst<R>(P).ih * cst<R>(P).ih);
-}
-
-// Right-hand side R and diagonal D of the u-momentum system; also the first
-// Jacobi iterate (u^n with the Dirichlet faces at t^{n+1}).
-template <typename R>
-__global__ void k_mom_u(TankP P, const StepScalars *S, const double *__restrict__ inp, Tabs<R> tb,
-                        const R *__restrict__ rho_n, const R *__restrict__ mu_n, const R *__restrict__ chi_1,
-                        const R *__restrict__ u, const R *__restrict__ v, const double *__restrict__ p,
-                        Bc bc, R *Ru, R *Du, R *ua)
+__global__ void __launch_bounds__(TX) k_faces(TankP P, const R *__restrict__ rho, const R *__restrict__ mu_n,
+                                              const R *__restrict__ mu_1, R *__restrict__ ru, R *__restrict__ rv,
+                                              R *__restrict__ nd_n, R *__restrict__ nd_1)
 {
     pdl_entry();
-    int f = blockIdx.x * blockDim.x + threadIdx.x;
-    const int nx = P.nx;
-    if (f >= (nx + 1) * P.ny) return;
-    const R dt = R(inp[0]);
-    int i = f % (nx + 1), j = f / (nx + 1);
-    if (i == 0) {
-        ua[f] = bc.uin1[j];
-        return;
+    const int nx = P.nx, ny = P.ny, i = blockIdx.y * TX + threadIdx.x, j = blockIdx.x;
+    if (i > nx) return;
+    const int i0 = max(i - 1, 0), i1 = min(i, nx - 1), j0 = max(j - 1, 0), j1 = min(j, ny - 1);
+    const int c00 = j0 * nx + i0, c01 = j0 * nx + i1, c10 = j1 * nx + i0, c11 = j1 * nx + i1;
+    if (j < ny) ru[j * (nx + 1) + i] = R(0.5) * (rho[c10] + rho[c11]);
+    if (i < nx) rv[j * nx + i] = R(0.5) * (rho[c01] + rho[c11]);
+    nd_n[j * (nx + 1) + i] = R(0.25) * ((mu_n[c00] + mu_n[c01]) + (mu_n[c10] + mu_n[c11]));
+    nd_1[j * (nx + 1) + i] = R(0.25) * ((mu_1[c00] + mu_1[c01]) + (mu_1[c10] + mu_1[c11]));
+}
+
+// One face of a momentum control volume of component C (0: u-face, 1: v-face) at
+// (i, j), in direction d, side s (0 lower, 1 upper): the mass flux m = U r and the
+// momentum flux f = m q, r and q the Koren-limited upwind face density and velocity
+// -- rho-breve and the convection share the mass flux.  Side 1 of a CV is side 0 of
+// the next one along d, the same values.
+template <bool IN, int C, typename R>
+__device__ __forceinline__ void cv_face(const TankP &P, const R *__restrict__ rf, const R *__restrict__ u,
+                                        const R *__restrict__ v, const double *__restrict__ vin, int i, int j, int d,
+                                        int s, R &m, R &f)
+{
+    const int o = s - 1;
+    R U;
+    if (C == 0)
+        U = d == 0 ? uq2<IN>(P, u, i + o, j) + uq2<IN>(P, u, i + o + 1, j)
+                   : vq2<IN>(P, v, vin, i - 1, j + s) + vq2<IN>(P, v, vin, i, j + s);
+    else
+        U = d == 0 ? uq2<IN>(P, u, i + s, j - 1) + uq2<IN>(P, u, i + s, j)
+                   : vq2<IN>(P, v, vin, i, j + o) + vq2<IN>(P, v, vin, i, j + o + 1);
+    U = R(0.5) * U;
+    const int di = d == 0, dj = d;
+    R rr[4], qq[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int a = i + (o - 1 + k) * di, b = j + (o - 1 + k) * dj;
+        rr[k] = C == 0 ? ruq2<IN>(P, rf, a, b) : rvq2<IN>(P, rf, a, b);
+        qq[k] = C == 0 ? uq2<IN>(P, u, a, b) : vq2<IN>(P, v, vin, a, b);
     }
-    if (i == nx) {
-        ua[f] = R(0.0);
-        return;
+    m = U * upw3(rr[0], rr[1], rr[2], rr[3], U);
+    f = m * upw3(qq[0], qq[1], qq[2], qq[3], U);
+}
+
+// The viscous operator div[mu (grad u + grad u^T)] of component C at a face:
+// h^2 L_mu(u) = S - Lc u_f, S the sum over the face's neighbours (its own component
+// and the cross terms; nd: node viscosities), Lc the sum of the coefficients (the
+// diagonal, which the Jacobi splitting moves to the left).
+template <bool IN, int C, typename R>
+__device__ __forceinline__ R visc_off(const TankP &P, const R *__restrict__ mu, const R *__restrict__ nd,
+                                      const R *__restrict__ u, const R *__restrict__ v, const double *__restrict__ vin,
+                                      int i, int j)
+{
+    const int nn = P.nx + 1;
+    if (C == 0) {
+        const R m1 = mu[j * P.nx + i], m0 = mu[j * P.nx + i - 1], n1 = nd[(j + 1) * nn + i], n0 = nd[j * nn + i];
+        return R(2.0) * (m1 * uq2<IN>(P, u, i + 1, j) + m0 * uq2<IN>(P, u, i - 1, j)) +
+               (n1 * ((uq2<IN>(P, u, i, j + 1) + vq2<IN>(P, v, vin, i, j + 1)) - vq2<IN>(P, v, vin, i - 1, j + 1)) +
+                n0 * ((uq2<IN>(P, u, i, j - 1) - vq2<IN>(P, v, vin, i, j)) + vq2<IN>(P, v, vin, i - 1, j)));
     }
-    ua[f] = R(u[f]);
-    Fields<R> X{rho_n, u, v, bc.vin0};
-    Visc<R> Vn{mu_n, u, v, bc.vin0};
-    R rb, C;
-    transport_u<R>(P, X, i, j, dt, rb, C);
-    R chi = R(0.5) * (cell_at<R>(P, chi_1, i - 1, j) + cell_at<R>(P, chi_1, i, j));
-    const R idt = R(1.0) / dt;
-    Du[f] = rb * idt + chi * cst<R>(P).ikp + tb.alpha_u[i] * rb * idt + vort_damp<R>(P, tb.vort_c[j], idt);
-    Ru[f] = ru_at<R>(P, rho_n, i, j) * R(u[f]) * idt - C + R(0.5) * visc_x<R>(P, Vn, i, j) -
-            R(p[j * nx + i] - p[j * nx + i - 1]) * cst<R>(P).ih;
+    const R m1 = mu[min(j, P.ny - 1) * P.nx + i], m0 = mu[(j - 1) * P.nx + i], n1 = nd[j * nn + i + 1], n0 = nd[j * nn + i];
+    return R(2.0) * (m1 * vq2<IN>(P, v, vin, i, j + 1) + m0 * vq2<IN>(P, v, vin, i, j - 1)) +
+           (n1 * ((vq2<IN>(P, v, vin, i + 1, j) + uq2<IN>(P, u, i + 1, j)) - uq2<IN>(P, u, i + 1, j - 1)) +
+            n0 * ((vq2<IN>(P, v, vin, i - 1, j) - uq2<IN>(P, u, i, j)) + uq2<IN>(P, u, i, j - 1)));
+}
+template <int C, typename R>
+__device__ __forceinline__ R visc_diag(const TankP &P, const R *__restrict__ mu, const R *__restrict__ nd, int i, int j)
+{
+    const int nn = P.nx + 1;
+    if (C == 0)
+        return R(2.0) * (mu[j * P.nx + i] + mu[j * P.nx + i - 1]) + (nd[(j + 1) * nn + i] + nd[j * nn + i]);
+    return R(2.0) * (mu[min(j, P.ny - 1) * P.nx + i] + mu[(j - 1) * P.nx + i]) + (nd[j * nn + i + 1] + nd[j * nn + i]);
+}
+
+// The stencils reach three cells each way (the transport's upwind triples).
+__device__ __forceinline__ bool inside2(const TankP &P, int i, int j)
+{
+    return i >= 3 && i <= P.nx - 4 && j >= 3 && j <= P.ny - 4;
 }
 
 template <typename R>
-__global__ void k_mom_v(TankP P, const StepScalars *S, const double *__restrict__ inp, Tabs<R> tb,
-                        const R *__restrict__ rho_n, const R *__restrict__ mu_n, const R *__restrict__ chi_1,
-                        const R *__restrict__ rf_1, const R *__restrict__ u, const R *__restrict__ v,
-                        const double *__restrict__ p, Bc bc, R *Rv, R *Dv, R *va)
+struct MomArgs {
+    const double *inp;
+    const StepScalars *S;
+    Tabs<R> tb;
+    const R *ru, *rv, *mu_n, *mu_1, *nd_n, *nd_1, *chi_1, *rf_1, *u, *v;
+    const double *p;
+    Bc bc;
+    R *Du, *Dv;                // diagonal (without the viscous part)
+    R *Ru, *Rv, *Qu, *Qv;      // R / D', (1 / (2 h^2)) / D' with D' = D + Lc / (2 h^2)
+    R *ua, *va;                // first Jacobi iterate: u^n with the Dirichlet faces at t^{n+1}
+};
+
+// The momentum system at the faces of component C along a row: a warp covers 31
+// control volumes, lane l forms the lower x face of its CV and takes the upper one
+// from lane l + 1 (lane 31 supplies its lower face only).
+template <int C, typename R>
+__device__ __forceinline__ void momentum_row(const TankP &P, const MomArgs<R> &M, int j)
+{
+    const int nx = P.nx, ny = P.ny, lane = threadIdx.x & 31;
+    const int ncv = C == 0 ? nx - 1 : nx;  // solved faces of the row
+    const int cv = (blockIdx.y * (TX >> 5) + (threadIdx.x >> 5)) * 31 + lane, i = cv + (C == 0 ? 1 : 0);
+    const R *rf = C == 0 ? M.ru : M.rv;
+    const double *vin = M.bc.vin0;
+    const bool in = inside2(P, i, j);
+    R m0 = R(0.0), f0 = R(0.0);
+    if (cv <= ncv) {
+        if (in)
+            cv_face<true, C, R>(P, rf, M.u, M.v, vin, i, j, 0, 0, m0, f0);
+        else
+            cv_face<false, C, R>(P, rf, M.u, M.v, vin, i, j, 0, 0, m0, f0);
+    }
+    const R m1 = shfl_down1<R>(m0), f1 = shfl_down1<R>(f0);
+    if (lane == 31 || cv >= ncv) return;
+    R my[2], fy[2], S;
+    if (in) {
+#pragma unroll
+        for (int s = 0; s < 2; ++s) cv_face<true, C, R>(P, rf, M.u, M.v, vin, i, j, 1, s, my[s], fy[s]);
+        S = visc_off<true, C, R>(P, M.mu_n, M.nd_n, M.u, M.v, vin, i, j);
+    } else {
+#pragma unroll
+        for (int s = 0; s < 2; ++s) cv_face<false, C, R>(P, rf, M.u, M.v, vin, i, j, 1, s, my[s], fy[s]);
+        S = visc_off<false, C, R>(P, M.mu_n, M.nd_n, M.u, M.v, vin, i, j);
+    }
+    const int f = C == 0 ? j * (nx + 1) + i : j * nx + i, c = min(j, ny - 1) * nx + i, cm = C == 0 ? c - 1 : (j - 1) * nx + i;
+    const TankC<R> &K = cst<R>(P);
+    const R dt = R(M.inp[0]), idt = R(1.0) / dt, ih = K.ih, hi2 = R(0.5) * ih * ih;
+    const R r0 = rf[f], w = (C == 0 ? M.u : M.v)[f];
+    const R rb = r0 - dt * ih * ((m1 - m0) + (my[1] - my[0]));
+    const R Cv = ((f1 - f0) + (fy[1] - fy[0])) * ih;
+    const R chi = R(0.5) * (M.chi_1[cm] + M.chi_1[c]), rbdt = rb * idt;
+    const R al = C == 0 ? M.tb.alpha_u[i] : M.tb.alpha_c[i];
+    const R D = rbdt + chi * K.ikp + al * rbdt + vort_damp<R>(P, C == 0 ? M.tb.vort_c[j] : M.tb.vort_v[j], idt);
+    R rhs = r0 * w * idt - Cv + hi2 * (S - visc_diag<C, R>(P, M.mu_n, M.nd_n, i, j) * w);
+    if (C == 0) {
+        rhs -= R(M.p[c] - M.p[c - 1]) * ih;
+    } else {
+        const R gp = j < ny ? R(M.p[c] - M.p[cm]) : R(-2.0) * R(M.p[cm]);
+        rhs += chi * R(M.S->zdot1) * K.ikp - R(0.5) * (M.rf_1[cm] + M.rf_1[c]) * K.g - gp * ih;
+    }
+    const R inv = R(1.0) / (D + hi2 * visc_diag<C, R>(P, M.mu_1, M.nd_1, i, j));
+    (C == 0 ? M.Du : M.Dv)[f] = D;
+    (C == 0 ? M.Ru : M.Rv)[f] = rhs * inv;
+    (C == 0 ? M.Qu : M.Qv)[f] = hi2 * inv;
+    (C == 0 ? M.ua : M.va)[f] = w;
+}
+
+// Block rows 0 .. ny-1: the u-faces; the ny+1 after them: the v-faces.
+template <typename R>
+__global__ void __launch_bounds__(TX) k_momentum(TankP P, MomArgs<R> M)
 {
     pdl_entry();
-    int f = blockIdx.x * blockDim.x + threadIdx.x;
     const int nx = P.nx, ny = P.ny;
-    if (f >= nx * (ny + 1)) return;
-    const R dt = R(inp[0]);
-    int i = f % nx, j = f / nx;
-    if (j == 0) {
-        va[f] = R(0.0);
-        return;
+    if ((int)blockIdx.x < ny) {
+        const int j = blockIdx.x;
+        if (blockIdx.y == 0 && threadIdx.x < 2) M.ua[j * (nx + 1) + threadIdx.x * nx] = threadIdx.x ? R(0.0) : R(M.bc.uin1[j]);
+        momentum_row<0, R>(P, M, j);
+    } else if ((int)blockIdx.x == ny) {  // v on the bed
+        const int cv = (blockIdx.y * (TX >> 5) + (threadIdx.x >> 5)) * 31 + (threadIdx.x & 31);
+        if (cv < nx) M.va[cv] = R(0.0);
+    } else {
+        momentum_row<1, R>(P, M, blockIdx.x - ny);
     }
-    va[f] = R(v[f]);
-    Fields<R> X{rho_n, u, v, bc.vin0};
-    Visc<R> Vn{mu_n, u, v, bc.vin0};
-    R rb, C;
-    transport_v<R>(P, X, i, j, dt, rb, C);
-    R chi = R(0.5) * (cell_at<R>(P, chi_1, i, j - 1) + cell_at<R>(P, chi_1, i, j));
-    R rf = R(0.5) * (cell_at<R>(P, rf_1, i, j - 1) + cell_at<R>(P, rf_1, i, j));
-    const R idt = R(1.0) / dt;
-    Dv[f] = rb * idt + chi * cst<R>(P).ikp + tb.alpha_c[i] * rb * idt + vort_damp<R>(P, tb.vort_v[j], idt);
-    R gp = j < ny ? R(p[j * nx + i] - p[(j - 1) * nx + i]) * cst<R>(P).ih : -R(2.0) * R(p[(ny - 1) * nx + i]) * cst<R>(P).ih;
-    Rv[f] = rv_at<R>(P, rho_n, i, j) * R(v[f]) * idt - C + R(0.5) * visc_y<R>(P, Vn, i, j) - rf * cst<R>(P).g +
-            chi * R(S->zdot1) * cst<R>(P).ikp - gp;
 }
 
 // Working buffers the stencil kernels read, in the compute type R.  An FP64 tank
@@ -740,6 +684,7 @@ struct Work {
     R *sa, *sgn, *r0, *r1, *rt;               // advected sigma, reinitialisation
     R *rho_n, *mu_n, *mu_1, *rf_1, *chi_1;    // materials
     R *Ru, *Du, *ua, *ub, *uc, *Rv, *Dv, *va, *vb, *vc;  // momentum systems, Jacobi iterates
+    R *ru, *rv, *Qu, *Qv, *nd_n, *nd_1;       // face densities, Jacobi factors, node viscosities
 };
 
 // sig, u, v -> FP32 mirrors (one thread per cell / face of the largest set).
@@ -754,37 +699,39 @@ __global__ void k_mirror(long long nc, long long nu, long long nv, const double 
     if (k < nv) v32[k] = float(v[k]);
 }
 
-// One Jacobi sweep of (D - L_mu / 2) u* = R (Crank-Nicolson implicit half),
-// splitting on the interior diagonal of L_mu; Dirichlet faces are copied.
+// One Jacobi sweep of (D - L_mu / 2) u* = R (Crank-Nicolson implicit half), split
+// on the diagonal of L_mu: B = R / D' + ((1 / (2 h^2)) / D') S(A), the two factors
+// formed with the system (k_momentum); Dirichlet faces are copied.  Block rows as
+// k_ppm_faces.
 template <typename R, typename TO>
-__global__ void k_jacobi(TankP P, const R *__restrict__ mu_1, const double *__restrict__ vin1,
-                         const R *__restrict__ Ru, const R *__restrict__ Du,
-                         const R *__restrict__ Rv, const R *__restrict__ Dv,
-                         const R *__restrict__ ua, const R *__restrict__ va, TO *__restrict__ ub,
-                         TO *__restrict__ vb)
+__global__ void __launch_bounds__(TX) k_jacobi(TankP P, const R *__restrict__ mu_1, const R *__restrict__ nd_1,
+                                               const double *__restrict__ vin1, const R *__restrict__ Ru,
+                                               const R *__restrict__ Qu, const R *__restrict__ Rv,
+                                               const R *__restrict__ Qv, const R *__restrict__ ua,
+                                               const R *__restrict__ va, TO *__restrict__ ub, TO *__restrict__ vb)
 {
     pdl_entry();
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    const int nx = P.nx, ny = P.ny;
-    const int nu = (nx + 1) * ny, nv = nx * (ny + 1);
-    Visc<R> Vk{mu_1, ua, va, vin1};
-    if (k < nu) {
-        int i = k % (nx + 1), j = k / (nx + 1);
+    const int nx = P.nx, ny = P.ny, i = blockIdx.y * TX + threadIdx.x;
+    if ((int)blockIdx.x < ny) {
+        const int j = blockIdx.x, f = j * (nx + 1) + i;
+        if (i > nx) return;
         if (i == 0 || i == nx) {
-            ub[k] = R(ua[k]);
+            ub[f] = ua[f];
             return;
         }
-        R ld = visc_diag_x<R>(P, Vk, i, j);
-        ub[k] = (R(Ru[k]) + R(0.5) * (visc_x<R>(P, Vk, i, j) - ld * R(ua[k]))) / (R(Du[k]) - R(0.5) * ld);
-    } else if (k < nu + nv) {
-        int f = k - nu;
-        int i = f % nx, j = f / nx;
+        const R S = inside2(P, i, j) ? visc_off<true, 0, R>(P, mu_1, nd_1, ua, va, vin1, i, j)
+                                     : visc_off<false, 0, R>(P, mu_1, nd_1, ua, va, vin1, i, j);
+        ub[f] = Ru[f] + Qu[f] * S;
+    } else {
+        const int j = blockIdx.x - ny, f = j * nx + i;
+        if (i >= nx) return;
         if (j == 0) {
-            vb[f] = R(va[f]);
+            vb[f] = va[f];
             return;
         }
-        R ld = visc_diag_y<R>(P, Vk, i, j);
-        vb[f] = (R(Rv[f]) + R(0.5) * (visc_y<R>(P, Vk, i, j) - ld * R(va[f]))) / (R(Dv[f]) - R(0.5) * ld);
+        const R S = inside2(P, i, j) ? visc_off<true, 1, R>(P, mu_1, nd_1, ua, va, vin1, i, j)
+                                     : visc_off<false, 1, R>(P, mu_1, nd_1, ua, va, vin1, i, j);
+        vb[f] = Rv[f] + Qv[f] * S;
     }
 }
 
@@ -931,15 +878,34 @@ __global__ void k_init_pressure(TankP P, const double *__restrict__ rf, double *
 
 inline size_t pad64(size_t n) { return (n + 63) & ~size_t(63); }
 
-// FP32 slab of a mixed tank: 11 cell arrays, 6 u-face and 6 v-face arrays, each
-// starting on a 256-byte boundary.
-size_t work_floats(size_t nc, size_t nu, size_t nv) { return 11 * pad64(nc) + 6 * pad64(nu) + 6 * pad64(nv); }
+// A tank's face and node arrays in its working type (ru, rv, Qu, Qv, nd_n, nd_1),
+// and the FP32 slab of a mixed tank: those, 11 cell arrays, 6 u-face and 6 v-face
+// arrays, each starting on a 256-byte boundary.
+size_t face_elems(size_t nu, size_t nv, size_t nn) { return 2 * (pad64(nu) + pad64(nv) + pad64(nn)); }
+size_t work_floats(size_t nc, size_t nu, size_t nv, size_t nn)
+{
+    return 11 * pad64(nc) + 6 * pad64(nu) + 6 * pad64(nv) + face_elems(nu, nv, nn);
+}
+size_t nodes(const wec_tank *T) { return (size_t)(T->P.nx + 1) * (T->P.ny + 1); }
+
+template <typename R>
+void take_faces(const wec_tank *T, Work<R> &W, R *q)
+{
+    const size_t n[6] = {T->nu, T->nv, T->nu, T->nv, nodes(T), nodes(T)};
+    R **dst[6] = {&W.ru, &W.rv, &W.Qu, &W.Qv, &W.nd_n, &W.nd_1};
+    for (int k = 0; k < 6; ++k) {
+        *dst[k] = q;
+        q += pad64(n[k]);
+    }
+}
 
 Work<double> work64(wec_tank *T)
 {
-    return Work<double>{T->sig, T->u, T->v, T->sa, T->sgn, T->r0, T->r1, T->rt, T->rho_n, T->mu_n, T->mu_1,
-                        T->rf_1, T->chi_1, T->Ru, T->Du, T->ua, T->ub, T->uc, T->Rv, T->Dv, T->va, T->vb,
-                        T->vc};
+    Work<double> W{T->sig, T->u, T->v, T->sa, T->sgn, T->r0, T->r1, T->rt, T->rho_n, T->mu_n, T->mu_1,
+                   T->rf_1, T->chi_1, T->Ru, T->Du, T->ua, T->ub, T->uc, T->Rv, T->Dv, T->va, T->vb,
+                   T->vc, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
+    take_faces(T, W, T->w64);
+    return W;
 }
 
 Work<float> work32(wec_tank *T)
@@ -953,6 +919,7 @@ Work<float> work32(wec_tank *T)
     for (float **c : uf) *c = take(T->nu);
     float **vf[] = {&W.v, &W.Rv, &W.Dv, &W.va, &W.vb, &W.vc};
     for (float **c : vf) *c = take(T->nv);
+    take_faces(T, W, q);
     return W;
 }
 
@@ -986,9 +953,13 @@ int tank_alloc_and_init(wec_tank *T)
     }
     double **vfaces[] = {&T->v, &T->vs, &T->va, &T->vb, &T->vc, &T->Rv, &T->Dv};
     if (T->opts.precision == WEC_PREC_MIXED) {
-        const size_t e = work_floats(nc, nu, nv);
+        const size_t e = work_floats(nc, nu, nv, nodes(T));
         WEC_CK(cudaMalloc(&T->w32, e * 4));
         WEC_CK(cudaMemset(T->w32, 0, e * 4));
+    } else {
+        const size_t e = face_elems(nu, nv, nodes(T));
+        WEC_CK(cudaMalloc(&T->w64, e * 8));
+        WEC_CK(cudaMemset(T->w64, 0, e * 8));
     }
     for (double **q : vfaces) {
         WEC_CK(cudaMalloc(q, nv * 8));
@@ -1099,29 +1070,32 @@ void enqueue_front_t(wec_tank *T, const Work<R> &W, cudaStream_t st)
     // (3) sigma advection + damping-zone relaxation, then reinitialisation; the
     // last pseudo-step writes sigma^{n+1} over sigma^n (no longer needed).
     {
-        WEC_PROF("advect", -1, rb * (nc + nu + nv) + (fb + (f32 ? rb : 0.0)) * nc, st);
-        launch_k(k_advect<R>, nblk(nc, TB), TB, 0, st, P, W.sig, W.u, W.v, T->bc.eta0, T->inp, tabs<R>(T).alpha_c, T->sa,
-                                                 f32 ? W.sa : nullptr);
+        // (the Jacobi buffers are free until the momentum system)
+        WEC_PROF("advect_faces", -1, rb * (nc + 2.0 * (nu + nv)), st);
+        launch_k(k_ppm_faces<R>, row_grid(P.nx + 1, 2 * P.ny + 1), TX, 0, st, P, W.sig, W.u, W.v, T->bc.eta0, T->inp, W.ub,
+                 W.vb);
+    }
+    {
+        WEC_PROF("advect", -1, rb * (nc + 2.0 * (nu + nv)) + (fb + (f32 ? rb : 0.0)) * nc, st);
+        launch_k(k_advect<R>, row_grid(P.nx, P.ny), TX, 0, st, P, W.sig, W.u, W.v, W.ub, W.vb, T->inp, tabs<R>(T).alpha_c,
+                 T->sa, f32 ? W.sa : nullptr);
     }
     const R dtau = R(0.3 * P.h);
+    const dim3 rg = row_grid(P.nx, P.ny);
     const R *f = W.sa;
     R *bufs[2] = {W.r0, W.r1};
     const int nr = T->opts.n_reinit;
-    if (nr > 0) {
-        WEC_PROF("reinit", -1, rb * 2.0 * nc, st);
-        launch_k(k_reinit_sign<R>, nblk(nc, TB), TB, 0, st, P, W.sa, W.sgn);
-    }
     for (int it = 0; it < nr; ++it) {
         {
             WEC_PROF("reinit", -1, rb * 3.0 * nc, st);
-            launch_k(k_reinit<R, R>, nblk(nc, TB), TB, 0, st, P, f, W.sgn, nullptr, T->bc.eta1, dtau, W.rt);
+            launch_k(k_reinit<R, R>, rg, TX, 0, st, P, f, W.sgn, nullptr, T->bc.eta1, dtau, W.rt, it == 0 ? 1 : 0);
         }
         WEC_PROF("reinit", -1, rb * 3.0 * nc + (it == nr - 1 ? fb : rb) * nc, st);
         if (it == nr - 1) {
-            launch_k(k_reinit<R, double>, nblk(nc, TB), TB, 0, st, P, W.rt, W.sgn, f, T->bc.eta1, dtau, T->sig);
+            launch_k(k_reinit<R, double>, rg, TX, 0, st, P, W.rt, W.sgn, f, T->bc.eta1, dtau, T->sig, 0);
         } else {
             R *dst = bufs[it & 1];
-            launch_k(k_reinit<R, R>, nblk(nc, TB), TB, 0, st, P, W.rt, W.sgn, f, T->bc.eta1, dtau, dst);
+            launch_k(k_reinit<R, R>, rg, TX, 0, st, P, W.rt, W.sgn, f, T->bc.eta1, dtau, dst, 0);
             f = dst;
         }
     }
@@ -1133,28 +1107,31 @@ void enqueue_front_t(wec_tank *T, const Work<R> &W, cudaStream_t st)
     }
     // (5) momentum right-hand side and diagonal, (6) Crank-Nicolson Jacobi sweeps
     {
-        WEC_PROF("mom_u", -1, rb * (3.0 * nc + nu + nv + 2.0 * nu) + fb * (nc + nu), st);
-        launch_k(k_mom_u<R>, nblk(nu, TB), TB, 0, st, P, T->S, T->inp, tabs<R>(T), W.rho_n, W.mu_n, W.chi_1, W.u, W.v, T->p,
-                                                T->bc, W.Ru, W.Du, W.ua);
+        WEC_PROF("faces", -1, rb * (3.0 * nc + 2.0 * (nu + nv)), st);
+        launch_k(k_faces<R>, row_grid(P.nx + 1, P.ny + 1), TX, 0, st, P, W.rho_n, W.mu_n, W.mu_1, W.ru, W.rv, W.nd_n,
+                 W.nd_1);
     }
     {
-        WEC_PROF("mom_v", -1, rb * (4.0 * nc + nu + nv + 2.0 * nv) + fb * (nc + nv), st);
-        launch_k(k_mom_v<R>, nblk(nv, TB), TB, 0, st, P, T->S, T->inp, tabs<R>(T), W.rho_n, W.mu_n, W.chi_1, W.rf_1, W.u,
-                                                W.v, T->p, T->bc, W.Rv, W.Dv, W.va);
+        WEC_PROF("momentum", -1, rb * (6.0 * nc + 6.0 * (nu + nv)) + fb * nc, st);
+        const MomArgs<R> M{T->inp, T->S, tabs<R>(T), W.ru, W.rv, W.mu_n, W.mu_1, W.nd_n, W.nd_1, W.chi_1, W.rf_1, W.u, W.v,
+                           T->p, T->bc, W.Du, W.Dv, W.Ru, W.Rv, W.Qu, W.Qv, W.ua, W.va};
+        // (31 control volumes per warp, one face more per row)
+        launch_k(k_momentum<R>, dim3(2 * P.ny + 1, (P.nx + 1 + 31 * (TX / 32) - 1) / (31 * (TX / 32))), TX, 0, st, P, M);
     }
     const R *ju = W.ua, *jv = W.va;
     R *tu[2] = {W.ub, W.uc}, *tv[2] = {W.vb, W.vc};
     const int nj = T->opts.n_jacobi;
+    const dim3 jg = row_grid(P.nx + 1, 2 * P.ny + 1);
     for (int it = 0; it < nj; ++it) {
         const bool last = it == nj - 1;
         WEC_PROF("jacobi", -1, rb * (nc + 4.0 * (nu + nv)) + fb * (nu + nv) + (last ? fb - rb : 0.0) * (nu + nv),
                  st);
         if (last) {
-            launch_k(k_jacobi<R, double>, nblk(nu + nv, TB), TB, 0, st, P, W.mu_1, T->bc.vin1, W.Ru, W.Du, W.Rv, W.Dv,
-                                                                  ju, jv, T->us, T->vs);
+            launch_k(k_jacobi<R, double>, jg, TX, 0, st, P, W.mu_1, W.nd_1, T->bc.vin1, W.Ru, W.Qu, W.Rv, W.Qv, ju, jv,
+                     T->us, T->vs);
         } else {
-            launch_k(k_jacobi<R, R>, nblk(nu + nv, TB), TB, 0, st, P, W.mu_1, T->bc.vin1, W.Ru, W.Du, W.Rv, W.Dv, ju,
-                                                             jv, tu[it & 1], tv[it & 1]);
+            launch_k(k_jacobi<R, R>, jg, TX, 0, st, P, W.mu_1, W.nd_1, T->bc.vin1, W.Ru, W.Qu, W.Rv, W.Qv, ju, jv,
+                     tu[it & 1], tv[it & 1]);
             ju = tu[it & 1];
             jv = tv[it & 1];
         }
@@ -1350,6 +1327,7 @@ void tank_free(wec_tank *T)
     for (double *q : all) cudaFree(q);
     if (T->inp_owned) cudaFree(T->inp);
     cudaFree(T->w32);
+    cudaFree(T->w64);
     cudaFree(T->tabs32);
     cudaFree(T->net_stats);
     cudaFree(T->S);

@@ -77,6 +77,7 @@ struct wec_tank {
     // mirrors, materials, reinitialisation stages, momentum right-hand sides,
     // Jacobi iterates), one allocation.  nullptr for an FP64 tank.
     float *w32 = nullptr;
+    double *w64 = nullptr;           // FP64 stencils: face densities, Jacobi factors, node viscosities
     wec::Bc bc{};
     wec::StepScalars *S = nullptr;   // device
     wec::StepScalars *Sh = nullptr;  // pinned host mirror
