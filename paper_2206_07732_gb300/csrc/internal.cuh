@@ -117,6 +117,7 @@ struct wec_poisson {
     wec::Level<double> L64[wec::kMaxLevels];
     wec::Level<float> L32[wec::kMaxLevels];
     int ncoarse = 0;
+    void *slab = nullptr;     // one allocation: the arrays from inv64 to y that follow but V, Z, w, d0
     double *inv64 = nullptr;  // explicit inverse of the coarsest operator
     float *inv32 = nullptr;
     void *band = nullptr;     // scratch of its factorisation

@@ -1435,25 +1435,9 @@ int poisson_init(wec_poisson *P, int nx, int ny, int prec, int restart, int nu1,
             P->bytes += (nu + nv + nw + 2 * nc) * 4;
         }
     }
-    const size_t ninv = (size_t)P->ncoarse * P->ncoarse;
     for (P->dense = nl - 1; P->dense > 0; --P->dense) {
         const Level<double> &A = P->L64[P->dense - 1];
         if ((long long)A.nx * A.ny * A.nz > kDense) break;
-    }
-    if (P->dense < nl - 1) {
-        const Level<double> &A = P->L64[P->dense];
-        const size_t nd = (size_t)A.nx * A.ny * A.nz;
-        if (prec == WEC_PREC_FP64)
-            WEC_CK(cudaMalloc(&P->dense64, nd * nd * 8));
-        else
-            WEC_CK(cudaMalloc(&P->dense32, nd * nd * 4));
-    }
-    if (prec == WEC_PREC_FP64) {
-        WEC_CK(cudaMalloc(&P->inv64, ninv * 8));
-        WEC_CK(cudaMalloc(&P->band, coarse_band_elems(coarse_op(P->L64[nl - 1])) * 8));
-    } else {
-        WEC_CK(cudaMalloc(&P->inv32, ninv * 4));
-        WEC_CK(cudaMalloc(&P->band, coarse_band_elems(coarse_op(P->L32[nl - 1])) * 4));
     }
     size_t n = (size_t)nx * ny * nz;
     int m = restart;
@@ -1467,19 +1451,44 @@ int poisson_init(wec_poisson *P, int nx, int ny, int prec, int restart, int nu1,
         WEC_CK(cudaMalloc(&P->kdf_d0, n * 8));
         P->bytes += (nf3[0] + nf3[1] + nf3[2] + n) * 8;
     }
-    // reduction partials: one per cluster and quantity
-    WEC_CK(cudaMalloc(&P->part, (size_t)(kMaxRestart + 2) * (kKrylovBlocks / kCl) * 8));
-    WEC_CK(cudaMalloc(&P->dots, (kMaxRestart + 2) * 8));
-    WEC_CK(cudaMalloc(&P->gram, KMAXV * KMAXV * 8));
-    WEC_CK(cudaMemset(P->gram, 0, KMAXV * KMAXV * 8));
-    size_t nh = (size_t)(m + 1) * m + 5 * (m + 1);
-    WEC_CK(cudaMalloc(&P->hess, nh * 8));
-    WEC_CK(cudaMemset(P->hess, 0, nh * 8));
-    P->cs = P->hess + (m + 1) * m;
-    P->sn = P->cs + (m + 1);
-    P->g = P->sn + (m + 1);
-    P->sc = P->g + (m + 1);
-    P->y = P->sc + (m + 1);
+    // the small arrays in one allocation: coarsest inverse, dense level's matrix,
+    // band; reduction partials (one per cluster and quantity), h1, Gram matrix,
+    // Hessenberg and the vectors beside it
+    {
+        const bool f64 = prec == WEC_PREC_FP64;
+        const size_t ts = f64 ? 8 : 4, nh = (size_t)(m + 1) * m + 5 * (m + 1);
+        const Level<double> &A = P->L64[P->dense];
+        const size_t nd = P->dense < nl - 1 ? (size_t)A.nx * A.ny * A.nz : 0, nc = P->ncoarse;
+        const size_t bytes[7] = {nc * nc * ts,
+                                 nd * nd * ts,
+                                 (f64 ? coarse_band_elems(coarse_op(P->L64[nl - 1])) : coarse_band_elems(coarse_op(P->L32[nl - 1]))) * ts,
+                                 (size_t)(kMaxRestart + 2) * (kKrylovBlocks / kCl) * 8,
+                                 (size_t)(kMaxRestart + 2) * 8,
+                                 (size_t)KMAXV * KMAXV * 8,
+                                 nh * 8};
+        size_t off[8] = {0};
+        for (int q = 0; q < 7; ++q) off[q + 1] = off[q] + (bytes[q] + 255) / 256 * 256;
+        WEC_CK(cudaMalloc(&P->slab, off[7]));
+        WEC_CK(cudaMemset(P->slab, 0, off[7]));
+        char *const b = (char *)P->slab;
+        if (f64) {
+            P->inv64 = (double *)b;
+            P->dense64 = nd ? (double *)(b + off[1]) : nullptr;
+        } else {
+            P->inv32 = (float *)b;
+            P->dense32 = nd ? (float *)(b + off[1]) : nullptr;
+        }
+        P->band = b + off[2];
+        P->part = (double *)(b + off[3]);
+        P->dots = (double *)(b + off[4]);
+        P->gram = (double *)(b + off[5]);
+        P->hess = (double *)(b + off[6]);
+        P->cs = P->hess + (m + 1) * m;
+        P->sn = P->cs + (m + 1);
+        P->g = P->sn + (m + 1);
+        P->sc = P->g + (m + 1);
+        P->y = P->sc + (m + 1);
+    }
     WEC_CK(cudaMalloc(&P->ks, sizeof(KState)));
     WEC_CK(cudaMemset(P->ks, 0, sizeof(KState)));
     WEC_CK(cudaMallocHost(&P->ksh, sizeof(KState)));
@@ -1497,10 +1506,8 @@ void poisson_free(wec_poisson *P)
         cudaFree(P->L64[l].xp); cudaFree(P->L32[l].xp);
         cudaFree(P->L64[l].id); cudaFree(P->L32[l].id);
     }
-    cudaFree(P->band);
-    cudaFree(P->inv64); cudaFree(P->inv32);
-    cudaFree(P->dense64); cudaFree(P->dense32);
-    cudaFree(P->V); cudaFree(P->Z); cudaFree(P->w); cudaFree(P->d0); cudaFree(P->part); cudaFree(P->dots); cudaFree(P->gram); cudaFree(P->hess);
+    cudaFree(P->slab);
+    cudaFree(P->V); cudaFree(P->Z); cudaFree(P->w); cudaFree(P->d0);
     for (double *&q : P->kdf_face) {
         cudaFree(q);
         q = nullptr;
