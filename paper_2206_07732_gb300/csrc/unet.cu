@@ -14,8 +14,8 @@
 // shifted descriptor; the weights of a stage arrive pre-packed in one bulk copy.
 // The stride-2 layer's input gradient (one 1x1 GEMM per sub-pixel) gathers its
 // operand with cp.async (k_conv_tc).  Weight gradients reduce over pixels, split
-// across CTAs, with m16n8k16 MMAs (k_wgrad); their partial tiles are summed in a
-// fixed order, so results are reproducible bit for bit.  ReLU masks, biases,
+// across CTAs (k_wgrad_tc); their partial tiles are summed in a fixed order, so
+// results are reproducible bit for bit.  ReLU masks, biases,
 // the skip gradient and the BF16 rounding are fused into the GEMM epilogues.
 #include <cuda_bf16.h>
 
@@ -68,10 +68,7 @@ inline int round_up(int a, int b) { return (a + b - 1) / b * b; }
 inline size_t round_up_z(size_t a, size_t b) { return (a + b - 1) / b * b; }
 
 // ----------------------------------------------------------- tile constants --
-constexpr int kBM = 128;     // GEMM rows (pixels, or weight rows in k_wgrad) per CTA
-constexpr int kBK = 32;      // reduction elements per pipeline stage
-constexpr int kGT = 256;     // threads (8 warps: 4 along M x 2 along N)
-constexpr int kStages = 3;
+constexpr int kBM = 128;     // GEMM rows (pixels, or weight rows in k_wgrad_tc) per CTA
 
 enum GatherKind { G_CONV3 = 0, G_UP3 = 1, G_DOWN2 = 2, G_DIRECT = 3 };
 enum EpiKind { E_FWD = 0, E_DX = 1, E_F32 = 2, E_DOWNDX = 3 };
@@ -121,23 +118,6 @@ template <int N>
 __device__ __forceinline__ void cp_wait()
 {
     asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
-
-__device__ __forceinline__ void ldm_x4_t(unsigned r[4], const void *p)
-{
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                 : "r"(smem_u32(p)));
-}
-
-// d += a (16x16, row) * b (16x8, col), BF16 inputs, FP32 accumulators.
-__device__ __forceinline__ void mma16816(float d[4], const unsigned a[4], const unsigned b[2])
-{
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-        "{%0,%1,%2,%3};\n"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
 // ---------------------------------------------------------- tensor layout --
@@ -948,110 +928,228 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_halo1(Halo h, const bf16
 }
 
 
-// Weight gradient: part[z][k][n] = sum over the rows p of split z of A(p, k)
-// G[p][n] for the weight rows [blockIdx.x kBM, +kBM) and columns [blockIdx.y BN,
-// +BN).  A(p, k) is the layer's forward gather; rows are taken kBK at a time.
-template <int BN>
-__global__ void __launch_bounds__(kGT) k_wgrad(Gat g, const bf16 *__restrict__ G, int ldg, int chunks_per_split,
-                                               int Kpad, float *__restrict__ part)
+// Weight gradient on tcgen05: part[z][k][n] = sum over the pixels of split z of
+// A(p, k) G[p][n], A the layer's forward gather.  The reduction runs over pixels,
+// and a chunk-planar row holds 8 channels of consecutive pixels 16 bytes apart:
+// both operands are MN-major core matrices (8 pixels x 8 channels in 128 bytes)
+// exactly as the tensors lie in memory, so a stage is one bulk copy per channel
+// chunk of a row segment.  M is the weight row (vertical tap, input channel) --
+// the 128-row tile stacks the chunks of the input rows of all vertical taps -- and
+// N the output channel; each horizontal tap is the same stage read through a
+// descriptor shifted by one 16-byte slot, into an accumulator of its own in tensor
+// memory.  An upsampling layer reads its half-grid input with the output gradient
+// de-interleaved by column parity, a stride-2 layer its input de-interleaved
+// likewise.  Units (one row segment of kWgP pixels) are split over blockIdx.z; the
+// partials are summed in split order.  Bound by the staging (an input row is read
+// once per vertical tap, from L2).  The m16n8k16 form with a per-pixel gather took
+// 2.5 ms for the 20 layers at 4 x 256 x 512; this one 0.86 (each launch timed on its
+// own).
+struct Wg {
+    const bf16 *in0, *in1, *G;
+    int c0, c1, cin;         // channels of the two tensors, and together
+    int H, W, Hi, Wi;        // output grid, input grid
+    int co, rows, Kpad;      // output channels; weight rows (vertical taps x cin; stride 2: taps x cin)
+    int xt, units, ups;      // segments per image row, units, units per split
+};
+enum WgKind { WG_CONV3 = 0, WG_UP3 = 1, WG_DOWN2 = 2 };
+constexpr int kWgP = 64;                   // reduction pixels per stage
+constexpr int kWgStages = 4;
+constexpr int kWgAcs = (kWgP + 3) * 16;    // a chunk's slots: one halo slot on either side, one of padding
+constexpr int kWgBcs = (kWgP + 1) * 16;
+
+template <int KIND, int BN>
+struct WgCfg {
+    static constexpr int kShifts = KIND == WG_DOWN2 ? 1 : 3;
+    static constexpr int kPar = KIND == WG_UP3 ? 2 : 1;  // column parities of G
+    static constexpr int kA = 16 * kWgAcs;
+    static constexpr int kB = kPar * (BN / 8) * kWgBcs;
+    static constexpr int kStage = (kA + kB + 127) / 128 * 128;
+    static constexpr int kBytes = kWgStages * kStage + 256;
+    static constexpr int kUsed = kShifts * BN;
+    static constexpr int kCols = kUsed <= 64 ? 64 : kUsed <= 128 ? 128 : kUsed <= 256 ? 256 : 512;
+    static_assert(kUsed <= 512, "accumulators exceed tensor memory");
+};
+
+template <int KIND, int BN>
+__global__ void __launch_bounds__(kTcThreads, 1) k_wgrad_tc(Wg w, float *__restrict__ part, int *err)
 {
     pdl_entry();
-    constexpr int AS = kBM + 8;
-    constexpr int BS = BN + 8;
-    constexpr int WN = BN / 2;
-    constexpr int NT = WN / 8;
-    __shared__ __align__(128) bf16 As[kStages][kBK][AS];  // [pixel][weight row]
-    __shared__ __align__(128) bf16 Bs[kStages][kBK][BS];  // [pixel][channel]
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int wm = warp & 3, wn = warp >> 2;
-    const int M = g.N * g.H * g.W, hw = g.H * g.W;
-    const int k0 = blockIdx.x * kBM, n0 = blockIdx.y * BN;
-    const int nchunks = (M + kBK - 1) / kBK;
-    const int c_begin = blockIdx.z * chunks_per_split;
-    const int c_end = min(c_begin + chunks_per_split, nchunks);
-    const int br = tid / (BN / 8), bc = tid % (BN / 8);
+    using C = WgCfg<KIND, BN>;
+    constexpr int NS = kWgStages;
+    extern __shared__ __align__(1024) unsigned char smem[];
+    unsigned char *const bars = smem + NS * C::kStage;
+    const unsigned full0 = smem_u32(bars), empty0 = full0 + 8 * NS, done = empty0 + 8 * NS;
+    unsigned *const tmem_slot = reinterpret_cast<unsigned *>(bars + 8 * (2 * NS + 1));
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int n0 = blockIdx.y * BN, u0 = blockIdx.z * w.ups, u1 = min(u0 + w.ups, w.units);
+    const int Kw = KIND == WG_UP3 ? w.Wi : w.W;  // reduction pixels of a row
+    if (tid == 0) {
+        for (int s = 0; s < NS; ++s) {
+            mbar_init(full0 + 8 * s, 128);
+            mbar_init(empty0 + 8 * s, 1);
+        }
+        mbar_init(done, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    if (warp == 4) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tmem_slot)),
+                     "r"(C::kCols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    const unsigned tmem = *tmem_slot;
+    bool ok = true;
+    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
 
-    auto load = [&](int stage, int chunk) {
-#pragma unroll
-        for (int s = 0; s < 2; ++s) {
-            const int q = tid + kGT * s, row = q >> 4, kcol = q & 15;
-            const int p = chunk * kBK + row;
+    if (warp < 4) {
+        // ---- producers: thread t < 16 stages chunk t of A, the next BN / 8 (one parity) those of B
+        const int cq = w.cin >> 3;
+        auto a_chunk = [&](int m, int &tg, const bf16 *&base, int &Ct, int &ch) {  // false: rows past the last
+            const int gc = blockIdx.x * 16 + m;
+            tg = gc / cq;
+            ch = (gc - tg * cq) * 8;
+            base = ch < w.c0 ? w.in0 : w.in1;
+            Ct = ch < w.c0 ? w.c0 : w.c1;
+            if (ch >= w.c0) ch -= w.c0;
+            return gc * 8 < w.rows;
+        };
+        int g = 0;
+        for (int un = u0; un < u1; ++un, ++g) {
+            const int s = g % NS;
+            if (g >= NS) ok = mbar_wait(empty0 + 8 * s, (unsigned)((g / NS - 1) & 1));
+            if (!ok) break;
+            unsigned char *const As = smem + s * C::kStage, *const Bs = As + C::kA;
+            const int rowid = un / w.xt, x0 = (un - rowid * w.xt) * kWgP, n = rowid / w.H, i = rowid - n * w.H;
+            unsigned bytes = 0, dst = 0;
             const bf16 *src = nullptr;
-            if (p < M) {
-                const int n = p / hw, r = p - n * hw, i = r / g.W, j = r - i * g.W;
-                src = gat_src(g, n, i, j, k0 + kcol * 8);
+            if (KIND != WG_DOWN2 && tid < 16) {
+                int tg, Ct, ch;
+                const bf16 *base;
+                const bool valid = a_chunk(tid, tg, base, Ct, ch);
+                int y = i + tg - 1;
+                const bool in = valid && y >= 0 && y < w.H;
+                if (KIND == WG_UP3) y >>= 1;
+                unsigned char *const a = As + tid * kWgAcs;
+                const int xs = max(x0 - 1, 0), xe = in ? min(x0 + kWgP + 1, w.Wi) : xs, s0 = xs - (x0 - 1);
+                for (int sl = 0; sl < s0; ++sl) *reinterpret_cast<uint4 *>(a + sl * 16) = zero;
+                for (int sl = s0 + xe - xs; sl < kWgP + 2; ++sl) *reinterpret_cast<uint4 *>(a + sl * 16) = zero;
+                if (in) {
+                    bytes = (unsigned)(xe - xs) * 16u;
+                    dst = smem_u32(a + s0 * 16);
+                    src = base + cofs((size_t)n * w.Hi + y, xs, ch, Ct, w.Wi);
+                }
             }
-            cp16(&As[stage][row][kcol * 8], src ? src : g.in0, src ? 16 : 0);
-        }
-        if (br < kBK) {
-            const int p = chunk * kBK + br;
-            const bf16 *src = G;
-            if (p < M) {
-                const size_t prow = (size_t)(p / g.W);
-                src = G + cofs(prow, p - (int)prow * g.W, n0 + bc * 8, ldg, g.W);
+            if (KIND == WG_DOWN2) {
+                // the input's even / odd columns, rows 2 i and 2 i + 1
+                for (int idx = tid; idx < 16 * kWgP; idx += 128) {
+                    const int m = idx / kWgP, k = idx - m * kWgP;
+                    int tg, Ct, ch;
+                    const bf16 *base;
+                    const bool v = a_chunk(m, tg, base, Ct, ch) && x0 + k < w.W;
+                    uint4 val = zero;
+                    if (v)
+                        val = *reinterpret_cast<const uint4 *>(
+                            base + cofs((size_t)n * w.Hi + 2 * i + (tg >> 1), 2 * (x0 + k) + (tg & 1), ch, Ct, w.Wi));
+                    *reinterpret_cast<uint4 *>(As + m * kWgAcs + k * 16) = val;
+                }
             }
-            cp16(&Bs[stage][br][bc * 8], src, p < M ? 16 : 0);
+            const int tb = tid - (KIND == WG_DOWN2 ? 0 : 16);
+            if (KIND != WG_UP3 && tb >= 0 && tb < BN / 8) {
+                unsigned char *const b = Bs + tb * kWgBcs;
+                const int nk = min(kWgP, w.W - x0);
+                for (int k = nk; k < kWgP; ++k) *reinterpret_cast<uint4 *>(b + k * 16) = zero;
+                bytes = (unsigned)nk * 16u;
+                dst = smem_u32(b);
+                src = w.G + cofs((size_t)rowid, x0, n0 + 8 * tb, w.co, w.W);
+            }
+            if (KIND == WG_UP3) {
+                for (int idx = tid; idx < 2 * (BN / 8) * kWgP; idx += 128) {
+                    const int r = idx / kWgP, k = idx - r * kWgP, b = r & 1, q = r >> 1;
+                    uint4 val = zero;
+                    if (x0 + k < w.Wi)
+                        val = *reinterpret_cast<const uint4 *>(
+                            w.G + cofs((size_t)rowid, 2 * (x0 + k) + b, n0 + 8 * q, w.co, w.W));
+                    *reinterpret_cast<uint4 *>(Bs + (b * (BN / 8) + q) * kWgBcs + k * 16) = val;
+                }
+            }
+            asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+            if (bytes) {
+                mbar_expect_tx(full0 + 8 * s, bytes);
+                bulk_g2s(dst, src, bytes, full0 + 8 * s);
+            } else {
+                mbar_arrive(full0 + 8 * s);
+            }
         }
-    };
-
-    float acc[2][NT][4];
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int b = 0; b < NT; ++b)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) acc[a][b][c] = 0.0f;
-
-    const int KT = max(c_end - c_begin, 0);
-#pragma unroll
-    for (int s = 0; s < kStages - 1; ++s) {
-        if (s < KT) load(s, c_begin + s);
-        cp_commit();
+        if (!ok)  // drain what is in flight
+            for (int q = max(0, g - NS); q < g; ++q) mbar_wait(full0 + 8 * (q % NS), (unsigned)((q / NS) & 1));
+    } else if (lane == 0) {
+        // ---- MMA issue: both operands MN-major (bits 15, 16), BF16 x BF16 -> FP32
+        constexpr unsigned idesc = umma_idesc<BN>() | (1u << 15) | (1u << 16);
+        int g = 0;
+        for (int un = u0; un < u1; ++un, ++g) {
+            const int s = g % NS;
+            ok = mbar_wait(full0 + 8 * s, (unsigned)((g / NS) & 1));
+            if (!ok) break;
+            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+            const unsigned a0 = smem_u32(smem + s * C::kStage), b0 = a0 + C::kA;
+            const int x0 = (un % w.xt) * kWgP, ks = (min(kWgP, Kw - x0) + 15) / 16;
+            for (int par = 0; par < C::kPar; ++par)
+                for (int tb = 0; tb < C::kShifts; ++tb) {
+                    const int so = KIND == WG_CONV3 ? tb : KIND == WG_UP3 ? (par + tb + 1) >> 1 : 0;
+                    for (int k = 0; k < ks; ++k) {
+                        // K step 128 B (8 pixels), M / N step one chunk
+                        const uint64_t ad = umma_desc_s(a0 + (so + 16 * k) * 16, 128, kWgAcs);
+                        const uint64_t bd = umma_desc_s(b0 + par * (BN / 8) * kWgBcs + 16 * k * 16, 128, kWgBcs);
+                        const unsigned acc = (g > 0 || par > 0 || k > 0) ? 1u : 0u;
+                        asm volatile(
+                            "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+                            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem + (unsigned)(tb * BN)),
+                            "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
+                            : "memory");
+                    }
+                }
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(empty0 + 8 * s)
+                         : "memory");
+        }
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(done) : "memory");
     }
-    for (int kt = 0; kt < KT; ++kt) {
-        cp_wait<kStages - 2>();
-        __syncthreads();
-        {
-            const int nk = kt + kStages - 1;
-            if (nk < KT) load(nk % kStages, c_begin + nk);
-            cp_commit();
-        }
-        const int st = kt % kStages;
+    // ---- the accumulators to this split's partial tile
+    const bool drained = mbar_wait(done, 0u);
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    const bool go = __all_sync(0xffffffffu, ok && drained);
+    if (warp < 4 && go) {
+        const int row = blockIdx.x * 128 + warp * 32 + lane, ta = row / w.cin, ci = row - ta * w.cin;
+        for (int tb = 0; tb < C::kShifts; ++tb) {
+            const int k = KIND == WG_DOWN2 ? row : (ta * 3 + tb) * w.cin + ci;
+            float *const o = part + ((size_t)blockIdx.z * w.Kpad + k) * w.co + n0;
+#pragma unroll 1
+            for (int c = 0; c < BN; c += 16) {
+                unsigned v[16];
+                asm volatile(
+                    "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
+                    "[%16];\n"
+                    : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+                      "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+                    : "r"(tmem + ((unsigned)(warp * 32) << 16) + (unsigned)(tb * BN + c)));
+                asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+                if (row < w.rows)
 #pragma unroll
-        for (int kk = 0; kk < kBK; kk += 16) {
-            unsigned a[2][4], b[NT][2];
-#pragma unroll
-            for (int mt = 0; mt < 2; ++mt)
-                ldm_x4_t(a[mt], &As[st][kk + (lane & 7) + ((lane >> 4) << 3)][wm * 32 + mt * 16 + ((lane >> 3) & 1) * 8]);
-#pragma unroll
-            for (int np = 0; np < NT / 2; ++np) {
-                unsigned r[4];
-                ldm_x4_t(r, &Bs[st][kk + (lane & 15)][wn * WN + np * 16 + (lane >> 4) * 8]);
-                b[2 * np][0] = r[0];
-                b[2 * np][1] = r[1];
-                b[2 * np + 1][0] = r[2];
-                b[2 * np + 1][1] = r[3];
+                    for (int q = 0; q < 4; ++q)
+                        *reinterpret_cast<uint4 *>(o + c + 4 * q) = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2],
+                                                                               v[4 * q + 3]);
             }
-#pragma unroll
-            for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-                for (int nt = 0; nt < NT; ++nt) mma16816(acc[mt][nt], a[mt], b[nt]);
         }
     }
-    cp_wait<0>();
-
-    const int ldp = gridDim.y * BN;
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int k = k0 + wm * 32 + mt * 16 + (lane >> 2) + 8 * h;
-                const int col = n0 + wn * WN + nt * 8 + 2 * (lane & 3);
-                *reinterpret_cast<float2 *>(part + ((size_t)blockIdx.z * Kpad + k) * ldp + col) =
-                    make_float2(acc[mt][nt][2 * h], acc[mt][nt][2 * h + 1]);
-            }
+    if (!(ok && drained)) atomicExch(err, 1);
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    if (warp == 4) {
+        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(C::kCols) : "memory");
+    }
 }
 
 // ------------------------------------------------------------ small kernels --
@@ -1148,19 +1246,27 @@ __global__ void __launch_bounds__(kT) k_head(const bf16 *__restrict__ a, const f
     }
 }
 
-// Head gradient and loss from the per-block partials (fixed order).
-__global__ void k_head_final(const float *__restrict__ part, int nblocks, float *__restrict__ gw, double *loss,
-                             double inv_m)
+// Head gradient and loss from the per-block partials: a CTA per value, in a
+// fixed order (one thread per value walked 2048 partials in 90 us).
+__global__ void __launch_bounds__(kT) k_head_final(const float *__restrict__ part, int nblocks, float *__restrict__ gw,
+                                                   double *loss, double inv_m)
 {
     pdl_entry();
-    const int v = threadIdx.x;
-    if (v >= kHeadVals) return;
+    __shared__ double sh[kT];
+    const int v = blockIdx.x;
     double s = 0.0;
-    for (int b = 0; b < nblocks; ++b) s += part[(size_t)b * kHeadVals + v];
+    for (int b = threadIdx.x; b < nblocks; b += kT) s += part[(size_t)b * kHeadVals + v];
+    sh[threadIdx.x] = s;
+    __syncthreads();
+    for (int h = kT / 2; h > 0; h >>= 1) {
+        if (threadIdx.x < h) sh[threadIdx.x] += sh[threadIdx.x + h];
+        __syncthreads();
+    }
+    if (threadIdx.x) return;
     if (v < 33)
-        gw[v] = (float)s;
+        gw[v] = (float)sh[0];
     else
-        *loss = s * inv_m;
+        *loss = sh[0] * inv_m;
 }
 
 // Input gradient of an upsampling layer: G(n, i, j, c) = bf16(sum of the 2x2
@@ -1186,63 +1292,67 @@ __global__ void k_up_pool(const float *__restrict__ tmp, const bf16 *__restrict_
     G[k] = __float2bfloat16_rn(__bfloat162float(low[k]) > 0.0f ? s : 0.0f);
 }
 
-// Column sums of a chunk-planar G [rows][C / 8][W][8] (bias gradient): block b
-// sums rows [b rpb, (b + 1) rpb) into part[b][C].  Thread t always meets
-// channel 8 q + t % 8 of chunk q (kT is a multiple of 8).
+// Column sums of a chunk-planar G [rows][C / 8][W][8] (bias gradient): block (q, b)
+// sums chunk q over rows [b rpb, (b + 1) rpb) into part[b][8 q ..], 16 bytes a load.
 __global__ void __launch_bounds__(kT) k_colsum(const bf16 *__restrict__ G, int rows, int W, int C, int rpb,
                                                float *__restrict__ part)
 {
     pdl_entry();
-    __shared__ float sh[32][kT];  // C / 8 <= 32 chunks
-    const int nq = C / 8;
-    float acc[32];
+    __shared__ float sh[kT / 32][8];
+    const int nq = C / 8, q = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float acc[8];
 #pragma unroll
-    for (int q = 0; q < 32; ++q) acc[q] = 0.0f;
-    const int r0 = blockIdx.x * rpb, r1 = min(r0 + rpb, rows);
-    for (int r = r0; r < r1; ++r)
+    for (int c = 0; c < 8; ++c) acc[c] = 0.0f;
+    const int r0 = blockIdx.y * rpb, r1 = min(r0 + rpb, rows);
+    for (int r = r0; r < r1; ++r) {
+        const uint4 *seg = reinterpret_cast<const uint4 *>(G + ((size_t)r * nq + q) * (size_t)W * 8);
+        for (int x = threadIdx.x; x < W; x += kT) {
+            const uint4 u = seg[x];
+            const bf16 *h = reinterpret_cast<const bf16 *>(&u);
 #pragma unroll
-        for (int q = 0; q < 32; ++q) {
-            if (q >= nq) break;
-            const bf16 *seg = G + ((size_t)r * nq + q) * (size_t)W * 8;
-            for (int idx = threadIdx.x; idx < W * 8; idx += kT) acc[q] += __bfloat162float(seg[idx]);
+            for (int c = 0; c < 8; ++c) acc[c] += __bfloat162float(h[c]);
         }
+    }
 #pragma unroll
-    for (int q = 0; q < 32; ++q)
-        if (q < nq) sh[q][threadIdx.x] = acc[q];
+    for (int c = 0; c < 8; ++c) {
+        const float s = warp_sum(acc[c]);
+        if (lane == 0) sh[warp][c] = s;
+    }
     __syncthreads();
-    if (threadIdx.x < C) {
-        const int q = threadIdx.x >> 3, c8 = threadIdx.x & 7;
+    if (threadIdx.x < 8) {
         float s = 0.0f;
-        for (int t = c8; t < kT; t += 8) s += sh[q][t];
-        part[(size_t)blockIdx.x * C + threadIdx.x] = s;
+        for (int v = 0; v < kT / 32; ++v) s += sh[v][threadIdx.x];
+        part[(size_t)blockIdx.y * C + 8 * q + threadIdx.x] = s;
     }
 }
 
-__global__ void k_colsum_final(const float *__restrict__ part, int nblocks, int C, float *__restrict__ gb)
+// A layer's gradient from its partials, in fixed order: weights gw[(t ci + c) co +
+// o] = sum_z part[z][t cinp + c][o], then the bias gw[nw + o] = sum_b cpart[b][o].
+// 32 values per CTA, the partials over 8 warps.
+__global__ void __launch_bounds__(kT) k_wgrad_reduce(const float *__restrict__ part, int splits, int Kpad, int co,
+                                                     int cinp, int ci, int nw, const float *__restrict__ cpart, int nb,
+                                                     float *__restrict__ gw)
 {
     pdl_entry();
-    const int c = blockIdx.x * kT + threadIdx.x;
-    if (c >= C) return;
+    __shared__ float sh[kT / 32][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, idx = blockIdx.x * 32 + lane;
     float s = 0.0f;
-    for (int b = 0; b < nblocks; ++b) s += part[(size_t)b * C + c];
-    gb[c] = s;
-}
-
-// Weight gradient of a layer from the split partials: gw[(t ci + c) co + o] =
-// sum_z part[z][t cinp + c][o], in split order.
-__global__ void k_wgrad_reduce(const float *__restrict__ part, int splits, int Kpad, int co, int cinp, int ci,
-                               int ntaps, float *__restrict__ gw)
-{
-    pdl_entry();
-    const long long idx = blockIdx.x * (long long)kT + threadIdx.x;
-    const long long total = (long long)ntaps * ci * co;
-    if (idx >= total) return;
-    const int o = (int)(idx % co);
-    const long long r = idx / co;
-    const int c = (int)(r % ci), t = (int)(r / ci);
-    const int k = t * cinp + c;
-    float s = 0.0f;
-    for (int z = 0; z < splits; ++z) s += part[((size_t)z * Kpad + k) * co + o];
+    if (idx < nw) {
+        const int r = idx / co, o = idx - r * co, t = r / ci, c = r - t * ci;
+        const float *p = part + (size_t)(t * cinp + c) * co + o;
+        const size_t zs = (size_t)Kpad * co;
+#pragma unroll 4
+        for (int z = warp; z < splits; z += kT / 32) s += p[z * zs];
+    } else if (idx < nw + co) {
+        const float *p = cpart + (idx - nw);
+#pragma unroll 4
+        for (int b = warp; b < nb; b += kT / 32) s += p[(size_t)b * co];
+    }
+    sh[warp][lane] = s;
+    __syncthreads();
+    if (warp || idx >= nw + co) return;
+    s = 0.0f;
+    for (int v = 0; v < kT / 32; ++v) s += sh[v][lane];
     gw[idx] = s;
 }
 
@@ -1452,8 +1562,7 @@ struct wec_net {
 namespace wec {
 namespace {
 
-constexpr int kCsumBlocks = 304;
-constexpr int kWgradTarget = 608;  // CTAs a weight-gradient launch aims for (4 per SM)
+constexpr int kCsumBlocks = 912;   // CTAs of a bias-gradient launch (6 per SM)
 
 int ilog2(int v)
 {
@@ -1650,14 +1759,60 @@ int conv_halo(wec_net *N, cudaStream_t st, int tag, int mode, int batch, int lev
     }
 }
 
-int wgrad_splits(long long M, int L, int *cps)
+// The weight-gradient GEMM of layer L: columns per CTA, CTAs per SM (by shared
+// memory), and the weight rows its 128-row tiles cover.
+struct WgShape {
+    int bn, occ, rows;
+};
+WgShape wgrad_shape(int L)
 {
-    const int co = kLayers[L].co, BN = co % 64 == 0 ? 64 : 32;
-    const int tiles = round_up(fwd_K(L), kBM) / kBM * (co / BN);
-    const int nchunks = (int)((M + kBK - 1) / kBK);
-    int splits = std::max(1, std::min((kWgradTarget + tiles - 1) / tiles, nchunks));
-    *cps = (nchunks + splits - 1) / splits;
-    return (nchunks + *cps - 1) / *cps;
+    const LayerDef &d = kLayers[L];
+    const int bn = std::min(d.co, 128);
+    return {bn, bn == 32 || (bn == 64 && d.kind != L_UP3) ? 2 : 1, (d.kind == L_DOWN2 ? 4 : 3) * cin_pad(d.ci)};
+}
+
+// Splits of its units (row segments) over blockIdx.z: at most as many CTAs as are resident.
+int wgrad_max_splits(long long units, int L)
+{
+    const WgShape w = wgrad_shape(L);
+    const int tiles = (w.rows + 127) / 128 * (kLayers[L].co / w.bn);
+    return (int)std::min<long long>(std::max(1, 152 * w.occ / tiles), units);
+}
+int wgrad_splits(long long units, int L, int *ups)
+{
+    const int splits = wgrad_max_splits(units, L);
+    *ups = (int)((units + splits - 1) / splits);
+    return (int)((units + *ups - 1) / *ups);
+}
+
+// Row segments of layer L over `rows` image rows of its output grid
+long long wgrad_units(const wec_net *N, int L, long long rows)
+{
+    const LayerDef &d = kLayers[L];
+    const int kw = level_w(N, d.level) / (d.kind == L_UP3 ? 2 : 1);
+    return rows * ((kw + kWgP - 1) / kWgP);
+}
+
+template <int KIND, int BN>
+int launch_wgrad_t(wec_net *N, const Wg &w, int splits)
+{
+    using C = WgCfg<KIND, BN>;
+    static bool set = false;
+    if (!set) {
+        WEC_CK(cudaFuncSetAttribute(k_wgrad_tc<KIND, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kBytes));
+        set = true;
+    }
+    const dim3 grid((unsigned)((w.rows + 127) / 128), (unsigned)(w.co / BN), (unsigned)splits);
+    WEC_CK(launch_k(k_wgrad_tc<KIND, BN>, grid, kTcThreads, C::kBytes, N->st, w, N->part, N->err));
+    return WEC_OK;
+}
+
+template <int KIND>
+int launch_wgrad(wec_net *N, const Wg &w, int bn, int splits)
+{
+    if constexpr (KIND != WG_DOWN2)  // (no stride-2 layer has 32 output channels)
+        if (bn == 32) return launch_wgrad_t<KIND, 32>(N, w, splits);
+    return bn == 64 ? launch_wgrad_t<KIND, 64>(N, w, splits) : launch_wgrad_t<KIND, 128>(N, w, splits);
 }
 
 // grad of layer L's weights and bias from its output gradient G.
@@ -1666,36 +1821,44 @@ int wgrad(wec_net *N, int L, int batch, const bf16 *G)
     const LayerDef &d = kLayers[L];
     const Gat g = fwd_gather(N, L, batch);
     const long long M = (long long)g.N * g.H * g.W;
-    const int Kw = round_up(g.K, kBM), BN = d.co % 64 == 0 ? 64 : 32;
-    int cps = 0;
-    const int splits = wgrad_splits(M, L, &cps);
+    const WgShape sh = wgrad_shape(L);
+    const int rows = g.N * g.H;
+    Wg w{};
+    w.in0 = g.in0;
+    w.in1 = g.in1;
+    w.G = G;
+    w.c0 = g.c0;
+    w.c1 = g.c1;
+    w.cin = g.c0 + g.c1;
+    w.H = g.H;
+    w.W = g.W;
+    w.Hi = g.Hi;
+    w.Wi = g.Wi;
+    w.co = d.co;
+    w.rows = sh.rows;
+    w.Kpad = round_up(g.K, kBM);
+    const long long units = wgrad_units(N, L, rows);
+    w.xt = (int)(units / rows);
+    w.units = (int)units;
+    const int splits = wgrad_splits(units, L, &w.ups);
     cudaStream_t st = N->st;
     {
-        WEC_PROF("net_wgrad", -1, 2.0 * M * ((double)(g.c0 + g.c1) * taps(d.kind) + d.co), st);
-        dim3 grid((unsigned)(Kw / kBM), (unsigned)(d.co / BN), (unsigned)splits);
-        if (BN == 64)
-            WEC_CK(launch_k(k_wgrad<64>, grid, kGT, 0, st, g, G, d.co, cps, Kw, N->part));
-        else
-            WEC_CK(launch_k(k_wgrad<32>, grid, kGT, 0, st, g, G, d.co, cps, Kw, N->part));
+        WEC_PROF("net_wgrad", L, 2.0 * M * ((double)w.cin + d.co), st);
+        const int e = d.kind == L_CONV3 ? launch_wgrad<WG_CONV3>(N, w, sh.bn, splits)
+                      : d.kind == L_UP3 ? launch_wgrad<WG_UP3>(N, w, sh.bn, splits)
+                                        : launch_wgrad<WG_DOWN2>(N, w, sh.bn, splits);
+        if (e) return e;
     }
-    float *gw = N->grad + N->flat[L];
-    const long long nw = (long long)weight_count(L);
-    {
-        WEC_PROF("net_wgrad_reduce", -1, 4.0 * nw * (splits + 1), st);
-        WEC_CK(launch_k(k_wgrad_reduce, nblk(nw, kT), kT, 0, st, (const float *)N->part, splits, Kw, d.co,
-                        cin_pad(d.ci), d.ci, taps(d.kind), gw));
-    }
-    const int rows = g.N * g.H;
-    const int nb = std::min(kCsumBlocks, rows);
-    const int rpb = (rows + nb - 1) / nb;
+    const int nq = d.co / 8, want = std::min(rows, std::max(1, kCsumBlocks / nq));
+    const int rpb = (rows + want - 1) / want, nb = (rows + rpb - 1) / rpb;
     {
         WEC_PROF("net_bias_grad", -1, 2.0 * M * d.co, st);
-        WEC_CK(launch_k(k_colsum, nb, kT, 0, st, G, rows, g.W, d.co, rpb, N->cpart));
+        WEC_CK(launch_k(k_colsum, dim3(nq, nb), kT, 0, st, G, rows, g.W, d.co, rpb, N->cpart));
     }
-    {
-        WEC_PROF("net_bias_grad", -1, 4.0 * nb * d.co, st);
-        WEC_CK(launch_k(k_colsum_final, nblk(d.co, kT), kT, 0, st, (const float *)N->cpart, nb, d.co, gw + nw));
-    }
+    const int nw = (int)weight_count(L);
+    WEC_PROF("net_wgrad_reduce", -1, 4.0 * nw * (splits + 1), st);
+    WEC_CK(launch_k(k_wgrad_reduce, nblk(nw + d.co, 32), kT, 0, st, (const float *)N->part, splits, w.Kpad, d.co,
+                    cin_pad(d.ci), d.ci, nw, (const float *)N->cpart, nb, N->grad + N->flat[L]));
     return WEC_OK;
 }
 
@@ -1766,7 +1929,7 @@ int forward(wec_net *N, int batch, const float *x, float *out, const float *targ
     }
     if (target) {
         WEC_PROF("net_head", -1, 4.0 * kHeadVals * nb, st);
-        WEC_CK(launch_k(k_head_final, 1, 64, 0, st, (const float *)N->cpart, nb, N->grad + N->flat[kHead], N->loss,
+        WEC_CK(launch_k(k_head_final, kHeadVals, kT, 0, st, (const float *)N->cpart, nb, N->grad + N->flat[kHead], N->loss,
                         1.0 / (double)M));
     }
     return WEC_OK;
@@ -1967,8 +2130,8 @@ int wec_net_create(int H, int W, int max_batch, void *cuda_stream, wec_net **out
     auto pix = [&](int l) { return P0 >> (2 * l); };
     size_t part_n = 0;
     for (int L = 0; L < kHead; ++L) {
-        int cps = 0;
-        const int s = wgrad_splits((long long)pix(kLayers[L].level), L, &cps);
+        // (a smaller batch may round to more splits than the largest, never above the cap)
+        const int s = wgrad_max_splits(wgrad_units(N, L, (long long)max_batch * level_h(N, kLayers[L].level)), L);
         part_n = std::max(part_n, (size_t)s * round_up(fwd_K(L), kBM) * kLayers[L].co);
     }
     int r = WEC_OK;
@@ -1990,7 +2153,7 @@ int wec_net_create(int H, int W, int max_batch, void *cuda_stream, wec_net **out
     }
     A((void **)&N->tmpf, 4 * P0 * 64);
     A((void **)&N->part, 4 * part_n);
-    A((void **)&N->cpart, 4 * (size_t)std::max(kCsumBlocks * 256, nblk((long long)P0, kT) * kHeadVals));
+    A((void **)&N->cpart, 4 * (size_t)std::max(kCsumBlocks * 8, nblk((long long)P0, kT) * kHeadVals));
     A((void **)&N->xb, 4 * P0 * kInCh);
     A((void **)&N->tb, 4 * P0);
     A((void **)&N->loss, 8);
