@@ -147,6 +147,8 @@ struct wec_poisson {
     int bottom_level = -1;      // the level the cluster kernel starts at (set by the last fused V-cycle)
     wec::KState *ks = nullptr;  // device
     wec::KState *ksh = nullptr; // pinned host mirror
+    volatile unsigned *kseq = nullptr;  // pinned, behind it: number of the last state a kernel published there
+    unsigned seq = 0;           // number of the state a host-polled solve waits for
     size_t bytes = 0;
 };
 
