@@ -211,13 +211,17 @@ __global__ void __launch_bounds__(128) k3t_materials(Tank3P P, const R *__restri
     q.c = ((long long)q.k * P.ny + q.j) * P.nx + q.i;
     const Tank3C<R> &K = cst3<R>(P);
     const R h = K.h;
-    R psi = R(1.0e3);
+    R hb = R(1);  // H_body(psi): 1 where psi exceeds the half-width
     if (P.has_body) {
+        // more than the half-width outside the cylinder's bounding box psi exceeds it
+        // too (r >= |x|, |y|): no square root and no Heaviside there
         const R x = (R(q.i) + R(0.5)) * h - K.bxc, y = (R(q.j) + R(0.5)) * h - K.byc,
                 z = (R(q.k) + R(0.5)) * h - zc;
-        psi = fmax(sqrt(x * x + y * y) - K.br, fabs(z) - scl2<R>(0.5f, K.blen));
+        const R pz = fabs(z) - scl2<R>(0.5f, K.blen), box = K.br + scl2<R>(2.f, h);
+        if (!(pz > h || fabs(x) > box || fabs(y) > box))
+            hb = heav3<R>(fmax(sqrt(x * x + y * y) - K.br, pz), h, K.ih);
     }
-    const R hf = heav3<R>(sig[q.c], h, K.ih), hb = heav3<R>(psi, h, K.ih);
+    const R hf = heav3<R>(sig[q.c], h, K.ih);
     const R rf = K.rho_w + (K.rho_a - K.rho_w) * hf;
     const R mf = K.mu_w + (K.mu_a - K.mu_w) * hf;
     rho[q.c] = K.rho_s + (rf - K.rho_s) * hb;
