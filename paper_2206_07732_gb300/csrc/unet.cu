@@ -71,7 +71,7 @@ inline size_t round_up_z(size_t a, size_t b) { return (a + b - 1) / b * b; }
 constexpr int kBM = 128;     // GEMM rows (pixels, or weight rows in k_wgrad_tc) per CTA
 
 enum GatherKind { G_CONV3 = 0, G_UP3 = 1, G_DOWN2 = 2, G_DIRECT = 3 };
-enum EpiKind { E_FWD = 0, E_DX = 1, E_F32 = 2, E_DOWNDX = 3 };
+enum EpiKind { E_FWD = 0, E_DX = 1, E_F32 = 2, E_DOWNDX = 3, E_POOL = 4 };
 
 // A operand of a convolution as an implicit GEMM.  Row (n, i, j) of the N x H x
 // W output grid, reduction index k = tap * cin + c with cin = c0 + c1 a power of
@@ -89,6 +89,8 @@ struct Gat {
 // columns < nsplit: out0 = bf16(acc * (mask0 > 0)), the rest: out1 = bf16(acc).
 // E_F32: outf = acc.  E_DOWNDX: the stride-2 layer's input gradient at the
 // sub-pixel blockIdx.z of each row's 2x2 block: out0 = bf16((acc + add) * (mask0 > 0)).
+// E_POOL (row-block tiles): an upsampling layer's input gradient on the half grid,
+// out0 = bf16(sum of acc over the 2x2 block * (mask0 > 0)).
 struct Epi {
     int kind;
     const float *bias;
@@ -729,6 +731,286 @@ __global__ void __launch_bounds__(kPThreads, 1) k_conv_halo(Halo h, const bf16 *
     if (warp == 8) {
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(kCols) : "memory");
+    }
+}
+
+// E_POOL epilogue of two image rows (accumulators t0 and t1 = rows 2i, 2i + 1): the
+// sum over each 2x2 block, rounded once, masked; lanes 2j and 2j + 1 hold a block's
+// columns and store one of its two 8-channel chunks each.  m: first pixel of the tile
+// in the half grid, nvalid: its pixels there, W2: the half grid's row length.
+template <int BN>
+__device__ __forceinline__ void pool_epilogue(const Epi &e, unsigned t0, unsigned t1, int m, int nvalid, int W2, int n0,
+                                              int warp, int lane)
+{
+    const int row = (warp * 32 + lane) >> 1, p = m + row;
+    const size_t prow = (size_t)(p / W2);
+    const int px = p - (int)prow * W2;
+#pragma unroll 1
+    for (int c0 = 0; c0 < BN; c0 += 16) {
+        float f[8];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {  // the step's two chunks; a lane keeps the one that it stores
+            float v[2][8];
+#pragma unroll
+            for (int a = 0; a < 2; ++a)
+                asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
+                             : "=f"(v[a][0]), "=f"(v[a][1]), "=f"(v[a][2]), "=f"(v[a][3]), "=f"(v[a][4]), "=f"(v[a][5]),
+                               "=f"(v[a][6]), "=f"(v[a][7])
+                             : "r"((a ? t1 : t0) + ((unsigned)(warp * 32) << 16) + (unsigned)(c0 + 8 * i)));
+            asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const float s = (v[0][q] + __shfl_xor_sync(0xffffffffu, v[0][q], 1)) +
+                                (v[1][q] + __shfl_xor_sync(0xffffffffu, v[1][q], 1));
+                if ((lane & 1) == i) f[q] = s;
+            }
+        }
+        if (row >= nvalid) continue;
+        const size_t o = cofs(prow, px, n0 + c0 + 8 * (lane & 1), e.ld0, W2);
+        const uint4 mv = *reinterpret_cast<const uint4 *>(e.mask0 + o);
+        const bf16 *mk = reinterpret_cast<const bf16 *>(&mv);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) f[q] = __bfloat162float(mk[q]) > 0.0f ? f[q] : 0.0f;
+        __align__(16) bf162 hv[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) hv[q] = __floats2bfloat162_rn(f[2 * q], f[2 * q + 1]);
+        *reinterpret_cast<uint4 *>(e.out0 + o) = *reinterpret_cast<const uint4 *>(hv);
+    }
+}
+
+// Stride-1 and upsampling convolutions of the two finest levels: a CTA's tile is
+// 128 pixels of R consecutive image rows, with an accumulator per row (two for the
+// column parities of the up mode), and the weights of all taps stay in shared
+// memory.  An input row is staged once and feeds the (up to three) output rows
+// around it, where the one-row tiles (k_conv_halo) stage it once per vertical tap
+// and fetch the weights with every stage -- at 64 channels more bytes than the
+// pixels.  The products of an output are added in the same order (channels, vertical
+// tap, horizontal tap), so the values are the same.  Persistent and
+// warp-specialised: producers (warps 0-3), MMA (warp 8), epilogue (warps 4-7), which
+// takes a row as soon as its last tap is in; a row's accumulator goes back to the
+// MMA by itself.  80 registers, so that two CTAs fit on an SM (with 100 the 32 -> 32
+// channel layer took 24 us, with 78 13).  Bound by the latency of the staged rows and
+// the epilogue's stores: 32 -> 32 channels at 256 x 1024 13 us (one-row tiles: 21) for
+// 34 MB, 64 -> 32 22 us (34); four images of 256 x 512, input gradients 32 -> 64 53 us
+// (87) and, pooled, 32 -> 64 31 us (116 + 55 with the pooling pass).
+template <int BN, int CS, bool UP, int NS>
+struct RowsCfg {
+    static constexpr int kLBO = 137 * 16;             // 136 pixel slots per chunk and one of padding
+    static constexpr int kStage = (CS / 8) * kLBO;    // an input row
+    static constexpr int kAcc = UP ? 2 : 1;           // accumulators per output row
+    static constexpr int kRows = 256 / (BN * kAcc);   // output rows per tile, at most (256 accumulator columns)
+    static int bytes(int cin) { return (9 * cin * BN * 2 + 1023) / 1024 * 1024 + NS * kStage + 256; }
+};
+
+template <int BN, int CS, bool UP, int NS>
+__global__ void __maxnreg__(80)
+    k_conv_rows(Halo h, int R, const bf16 *__restrict__ Bp, Epi e, int *err)
+{
+    pdl_entry();
+    extern __shared__ __align__(1024) unsigned char smem[];
+    using S = RowsCfg<BN, CS, UP, NS>;
+    constexpr int CH = CS / 8, RM = S::kRows, NA = S::kAcc;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int wbytes = h.nst * 3 * BN * CS * 2, ncc = h.nst / 3;
+    unsigned char *const ring = smem + (wbytes + 1023) / 1024 * 1024;
+    unsigned char *const bars = ring + NS * S::kStage;
+    const unsigned full0 = smem_u32(bars), empty0 = full0 + 8 * NS, accf0 = empty0 + 8 * NS, acce0 = accf0 + 8 * RM,
+                   wfull = acce0 + 8 * RM;
+    unsigned *const tmem_slot = reinterpret_cast<unsigned *>(bars + 8 * (2 * NS + 2 * RM + 1));
+    const int rblocks = (h.H + R - 1) / R, ntiles = h.N * rblocks * h.xtiles, nt = blockIdx.y;
+
+    if (tid == 0) {
+        for (int s = 0; s < NS; ++s) {
+            mbar_init(full0 + 8 * s, 129);  // 128 producers + the bulk copies' expect_tx arrival
+            mbar_init(empty0 + 8 * s, 1);
+        }
+        for (int q = 0; q < RM; ++q) {  // per output row: accumulator full, and read
+            mbar_init(accf0 + 8 * q, 1);
+            mbar_init(acce0 + 8 * q, 128);
+        }
+        mbar_init(wfull, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    if (warp == 8) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tmem_slot)),
+                     "r"(256)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    const unsigned tmem = *tmem_slot;
+    bool ok = true;
+
+    // tile t: column tile xt (fastest) of row block rb of image n
+    auto decode = [&](int t, int &n, int &i0, int &rv, int &x0) {
+        const int r = t / h.xtiles;
+        x0 = (t - r * h.xtiles) * kBM;
+        n = r / rblocks;
+        i0 = (r - n * rblocks) * R;
+        rv = min(R, h.H - i0);
+    };
+
+    // input rows of a tile (the up mode reads the half grid)
+    auto first_row = [&](int i0) { return UP ? (i0 >> 1) - 1 : i0 - 1; };
+    auto row_count = [&](int rv) { return UP ? (rv >> 1) + 2 : rv + 2; };
+
+    if (warp < 4) {
+        // ---- producers
+        if (tid == 0) {
+            mbar_expect_tx(wfull, (unsigned)wbytes);
+            bulk_g2s(smem_u32(smem), Bp + (size_t)nt * h.nst * 3 * BN * CS, (unsigned)wbytes, wfull);
+        }
+        int g = 0;
+        for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+            int n, i0, rv, x0;
+            decode(t, n, i0, rv, x0);
+            const int xs = max(x0 - 1, 0), xe = min(x0 - 1 + 136, h.Wi), s0 = xs - (x0 - 1);
+            for (int cc = 0; cc < ncc && ok; ++cc) {
+                const int cb = cc * CS;
+                const bf16 *tbase = cb < h.c0 ? h.in0 : h.in1;
+                const int tC = cb < h.c0 ? h.c0 : h.c1, coff = cb < h.c0 ? cb : cb - h.c0;
+                for (int q = 0; q < row_count(rv); ++q, ++g) {
+                    const int s = g % NS, y = first_row(i0) + q;
+                    if (g >= NS) ok = mbar_wait(empty0 + 8 * s, (unsigned)((g / NS - 1) & 1));
+                    if (!ok) break;
+                    unsigned char *const As = ring + s * S::kStage;
+                    const bool row_ok = y >= 0 && y < h.Hi;
+                    if (tid == 0) {
+                        mbar_expect_tx(full0 + 8 * s, row_ok ? (unsigned)(xe - xs) * 16u * CH : 0u);
+                        if (row_ok)
+                            for (int c = 0; c < CH; ++c)
+                                bulk_g2s(smem_u32(As + c * S::kLBO + s0 * 16),
+                                         tbase + cofs((size_t)n * h.Hi + y, xs, coff + 8 * c, tC, h.Wi),
+                                         (unsigned)(xe - xs) * 16u, full0 + 8 * s);
+                    }
+                    if (!row_ok || s0 > 0 || xe - xs < 136)
+                        for (int idx = tid; idx < 136 * CH; idx += 128) {
+                            const int c = idx % CH, sl = idx / CH;
+                            if (!(row_ok && sl >= s0 && sl < s0 + (xe - xs)))
+                                *reinterpret_cast<uint4 *>(As + c * S::kLBO + sl * 16) = make_uint4(0u, 0u, 0u, 0u);
+                        }
+                    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+                    mbar_arrive(full0 + 8 * s);
+                }
+            }
+        }
+        if (!ok)  // drain what is in flight
+            for (int q = max(0, g - NS); q < g; ++q) mbar_wait(full0 + 8 * (q % NS), (unsigned)((q / NS) & 1));
+    } else if (warp == 8) {
+        if (lane == 0) {
+            // ---- MMA issue
+            constexpr unsigned idesc = umma_idesc<BN>();
+            ok = mbar_wait(wfull, 0u);
+            const unsigned w0 = smem_u32(smem);
+            unsigned used = 0;  // per output row: parity of the uses of its accumulator
+            int g = 0;
+            for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+                int n, i0, rv, x0;
+                decode(t, n, i0, rv, x0);
+                for (int cc = 0; cc < ncc && ok; ++cc)
+                    for (int q = 0; q < row_count(rv); ++q, ++g) {
+                        const int s = g % NS; // input row first_row + q
+                        ok = mbar_wait(full0 + 8 * s, (unsigned)((g / NS) & 1));
+                        if (!ok) break;
+                        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                        const unsigned a0 = smem_u32(ring + s * S::kStage);
+                        // output row r reads it with vertical tap q - r; in the up mode with those of
+                        // r + ta = 2q - 1 and 2q
+                        for (int r = max(0, (UP ? 2 * q : q) - (UP ? 3 : 2)); r < min(rv, (UP ? 2 * q : q) + 1) && ok; ++r) {
+                            const int ta0 = UP ? max(2 * q - 1 - r, 0) : q - r, ta1 = UP ? min(2 * q - r, 2) : q - r;
+                            for (int ta = ta0; ta <= ta1; ++ta) {
+                                if (cc == 0 && ta == 0) {  // the last tile's row r has been read
+                                    ok = mbar_wait(acce0 + 8 * r, (~used >> r) & 1u);
+                                    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                                    if (!ok) break;
+                                }
+                                const unsigned b0 = w0 + (unsigned)((cc * 3 + ta) * 3) * (BN * CS * 2);
+#pragma unroll
+                                for (int b = 0; b < NA; ++b)
+#pragma unroll
+                                    for (int tb = 0; tb < 3; ++tb) {
+                                        const int so = UP ? (b + tb + 1) >> 1 : tb;
+#pragma unroll
+                                        for (int kk = 0; kk < CS / 16; ++kk) {
+                                            const uint64_t ad = umma_desc_s(a0 + 2 * kk * S::kLBO + so * 16, S::kLBO, 128);
+                                            const uint64_t bd =
+                                                umma_desc_s(b0 + tb * (BN * CS * 2) + 2 * kk * 128, 128, CH * 128);
+                                            const unsigned acc = (cc > 0 || ta > 0 || tb > 0 || kk > 0) ? 1u : 0u;
+                                            asm volatile(
+                                                "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+                                                "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
+                                                    tmem + (unsigned)((r * NA + b) * BN)),
+                                                "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
+                                                : "memory");
+                                        }
+                                    }
+                            }
+                        }
+                        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
+                                         empty0 + 8 * s)
+                                     : "memory");
+                        if (cc == ncc - 1)  // rows that took their last tap here
+                            for (int r = max(0, UP ? 2 * q - 3 : q - 2); r < min(rv, UP ? 2 * q - 1 : q - 1); ++r) {
+                                used ^= 1u << r;
+                                asm volatile(
+                                    "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
+                                        accf0 + 8 * r)
+                                    : "memory");
+                            }
+                    }
+            }
+            // no MMA in flight past this point (the last stage's commit covers all before it)
+            if (g > 0 && !mbar_wait(empty0 + 8 * ((g - 1) % NS), (unsigned)(((g - 1) / NS) & 1))) ok = false;
+        }
+    } else {
+        // ---- epilogue (warps 4-7: TMEM lanes 32 (warp - 4) .. +31)
+        Gat g{};  // the epilogue needs only the output grid
+        g.N = h.N;
+        g.H = h.H;
+        g.W = h.W;
+        unsigned used = 0;
+        for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+            int n, i0, rv, x0;
+            decode(t, n, i0, rv, x0);
+            const bool pool = e.kind == E_POOL;
+            const int ps = UP ? 2 : 1, nvalid = min(kBM, (UP ? h.Wi : h.W) - x0);
+            bool go = true;
+            for (int r = 0; r < rv && go; ++r) {
+                const bool ok2 = mbar_wait(accf0 + 8 * r, (used >> r) & 1u);
+                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                go = __all_sync(0xffffffffu, ok2);
+                used ^= 1u << r;
+                if (pool) {  // rows in pairs (rv is even)
+                    if (!(r & 1) || !go) continue;
+                    const int W2 = h.W >> 1, m = (n * (h.H >> 1) + ((i0 + r) >> 1)) * W2 + (x0 >> 1);
+                    pool_epilogue<BN>(e, tmem + (unsigned)((r - 1) * BN), tmem + (unsigned)(r * BN), m, nvalid >> 1, W2,
+                                      nt * BN, warp - 4, lane);
+                } else {
+#pragma unroll
+                    for (int b = 0; b < NA; ++b) {
+                        const int m0 = (n * h.H + i0 + r) * h.W + ps * x0 + b;
+                        tc_epilogue<BN>(e, g, tmem + (unsigned)((r * NA + b) * BN), m0, nt * BN, m0 + ps * nvalid, warp - 4,
+                                        lane, go, ps);
+                    }
+                }
+                asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+                if (pool) mbar_arrive(acce0 + 8 * (r - 1));
+                mbar_arrive(acce0 + 8 * r);
+            }
+            if (!go) {
+                ok = false;
+                break;
+            }
+        }
+    }
+    if (!ok) atomicExch(err, 1);
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    if (warp == 8) {
+        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(256) : "memory");
     }
 }
 
@@ -1548,7 +1830,7 @@ struct wec_net {
     bf16 *act[wec::kNumLayers] = {};          // layer outputs
     float *out = nullptr;                     // [maxb][H][W]
     bf16 *gA[4] = {}, *gB[4] = {}, *skip[3] = {};  // gradients per level
-    float *tmpf = nullptr;                    // input gradient of an upsampling layer (full grid)
+    float *tmpf = nullptr;                    // input gradient of the coarsest upsampling layer (its output grid)
     float *part = nullptr;                    // split-K partials of the weight gradients
     size_t part_n = 0;
     float *cpart = nullptr;                   // column-sum / head partials
@@ -1728,6 +2010,54 @@ int launch_halo_cs(int CS, bool down, cudaStream_t st, long long ntiles, const H
     return fail(WEC_ERR_INVALID, "net: unsupported channels per stage");
 }
 
+// Column-tile width of the row-block kernel (k_conv_rows), or 0 where it does not
+// apply: the two finest levels (below them the weights of all taps do not fit beside
+// a second CTA), the widest tile whose weights take at most 76 KB, and at most 64
+// output columns: 64 -> 128 channels took 49 us against 46 with the one-row tiles,
+// four images of 256 x 512, but with E_POOL, which replaces two passes over an FP32
+// full grid, 27 against 55 + 30.  The up mode only with three stages: with two,
+// 128 -> 64 channels took 25 us against 22.
+int rows_bn(int mode, int level, int cin, int ncols, bool pool = false)
+{
+    if (mode == H_DOWN2 || level > 1 || (ncols > 64 && !pool)) return 0;
+    if (mode == H_UP3) return cin == 64 && ncols == 32 ? 32 : 0;
+    for (int bn : {64, 32})
+        if (ncols % bn == 0 && 9 * cin * bn * 2 <= 76 * 1024) return bn;
+    return 0;
+}
+
+template <int BN, int CS, bool UP, int NS>
+int launch_rows_t(cudaStream_t st, const Halo &h, const bf16 *B, const Epi &e, int *err)
+{
+    using S = RowsCfg<BN, CS, UP, NS>;
+    auto kern = k_conv_rows<BN, CS, UP, NS>;
+    const int smem = S::bytes(h.c0 + h.c1);
+    static bool attr = false;
+    if (!attr) {
+        WEC_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 113 * 1024));
+        attr = true;
+    }
+    const int ntn = h.ncols / BN, slots = 2 * 152 / ntn;
+    // rows per tile: as many as the accumulators hold, fewer where the tiles would not fill the GPU
+    int R = S::kRows;
+    auto tiles = [&](int r) { return (long long)h.N * ((h.H + r - 1) / r) * h.xtiles; };
+    while (R > 2 && tiles(R) < slots) R /= 2;
+    const dim3 grid((unsigned)std::min<long long>(tiles(R), slots), (unsigned)ntn);
+    WEC_CK(launch_k(kern, grid, kPThreads, smem, st, h, R, B, e, err));
+    return WEC_OK;
+}
+
+int launch_rows(int BN, int CS, cudaStream_t st, const Halo &h, const bf16 *B, const Epi &e, int *err)
+{
+    const bool wide = 9 * (h.c0 + h.c1) * BN * 2 > 56 * 1024;  // two stages beside the weights, else three or four
+    if (h.mode == H_UP3) return launch_rows_t<32, 64, true, 3>(st, h, B, e, err);
+    if (BN == 64)
+        return wide ? launch_rows_t<64, 64, false, 2>(st, h, B, e, err) : launch_rows_t<64, 32, false, 4>(st, h, B, e, err);
+    if (CS == 64)
+        return wide ? launch_rows_t<32, 64, false, 2>(st, h, B, e, err) : launch_rows_t<32, 64, false, 3>(st, h, B, e, err);
+    return CS == 32 ? launch_rows_t<32, 32, false, 4>(st, h, B, e, err) : launch_rows_t<32, 16, false, 4>(st, h, B, e, err);
+}
+
 // A convolution of the given HaloMode whose output grid is the level's: input
 // channels [0, c0) from in0 and [c0, c0 + c1) from in1 (concatenation; c1 = 0:
 // one tensor), ncols output channels, halo-ordered weights B of tile width BN.
@@ -1752,6 +2082,7 @@ int conv_halo(wec_net *N, cudaStream_t st, int tag, int mode, int batch, int lev
     const long long ntiles = (long long)batch * h.H * h.xtiles * (ncols / BN);
     const double M = (double)batch * h.H * h.W;
     WEC_PROF("net_conv", tag, 2.0 * M * ((double)(h.c0 + h.c1) + ncols) + 2.0 * tv * tv * (h.c0 + h.c1) * ncols, st);
+    if (rows_bn(mode, level, h.c0 + h.c1, ncols, e.kind == E_POOL)) return launch_rows(BN, CS, st, h, B, e, N->err);
     switch (BN) {
     case 128: return launch_halo_cs<128>(CS, mode == H_DOWN2, st, ntiles, h, B, e, N->err);
     case 64: return launch_halo_cs<64>(CS, mode == H_DOWN2, st, ntiles, h, B, e, N->err);
@@ -1955,16 +2286,23 @@ int backward(wec_net *N, int batch)
         e.ld1 = C;
         if (int r = dx_conv(N, cat(l), batch, N->gB[l], e)) return r;
         if (int r = wgrad(N, up(l), batch, N->gA[l])) return r;
+        const bf16 *low = l == 2 ? N->act[enc_b(3)] : N->act[dec(l + 1)];
         Epi f{};
+        f.ld0 = 2 * C;
+        if (rows_bn(H_CONV3, l, C, 2 * C, true)) {  // the 2x2 sums in the epilogue
+            f.kind = E_POOL;
+            f.out0 = N->gA[l + 1];
+            f.mask0 = low;
+            if (int r = dx_conv(N, up(l), batch, N->gA[l], f)) return r;
+            continue;
+        }
         f.kind = E_F32;
         f.outf = N->tmpf;
-        f.ld0 = 2 * C;
         if (int r = dx_conv(N, up(l), batch, N->gA[l], f)) return r;
         const int h = level_h(N, l + 1), w = level_w(N, l + 1);
         const long long n = (long long)batch * h * w * 2 * C;
         WEC_PROF("net_up_pool", -1, 16.0 * n + 4.0 * n, st);
-        WEC_CK(launch_k(k_up_pool, nblk(n, kT), kT, 0, st, (const float *)N->tmpf,
-                        (const bf16 *)(l == 2 ? N->act[enc_b(3)] : N->act[dec(l + 1)]), batch, h, w, 2 * C,
+        WEC_CK(launch_k(k_up_pool, nblk(n, kT), kT, 0, st, (const float *)N->tmpf, low, batch, h, w, 2 * C,
                         N->gA[l + 1]));
     }
     for (int l = 3; l >= 0; --l) {  // encoder; G of down(l)'s output is in gA[l + 1]
@@ -2116,12 +2454,14 @@ int wec_net_create(int H, int W, int max_batch, void *cuda_stream, wec_net **out
             nw = round_up_z(nw + weight_count(L), 64);
         }
         if (halo_fwd(L)) {
-            N->bnf[L] = halo_bn(N, d.level, d.co, d.kind == L_UP3);
+            N->bnf[L] = rows_bn(halo_mode(d.kind), d.level, cin_pad(d.ci), d.co);
+            if (!N->bnf[L]) N->bnf[L] = halo_bn(N, d.level, d.co, d.kind == L_UP3);
             N->hf[L] = nw;
             nw = round_up_z(nw + (size_t)taps(d.kind) * halo_kin(L, false) * d.co, 64);
         }
         if (halo_bwd(L)) {
-            N->bnb[L] = halo_bn(N, d.level, d.ci);
+            N->bnb[L] = rows_bn(H_CONV3, d.level, d.co, d.ci, d.kind == L_UP3);
+            if (!N->bnb[L]) N->bnb[L] = halo_bn(N, d.level, d.ci);
             N->hb[L] = nw;
             nw = round_up_z(nw + 9 * (size_t)halo_kin(L, true) * d.ci, 64);
         }
@@ -2151,7 +2491,7 @@ int wec_net_create(int H, int W, int max_batch, void *cuda_stream, wec_net **out
         A((void **)&N->gB[l], 2 * pix(l) * chans(l));
         if (l < 3) A((void **)&N->skip[l], 2 * pix(l) * chans(l));
     }
-    A((void **)&N->tmpf, 4 * P0 * 64);
+    A((void **)&N->tmpf, 4 * pix(2) * 2 * chans(2));
     A((void **)&N->part, 4 * part_n);
     A((void **)&N->cpart, 4 * (size_t)std::max(kCsumBlocks * 8, nblk((long long)P0, kT) * kHeadVals));
     A((void **)&N->xb, 4 * P0 * kInCh);
