@@ -8,12 +8,12 @@
 // BF16 tensors ([rows][C / 8][W][8]).  The forward convolutions (3x3, nearest
 // upsampling + 3x3, 2x2 stride 2) and the 3x3 input gradients (the 3x3
 // convolution of the output gradient with the flipped, transposed weights) run
-// in the halo kernels (k_conv_halo persistent and warp-specialised,
-// k_conv_halo1 one tile per CTA): a stage holds one input row of one channel
-// chunk, staged by bulk copy, and every horizontal tap reads it through a
-// shifted descriptor; the weights of a stage arrive pre-packed in one bulk copy.
-// The stride-2 layer's input gradient (one 1x1 GEMM per sub-pixel) gathers its
-// operand with cp.async (k_conv_tc).  Weight gradients reduce over pixels, split
+// in the halo kernels (k_conv_rows for the two finest levels, k_conv_halo persistent
+// and warp-specialised, k_conv_halo1 one tile per CTA): a stage holds one input row of
+// one channel chunk, staged by bulk copy, and every horizontal tap reads it through a
+// shifted descriptor; the weights arrive pre-packed by bulk copy.  The stride-2
+// layer's input gradient is one GEMM for all four sub-pixels (k_down_dx).  Weight
+// gradients reduce over pixels, split
 // across CTAs (k_wgrad_tc); their partial tiles are summed in a fixed order, so
 // results are reproducible bit for bit.  ReLU masks, biases,
 // the skip gradient and the BF16 rounding are fused into the GEMM epilogues.
@@ -70,25 +70,23 @@ inline size_t round_up_z(size_t a, size_t b) { return (a + b - 1) / b * b; }
 // ----------------------------------------------------------- tile constants --
 constexpr int kBM = 128;     // GEMM rows (pixels, or weight rows in k_wgrad_tc) per CTA
 
-enum GatherKind { G_CONV3 = 0, G_UP3 = 1, G_DOWN2 = 2, G_DIRECT = 3 };
 enum EpiKind { E_FWD = 0, E_DX = 1, E_F32 = 2, E_DOWNDX = 3, E_POOL = 4 };
 
-// A operand of a convolution as an implicit GEMM.  Row (n, i, j) of the N x H x
-// W output grid, reduction index k = tap * cin + c with cin = c0 + c1 a power of
-// two; channel c < c0 comes from in0, the rest from in1 (concatenation).
+// The input tensors of a layer and its output grid: channel c < c0 comes from in0,
+// the rest from in1 (concatenation).
 struct Gat {
     const bf16 *in0, *in1;
-    int c0, c1, lcin;  // log2(cin)
-    int kind;
+    int c0, c1;
     int N, H, W;       // output grid
     int Hi, Wi;        // grid of the input tensors
-    int K;             // taps * cin; k >= K reads zeros (padding of the reduction)
+    int K;             // taps * (c0 + c1)
 };
 
 // Fused epilogue.  E_FWD: out0 = bf16(relu(acc + bias)).  E_DX: input gradient;
 // columns < nsplit: out0 = bf16(acc * (mask0 > 0)), the rest: out1 = bf16(acc).
-// E_F32: outf = acc.  E_DOWNDX: the stride-2 layer's input gradient at the
-// sub-pixel blockIdx.z of each row's 2x2 block: out0 = bf16((acc + add) * (mask0 > 0)).
+// E_F32: outf = acc.  E_DOWNDX: the stride-2 layer's input gradient, column z ld0 + c
+// channel c at sub-pixel z of each half-grid pixel's 2x2 block:
+// out0 = bf16((acc + add) * (mask0 > 0)).
 // E_POOL (row-block tiles): an upsampling layer's input gradient on the half grid,
 // out0 = bf16(sum of acc over the 2x2 block * (mask0 > 0)).
 struct Epi {
@@ -132,89 +130,16 @@ __device__ __forceinline__ size_t cofs(size_t row, int x, int c, int C, int W)
     return ((row * (size_t)(C >> 3) + (size_t)(c >> 3)) * (size_t)W + (size_t)x) * 8 + (size_t)(c & 7);
 }
 
-// ------------------------------------------------------------------ gather --
-// Address of the 8 channels [c, c + 8) of reduction index k for output pixel
-// (n, i, j), or nullptr where the operand is zero (outside the image, k >= K).
-__device__ __forceinline__ const bf16 *gat_src(const Gat &g, int n, int i, int j, int k)
-{
-    if (k >= g.K) return nullptr;
-    const int t = k >> g.lcin, c = k & ((1 << g.lcin) - 1);
-    int ii = i, jj = j;
-    if (g.kind == G_CONV3 || g.kind == G_UP3) {
-        const int ta = t / 3, tb = t - 3 * ta;
-        ii = i + ta - 1;
-        jj = j + tb - 1;
-        if (ii < 0 || jj < 0 || ii >= g.H || jj >= g.W) return nullptr;
-        if (g.kind == G_UP3) {  // nearest upsampling: the input is the half grid
-            ii >>= 1;
-            jj >>= 1;
-        }
-    } else if (g.kind == G_DOWN2) {
-        ii = 2 * i + (t >> 1);
-        jj = 2 * j + (t & 1);
-    }
-    const size_t row = (size_t)n * g.Hi + ii;
-    return c < g.c0 ? g.in0 + cofs(row, jj, c, g.c0, g.Wi) : g.in1 + cofs(row, jj, c - g.c0, g.c1, g.Wi);
-}
-
-__device__ __forceinline__ void epi_store(const Epi &e, const Gat &g, int p, int col, float v0, float v1)
-{
-    const size_t prow = (size_t)(p / g.W);
-    const int px = p - (int)prow * g.W;
-    if (e.kind == E_FWD) {
-        v0 = fmaxf(v0 + e.bias[col], 0.0f);
-        v1 = fmaxf(v1 + e.bias[col + 1], 0.0f);
-        *reinterpret_cast<bf162 *>(e.out0 + cofs(prow, px, col, e.ld0, g.W)) = __floats2bfloat162_rn(v0, v1);
-    } else if (e.kind == E_DX) {
-        if (col < e.nsplit) {
-            const size_t o = cofs(prow, px, col, e.ld0, g.W);
-            const bf162 m = *reinterpret_cast<const bf162 *>(e.mask0 + o);
-            v0 = __bfloat162float(m.x) > 0.0f ? v0 : 0.0f;
-            v1 = __bfloat162float(m.y) > 0.0f ? v1 : 0.0f;
-            *reinterpret_cast<bf162 *>(e.out0 + o) = __floats2bfloat162_rn(v0, v1);
-        } else {
-            *reinterpret_cast<bf162 *>(e.out1 + cofs(prow, px, col - e.nsplit, e.ld1, g.W)) =
-                __floats2bfloat162_rn(v0, v1);
-        }
-    } else if (e.kind == E_F32) {
-        *reinterpret_cast<float2 *>(e.outf + (size_t)p * e.ld0 + col) = make_float2(v0, v1);
-    } else {  // E_DOWNDX: row p = (n, i, j) of the half grid -> (n, 2i + a, 2j + b)
-        const int hw = g.H * g.W, n = p / hw, r = p - n * hw, i = r / g.W, j = r - i * g.W;
-        const int a = blockIdx.z >> 1, b = blockIdx.z & 1;
-        const size_t o = cofs((size_t)n * (2 * g.H) + 2 * i + a, 2 * j + b, col, e.ld0, 2 * g.W);
-        const bf162 s = *reinterpret_cast<const bf162 *>(e.add + o);
-        const bf162 m = *reinterpret_cast<const bf162 *>(e.mask0 + o);
-        v0 = __bfloat162float(m.x) > 0.0f ? v0 + __bfloat162float(s.x) : 0.0f;
-        v1 = __bfloat162float(m.y) > 0.0f ? v1 + __bfloat162float(s.y) : 0.0f;
-        *reinterpret_cast<bf162 *>(e.out0 + o) = __floats2bfloat162_rn(v0, v1);
-    }
-}
-
-// ------------------------------------------------- tcgen05 implicit GEMM --
-// The same convolution GEMM on the 5th-generation tensor cores: one CTA owns a
-// 128-pixel x BN-channel tile whose FP32 accumulator lives in tensor memory.
-// Warps 0-3 gather A (one pixel row each) and B (K-major weights) into shared
-// memory in the no-swizzle K-major core-matrix layout (8 rows x 16 bytes per
-// core matrix; K-adjacent core matrices 128 B apart, 8-row groups 1024 B
-// apart), kTcStages stages of 64 reduction elements; one thread of warp 4
-// issues tcgen05.mma (M = 128, N = BN, K = 16, BF16 x BF16 -> FP32) and
-// signals each consumed stage through tcgen05.commit.  Warps 0-3 then read
-// their 32 TMEM lanes (tcgen05.ld) and run the fused epilogue.  Every wait is
-// bounded: on expiry the kernel raises *err, drains its copies, frees its
-// tensor memory and returns.
-constexpr int kTcStages = 4;
+// ---------------------------------------------------------------- tcgen05 --
+// Tensor-core tiles: one CTA owns 128 pixels x BN channels whose FP32 accumulator
+// lives in tensor memory; operands in shared memory in the no-swizzle K-major
+// core-matrix layout (8 rows x 16 bytes per core matrix); one thread issues
+// tcgen05.mma (M = 128, N = BN, K = 16, BF16 x BF16 -> FP32).  Every wait is bounded:
+// on expiry the kernel raises *err, drains its copies, frees its tensor memory and
+// returns.
 constexpr int kTcK = 64;               // reduction elements per stage
 constexpr int kTcThreads = 160;        // warps 0-3: producers / epilogue; warp 4: MMA
-constexpr int kTcLag = 2;              // stages a producer keeps in flight before signalling
 constexpr long long kWaitLimit = 1LL << 22;  // polls; far above any legitimate wait here
-
-template <int BN>
-struct TcSmem {
-    static constexpr int kA = kBM * kTcK * 2;   // 16 KB
-    static constexpr int kB = BN * kTcK * 2;
-    static constexpr int kStage = kA + kB;
-    static constexpr int kBytes = kTcStages * kStage + 256;  // + barriers and the TMEM address
-};
 
 __device__ __forceinline__ void mbar_init(unsigned a, unsigned count)
 {
@@ -257,17 +182,14 @@ __host__ __device__ constexpr unsigned umma_idesc()
 
 // Epilogue of a tensor-core tile: the calling warp (warp = TMEM lane quarter)
 // reads its 32 tile rows; tile row r is pixel m0 + r ps, valid below M.  The
-// forward (bias + ReLU) and input-gradient (ReLU mask of the layer input, split
-// into two outputs at nsplit) epilogues store each 8-channel chunk of a row as
-// one 16-byte vector: the warp's 32 rows are consecutive pixels of one image
-// row, so in the chunk-planar layout a warp's store of one chunk is contiguous.
-// The others store pairs.  go is warp-uniform (tcgen05.ld is warp-collective).
+// BF16 results are stored an 8-channel chunk of a row at a time, as one 16-byte
+// vector: the warp's 32 rows are consecutive pixels of one image row, so in the
+// chunk-planar layout a warp's store of one chunk is contiguous.  go is warp-uniform (tcgen05.ld is warp-collective).
 template <int BN>
 __device__ __forceinline__ void tc_epilogue(const Epi &e, const Gat &g, unsigned tmem, int m0, int n0, int M,
                                             int warp, int lane, bool go, int ps = 1)
 {
     if (!go) return;
-    const bool vec = e.kind == E_FWD || e.kind == E_DX;
     const int row = warp * 32 + lane, p = m0 + row * ps;
     const size_t prow = (size_t)(p / g.W);
     const int px = p - (int)prow * g.W;
@@ -283,9 +205,12 @@ __device__ __forceinline__ void tc_epilogue(const Epi &e, const Gat &g, unsigned
         asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
         if (p >= M) continue;
         const int col = n0 + c0;
-        if (!vec) {
+        if (e.kind == E_F32) {
+            float4 *d = reinterpret_cast<float4 *>(e.outf + (size_t)p * e.ld0 + col);
 #pragma unroll
-            for (int q = 0; q < 16; q += 2) epi_store(e, g, p, col + q, __uint_as_float(v[q]), __uint_as_float(v[q + 1]));
+            for (int q = 0; q < 4; ++q)
+                d[q] = make_float4(__uint_as_float(v[4 * q]), __uint_as_float(v[4 * q + 1]), __uint_as_float(v[4 * q + 2]),
+                                   __uint_as_float(v[4 * q + 3]));
             continue;
         }
 #pragma unroll
@@ -299,6 +224,16 @@ __device__ __forceinline__ void tc_epilogue(const Epi &e, const Gat &g, unsigned
 #pragma unroll
                 for (int q = 0; q < 8; ++q) f[q] = fmaxf(f[q] + e.bias[cc + q], 0.0f);
                 dst = e.out0 + cofs(prow, px, cc, e.ld0, g.W);
+            } else if (e.kind == E_DOWNDX) {
+                const int z = cc / e.ld0;
+                const size_t o = cofs(2 * prow + (z >> 1), 2 * px + (z & 1), cc - z * e.ld0, e.ld0, 2 * g.W);
+                const uint4 mv = *reinterpret_cast<const uint4 *>(e.mask0 + o);
+                const uint4 av = *reinterpret_cast<const uint4 *>(e.add + o);
+                const bf16 *m = reinterpret_cast<const bf16 *>(&mv), *a = reinterpret_cast<const bf16 *>(&av);
+#pragma unroll
+                for (int q = 0; q < 8; ++q)
+                    f[q] = __bfloat162float(m[q]) > 0.0f ? f[q] + __bfloat162float(a[q]) : 0.0f;
+                dst = e.out0 + o;
             } else if (cc < e.nsplit) {
                 const uint4 mv = *reinterpret_cast<const uint4 *>(e.mask0 + cofs(prow, px, cc, e.ld0, g.W));
                 const bf16 *m = reinterpret_cast<const bf16 *>(&mv);
@@ -316,34 +251,36 @@ __device__ __forceinline__ void tc_epilogue(const Epi &e, const Gat &g, unsigned
     }
 }
 
+// Input gradient of a stride-2 layer: every half-grid pixel's K = 2C output gradients
+// times the 4C x K matrix B (row z C + c: sub-pixel z of the pixel's 2x2 block) gives
+// the C input gradients of its four sub-pixels (E_DOWNDX).  The four sub-pixels are
+// columns of one product, so a pixel is staged once for all of them, and K <= 256
+// fits in shared memory whole.  Bound by the epilogue's traffic (reads the mask and
+// the skip gradient, writes the result: 6 bytes per value); four images of
+// 256 x 512, C = 32: 38 us for 118 MB (105 with a launch plane per sub-pixel and
+// 4-byte accesses).
 template <int BN>
-__global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(Gat g, const bf16 *__restrict__ B, int Kpad, size_t bz,
-                                                          Epi e, int *err)
+__global__ void __launch_bounds__(kTcThreads) k_down_dx(const bf16 *__restrict__ G, int K, int M, int W,
+                                                        const bf16 *__restrict__ B, Epi e, int *err)
 {
     pdl_entry();
     extern __shared__ __align__(1024) unsigned char smem[];
-    using S = TcSmem<BN>;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    unsigned char *bar_base = smem + kTcStages * S::kStage;
-    const unsigned full0 = smem_u32(bar_base), empty0 = full0 + 8 * kTcStages, done = empty0 + 8 * kTcStages;
-    unsigned *tmem_slot = reinterpret_cast<unsigned *>(bar_base + 8 * (2 * kTcStages + 1));
-    const int M = g.N * g.H * g.W;
+    const int KT = K / kTcK;
+    constexpr int kA = kBM * kTcK * 2, kStage = kA + BN * kTcK * 2;
+    unsigned char *bar_base = smem + KT * kStage;
+    const unsigned full = smem_u32(bar_base), done = full + 8;
+    unsigned *tmem_slot = reinterpret_cast<unsigned *>(bar_base + 16);
     const int m0 = blockIdx.x * kBM, n0 = blockIdx.y * BN;
-    B += blockIdx.z * bz;
-    const int KT = Kpad / kTcK;
-    constexpr int kCols = BN < 32 ? 32 : BN;
 
     if (tid == 0) {
-        for (int s = 0; s < kTcStages; ++s) {
-            mbar_init(full0 + 8 * s, 128);
-            mbar_init(empty0 + 8 * s, 1);
-        }
+        mbar_init(full, 128);
         mbar_init(done, 1);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
     if (warp == 4) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tmem_slot)),
-                     "r"(kCols)
+                     "r"(BN)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
     }
@@ -354,89 +291,58 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(Gat g, const bf16 *__
     bool ok = true;
 
     if (warp < 4) {
-        // ---- producers.  A: lane l of warp w stages rows 32 w + 8 s + (l & 7),
-        // s = 0..3, chunks (l >> 3) and (l >> 3) + 4: one warp instruction reads
-        // 8 pixels x 64 contiguous bytes.  B: BN / 16 chunks per thread, 4 rows
-        // x 128 contiguous bytes per warp instruction ----
-        const int hw = g.H * g.W, qh = lane >> 3;
-        int rn[4], ri[4], rj[4];
-        bool rv[4];
+        // ---- staging: thread t takes tile pixel t (a chunk is one contiguous run of
+        // pixels), and of the weights 8 rows x 16 bytes per 8 threads ----
+        const int p = m0 + tid;
+        const bool v = p < M;
+        const size_t row = v ? (size_t)(p / W) : 0;
+        const bf16 *src = G + cofs(row, v ? p - (int)row * W : 0, 0, K, W);
+        for (int kt = 0; kt < KT; ++kt) {
+            unsigned char *As = smem + kt * kStage, *Bs = As + kA;
 #pragma unroll
-        for (int s4 = 0; s4 < 4; ++s4) {
-            const int p = m0 + warp * 32 + 8 * s4 + (lane & 7);
-            rv[s4] = p < M;
-            const int n = rv[s4] ? p / hw : 0, r = p - n * hw;
-            rn[s4] = n;
-            ri[s4] = rv[s4] ? r / g.W : 0;
-            rj[s4] = rv[s4] ? r - ri[s4] * g.W : 0;
-        }
-        int signalled = 0;
-        for (int kt = 0; kt < KT && ok; ++kt) {
-            const int s = kt % kTcStages;
-            if (kt >= kTcStages) ok = mbar_wait(empty0 + 8 * s, ((kt / kTcStages) - 1) & 1);
-            if (!ok) break;
-            unsigned char *As = smem + s * S::kStage, *Bs = As + S::kA;
-            const int k0 = kt * kTcK;
-#pragma unroll
-            for (int s4 = 0; s4 < 4; ++s4) {
-                const int row = warp * 32 + 8 * s4 + (lane & 7);
-                unsigned char *dst = As + ((row >> 3) * 8) * 128 + (row & 7) * 16;
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int q = qh + 4 * h;
-                    const bf16 *src = rv[s4] ? gat_src(g, rn[s4], ri[s4], rj[s4], k0 + q * 8) : nullptr;
-                    cp16(dst + q * 128, src ? src : g.in0, src ? 16 : 0);
-                }
-            }
+            for (int q = 0; q < 8; ++q)
+                cp16(As + ((tid >> 3) * 8 + q) * 128 + (tid & 7) * 16, src + (size_t)(8 * kt + q) * W * 8, v ? 16 : 0);
 #pragma unroll
             for (int rr = 0; rr < BN / 16; ++rr) {
                 const int c = tid + 128 * rr, nn = c >> 3, q = c & 7;
-                cp16(Bs + ((nn >> 3) * 8 + q) * 128 + (nn & 7) * 16, B + (size_t)(n0 + nn) * Kpad + k0 + q * 8, 16);
-            }
-            cp_commit();
-            if (kt >= kTcLag) {
-                cp_wait<kTcLag>();
-                asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-                mbar_arrive(full0 + 8 * ((kt - kTcLag) % kTcStages));
-                signalled = kt - kTcLag + 1;
+                cp16(Bs + ((nn >> 3) * 8 + q) * 128 + (nn & 7) * 16, B + (size_t)(n0 + nn) * K + kt * kTcK + q * 8, 16);
             }
         }
+        cp_commit();
         cp_wait<0>();
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-        if (ok)
-            for (int kt = signalled; kt < KT; ++kt) mbar_arrive(full0 + 8 * (kt % kTcStages));
+        mbar_arrive(full);
     } else if (lane == 0) {
         // ---- MMA issuer ----
         constexpr unsigned idesc = umma_idesc<BN>();
-        for (int kt = 0; kt < KT && ok; ++kt) {
-            const int s = kt % kTcStages;
-            ok = mbar_wait(full0 + 8 * s, (kt / kTcStages) & 1);
-            if (!ok) break;
+        ok = mbar_wait(full, 0);
+        if (ok) {
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-            const unsigned a0 = smem_u32(smem + s * S::kStage), b0 = a0 + S::kA;
+            for (int kt = 0; kt < KT; ++kt) {
+                const unsigned a0 = smem_u32(smem + kt * kStage), b0 = a0 + kA;
 #pragma unroll
-            for (int kk = 0; kk < kTcK / 16; ++kk) {
-                const uint64_t ad = umma_desc(a0 + kk * 256), bd = umma_desc(b0 + kk * 256);
-                const unsigned acc = (kt > 0 || kk > 0) ? 1u : 0u;
-                asm volatile(
-                    "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-                    "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-                    "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
-                    : "memory");
+                for (int kk = 0; kk < kTcK / 16; ++kk) {
+                    const uint64_t ad = umma_desc(a0 + kk * 256), bd = umma_desc(b0 + kk * 256);
+                    const unsigned acc = (kt > 0 || kk > 0) ? 1u : 0u;
+                    asm volatile(
+                        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+                        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
+                        "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
+                        : "memory");
+                }
             }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
-                             empty0 + 8 * s)
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(done)
                          : "memory");
+            if (!mbar_wait(done, 0)) ok = false;  // no MMA in flight past this point
         }
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(done)
-                     : "memory");
-        if (!mbar_wait(done, 0)) ok = false;  // no MMA in flight past this point
     }
 
     if (warp < 4) {
         // ---- epilogue: TMEM lanes 32 warp .. +31 are this warp's rows ----
-        if (ok) ok = mbar_wait(done, 0);
+        ok = mbar_wait(done, 0);
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+        Gat g{};  // the epilogue needs only the row length
+        g.W = W;
         tc_epilogue<BN>(e, g, tmem, m0, n0, M, warp, lane, __all_sync(0xffffffffu, ok));
     }
     if (!ok) atomicExch(err, 1);
@@ -444,7 +350,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(Gat g, const bf16 *__
     __syncthreads();
     if (warp == 4) {
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(kCols) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(BN) : "memory");
     }
 }
 
@@ -1846,13 +1752,6 @@ namespace {
 
 constexpr int kCsumBlocks = 912;   // CTAs of a bias-gradient launch (6 per SM)
 
-int ilog2(int v)
-{
-    int l = 0;
-    while ((1 << l) < v) ++l;
-    return l;
-}
-
 size_t weight_count(int L) { return (size_t)taps(kLayers[L].kind) * kLayers[L].ci * kLayers[L].co; }
 int fwd_K(int L) { return taps(kLayers[L].kind) * cin_pad(kLayers[L].ci); }
 int level_h(const wec_net *N, int l) { return N->H >> l; }
@@ -1875,7 +1774,7 @@ void layer_inputs(const wec_net *N, int L, const bf16 **in0, const bf16 **in1)
     }
 }
 
-// The forward gather of layer L (its input tensors, output grid of its level).
+// Layer L's input tensors and output grid.
 Gat fwd_gather(const wec_net *N, int L, int batch)
 {
     const LayerDef &d = kLayers[L];
@@ -1884,8 +1783,6 @@ Gat fwd_gather(const wec_net *N, int L, int batch)
     layer_inputs(N, L, &g.in0, &g.in1);
     g.c0 = g.in1 ? cinp / 2 : cinp;
     g.c1 = g.in1 ? cinp / 2 : 0;
-    g.lcin = ilog2(cinp);
-    g.kind = d.kind == L_CONV3 ? G_CONV3 : (d.kind == L_UP3 ? G_UP3 : G_DOWN2);
     g.N = batch;
     g.H = H;
     g.W = W;
@@ -1895,42 +1792,40 @@ Gat fwd_gather(const wec_net *N, int L, int batch)
     return g;
 }
 
-
 template <int BN>
-int launch_tc(cudaStream_t st, dim3 grid, const Gat &g, const bf16 *B, int Kpad, size_t bz, const Epi &e, int *err)
+int launch_down_dx(cudaStream_t st, unsigned mt, const bf16 *G, int K, int ncols, int M, int W, const bf16 *B, const Epi &e,
+                   int *err)
 {
+    const int smem = K / kTcK * (kBM + BN) * kTcK * 2 + 256;
     static bool attr = false;  // dynamic shared memory above 48 KB, set once per instantiation
     if (!attr) {
-        WEC_CK(cudaFuncSetAttribute(k_conv_tc<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, TcSmem<BN>::kBytes));
+        WEC_CK(cudaFuncSetAttribute(k_down_dx<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
         attr = true;
     }
-    WEC_CK(launch_k(k_conv_tc<BN>, grid, kTcThreads, TcSmem<BN>::kBytes, st, g, B, Kpad, bz, e, err));
+    WEC_CK(launch_k(k_down_dx<BN>, dim3(mt, (unsigned)(ncols / BN)), kTcThreads, smem, st, G, K, M, W, B, e, err));
     return WEC_OK;
 }
 
-// One convolution GEMM on the tensor cores: B is the K-major weight matrix
-// (ncols rows of Kpad elements; blockIdx.z selects one bz elements further on).
-// Tile width: the widest of 256/128/64/32 dividing ncols that still gives >= 256
-// CTAs (about two per SM), else 32.  tag: the layer index (forward) or 100 +
-// layer (input gradient), reported as the profile level of the launch.
-int gemm(wec_net *N, cudaStream_t st, int tag, const Gat &g, const bf16 *B, int Kpad, size_t bz, int ncols, int nz,
-         const Epi &e)
+// Input gradient of down(l) (profile level 100 + layer) from its output gradient G on
+// the half grid.  Tile width: the widest of 256/128/64/32 dividing the 4C columns
+// that still gives >= 256 CTAs (about two per SM), else 32.
+int down_dx(wec_net *N, int l, int batch, const bf16 *G, const Epi &e)
 {
-    const long long M = (long long)g.N * g.H * g.W;
-    const long long mt = (M + kBM - 1) / kBM;
+    const int C = chans(l), K = 2 * C, ncols = 4 * C, W = level_w(N, l + 1), M = batch * level_h(N, l + 1) * W;
+    const unsigned mt = (unsigned)((M + kBM - 1) / kBM);
     int bn = 32;
     for (int c : {256, 128, 64})
-        if (ncols % c == 0 && mt * (ncols / c) * nz >= 256) {
+        if (ncols % c == 0 && mt * (ncols / c) >= 256) {
             bn = c;
             break;
         }
-    dim3 grid((unsigned)mt, (unsigned)(ncols / bn), (unsigned)nz);
-    WEC_PROF("net_conv", tag, 2.0 * M * nz * ((double)(g.c0 + g.c1) + ncols) + 2.0 * Kpad * ncols * nz, st);
+    const bf16 *B = N->wmat + N->wb[down(l)];
+    WEC_PROF("net_conv", 100 + down(l), 2.0 * M * (K + 3.0 * ncols) + 2.0 * K * ncols, N->st);
     switch (bn) {
-    case 256: return launch_tc<256>(st, grid, g, B, Kpad, bz, e, N->err);
-    case 128: return launch_tc<128>(st, grid, g, B, Kpad, bz, e, N->err);
-    case 64: return launch_tc<64>(st, grid, g, B, Kpad, bz, e, N->err);
-    default: return launch_tc<32>(st, grid, g, B, Kpad, bz, e, N->err);
+    case 256: return launch_down_dx<256>(N->st, mt, G, K, ncols, M, W, B, e, N->err);
+    case 128: return launch_down_dx<128>(N->st, mt, G, K, ncols, M, W, B, e, N->err);
+    case 64: return launch_down_dx<64>(N->st, mt, G, K, ncols, M, W, B, e, N->err);
+    default: return launch_down_dx<32>(N->st, mt, G, K, ncols, M, W, B, e, N->err);
     }
 }
 
@@ -2309,23 +2204,13 @@ int backward(wec_net *N, int batch)
         const int C = chans(l);
         if (l < 3) {
             if (int r = wgrad(N, down(l), batch, N->gA[l + 1])) return r;
-            Gat g{};
-            g.in0 = N->gA[l + 1];
-            g.c0 = 2 * C;
-            g.lcin = ilog2(2 * C);
-            g.kind = G_DIRECT;
-            g.N = batch;
-            g.H = g.Hi = level_h(N, l + 1);
-            g.W = g.Wi = level_w(N, l + 1);
-            g.K = 2 * C;
             Epi e{};
             e.kind = E_DOWNDX;
             e.out0 = N->gA[l];
             e.mask0 = N->act[enc_b(l)];
             e.ld0 = C;
             e.add = N->skip[l];
-            if (int r = gemm(N, st, 100 + down(l), g, N->wmat + N->wb[down(l)], 2 * C, (size_t)2 * C * C, C, 4, e))
-                return r;
+            if (int r = down_dx(N, l, batch, N->gA[l + 1], e)) return r;
         }
         if (int r = wgrad(N, enc_b(l), batch, N->gA[l])) return r;
         Epi e{};

@@ -21,7 +21,7 @@ def built():
     wec.load()
 
 
-@pytest.mark.parametrize("n,h,w", [(3, 312, 520), (1, 8, 1040)])
+@pytest.mark.parametrize("n,h,w", [(3, 312, 520), (1, 8, 1040), (4, 256, 512)])
 def test_rows_of_several_tiles(n, h, w):
     # weights, biases and inputs are short dyadic numbers: the activations are exact on
     # both sides; in the gradients 1 / M is not, and a BF16 rounding falls the other
