@@ -612,7 +612,7 @@ __device__ __forceinline__ void momentum_row(const TankP &P, const MomArgs<R> &M
     const int cv = (blockIdx.y * (TX >> 5) + (threadIdx.x >> 5)) * 31 + lane, i = cv + (C == 0 ? 1 : 0);
     const R *rf = C == 0 ? M.ru : M.rv;
     const double *vin = M.bc.vin0;
-    const bool in = inside2(P, i, j);
+    const bool in = warp_inside(inside2(P, i, j), cv <= ncv);
     R m0 = R(0.0), f0 = R(0.0);
     if (cv <= ncv) {
         if (in)
@@ -714,23 +714,25 @@ __global__ void __launch_bounds__(TX) k_jacobi(TankP P, const R *__restrict__ mu
     const int nx = P.nx, ny = P.ny, i = blockIdx.y * TX + threadIdx.x;
     if ((int)blockIdx.x < ny) {
         const int j = blockIdx.x, f = j * (nx + 1) + i;
+        const bool in = warp_inside(inside2(P, i, j), i > 0 && i < nx);
         if (i > nx) return;
         if (i == 0 || i == nx) {
             ub[f] = ua[f];
             return;
         }
-        const R S = inside2(P, i, j) ? visc_off<true, 0, R>(P, mu_1, nd_1, ua, va, vin1, i, j)
-                                     : visc_off<false, 0, R>(P, mu_1, nd_1, ua, va, vin1, i, j);
+        const R S = in ? visc_off<true, 0, R>(P, mu_1, nd_1, ua, va, vin1, i, j)
+                       : visc_off<false, 0, R>(P, mu_1, nd_1, ua, va, vin1, i, j);
         ub[f] = Ru[f] + Qu[f] * S;
     } else {
         const int j = blockIdx.x - ny, f = j * nx + i;
+        const bool in = warp_inside(inside2(P, i, j), i < nx);
         if (i >= nx) return;
         if (j == 0) {
             vb[f] = va[f];
             return;
         }
-        const R S = inside2(P, i, j) ? visc_off<true, 1, R>(P, mu_1, nd_1, ua, va, vin1, i, j)
-                                     : visc_off<false, 1, R>(P, mu_1, nd_1, ua, va, vin1, i, j);
+        const R S = in ? visc_off<true, 1, R>(P, mu_1, nd_1, ua, va, vin1, i, j)
+                       : visc_off<false, 1, R>(P, mu_1, nd_1, ua, va, vin1, i, j);
         vb[f] = Rv[f] + Qv[f] * S;
     }
 }

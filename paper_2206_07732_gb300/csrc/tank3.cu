@@ -235,39 +235,41 @@ __global__ void __launch_bounds__(128) k3t_materials(Tank3P P, const R *__restri
 // along D around it and its velocity -- so it is formed once and read by the two
 // cells beside it (k3t_advect) instead of once by each.  One 128-thread row per
 // face row (gridf); F and vel in the face layout of component D.
-// (x: the grid covers nx faces per row, the thread of face 0 forming the last
-// one, nx, as well -- an extra block per row would hold one face)
+// (x: a block row covers the ny (nx + 1) faces of a z layer, so that the last face of
+// a row costs no block or second pass of its own)
 template <int D, typename R>
 __global__ void __launch_bounds__(128) k3t_ppm_faces(Tank3P P, const R *__restrict__ s, const R *__restrict__ vel,
                                                      R dt, Ghost3 G, R *__restrict__ F)
 {
     pdl_entry();
     const int nx = P.nx, ny = P.ny, nz = P.nz, nxf = nx + (D == 0), nyf = ny + (D == 1);
-    const int i0 = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y, k = blockIdx.z;
-    if (i0 >= nx) return;
-    const Tank3C<R> &K = cst3<R>(P);
-    const R dtih = dt * K.ih;
+    int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
+    const int k = blockIdx.z;
+    if (D == 0) {
+        j = i / nxf;
+        i -= j * nxf;
+        if (j >= ny) return;
+    } else if (i >= nx) {
+        return;
+    }
+    const R dtih = dt * cst3<R>(P).ih;
     // the face lies below cell (i, j, k) along D; its stencil is the cells -3 .. 2
     // from that cell along D, at fixed offsets (32-bit indices) when all six are
     // inside, else through sig3 (ghost cells)
     constexpr int di = D == 0, dj = D == 1, dk = D == 2;
     const int sd = D == 0 ? 1 : D == 1 ? nx : nx * ny;
-    auto face = [&](int i) {
-        const long long f = ((long long)k * nyf + j) * nxf + i;
-        const int cd = D == 0 ? i : D == 1 ? j : k, nd = D == 0 ? nx : D == 1 ? ny : nz;
-        R a[6];
-        if (cd >= 3 && cd + 2 < nd) {
-            const int c32 = (k * ny + j) * nx + i;
+    const long long f = ((long long)k * nyf + j) * nxf + i;
+    const int cd = D == 0 ? i : D == 1 ? j : k, nd = D == 0 ? nx : D == 1 ? ny : nz;
+    R a[6];
+    if (cd >= 3 && cd + 2 < nd) {
+        const int c32 = (k * ny + j) * nx + i;
 #pragma unroll
-            for (int m = 0; m < 6; ++m) a[m] = s[c32 + (m - 3) * sd];
-        } else {
+        for (int m = 0; m < 6; ++m) a[m] = s[c32 + (m - 3) * sd];
+    } else {
 #pragma unroll
-            for (int m = 0; m < 6; ++m) a[m] = sig3<R>(P, s, i + (m - 3) * di, j + (m - 3) * dj, k + (m - 3) * dk, G);
-        }
-        F[f] = ppm_face3<R>(a, vel[f], dtih);
-    };
-    face(i0);
-    if (D == 0 && i0 == 0) face(nx);
+        for (int m = 0; m < 6; ++m) a[m] = sig3<R>(P, s, i + (m - 3) * di, j + (m - 3) * dj, k + (m - 3) * dk, G);
+    }
+    F[f] = ppm_face3<R>(a, vel[f], dtih);
 }
 
 // out = base - dt Q(u, s), then the damping-zone blend (base = s for the plain
@@ -751,8 +753,9 @@ __global__ void __launch_bounds__(128) k3t_momentum(Tank3P P, MomIn<R> M, R *__r
     pdl_entry();
     int i, j, k;
     long long f;
-    if (!face_of(P, COMP, i, j, k, f)) return;
-    if (interior3(P, i, j, k))
+    const bool use = face_of(P, COMP, i, j, k, f), in = warp_inside(interior3(P, i, j, k), use);
+    if (!use) return;
+    if (in)
         momentum_at<true, R>(P, M, COMP, i, j, k, f, Dout, Rout);
     else
         momentum_at<false, R>(P, M, COMP, i, j, k, f, Dout, Rout);
@@ -775,7 +778,7 @@ __global__ void __launch_bounds__(128, 8) k3t_transport(Tank3P P, MomIn<R> M, R 
     const int ncv = P.nx - (COMP == 0 ? 1 : 0);  // solved faces along x in the row
     const int cv = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 31 + lane;
     const int i = cv + (COMP == 0 ? 1 : 0), j = blockIdx.y + (COMP == 1 ? 1 : 0), k = blockIdx.z + (COMP == 2 ? 1 : 0);
-    const bool in = interior3(P, i, j, k);
+    const bool in = warp_inside(interior3(P, i, j, k), cv <= ncv);
     const R *rfc = M.rfc[COMP];
     R m0 = R(0), f0 = R(0);
     if (cv <= ncv) {
@@ -809,9 +812,17 @@ __global__ void __launch_bounds__(128) k3t_momentum_finish(Tank3P P, MomIn<R> M,
     pdl_entry();
     int i, j, k;
     long long f;
-    if (!face_of(P, COMP, i, j, k, f)) return;
+    bool in;
+    if constexpr (is_f64<R>) {
+        const bool use = face_of(P, COMP, i, j, k, f);
+        in = warp_inside(interior3(P, i, j, k), use);
+        if (!use) return;
+    } else {  // bound by latency rather than arithmetic
+        if (!face_of(P, COMP, i, j, k, f)) return;
+        in = interior3(P, i, j, k);
+    }
     const R rb = Dout[f], C = Rout[f];
-    if (interior3(P, i, j, k))
+    if (in)
         momentum_finish<true, R>(P, M, COMP, i, j, k, f, rb, C, Dout, Rout);
     else
         momentum_finish<false, R>(P, M, COMP, i, j, k, f, rb, C, Dout, Rout);
@@ -859,9 +870,17 @@ __global__ void __launch_bounds__(128) k3t_jacobi(Tank3P P, const R *__restrict_
     pdl_entry();
     int i, j, k;
     long long f;
-    if (!face_of(P, COMP, i, j, k, f)) return;
+    bool in;
+    if constexpr (is_f64<R>) {
+        const bool use = face_of(P, COMP, i, j, k, f);
+        in = warp_inside(interior3(P, i, j, k), use);
+        if (!use) return;
+    } else {  // bound by latency rather than arithmetic
+        if (!face_of(P, COMP, i, j, k, f)) return;
+        in = interior3(P, i, j, k);
+    }
     R S, Lc;
-    if (interior3(P, i, j, k))
+    if (in)
         offdiag3<true, R>(P, mu1, E, A, COMP, i, j, k, S, Lc);
     else
         offdiag3<false, R>(P, mu1, E, A, COMP, i, j, k, S, Lc);
@@ -1211,7 +1230,7 @@ void advect3(const Tank3P &P, const size_t nf[3], const R *base, const R *s, con
     const double nc = (double)P.nx * P.ny * P.nz;
     {
         WEC_PROF("tank3_advect_faces", 0, sizeof(R) * (nc + 2.0 * nf[0]), st);
-        launch_k(k3t_ppm_faces<0, R>, grid3(P), 128, 0, st, P, s, V.u, dt, G, F[0]);
+        launch_k(k3t_ppm_faces<0, R>, dim3((unsigned)(((long long)P.ny * (P.nx + 1) + 127) / 128), 1, P.nz), 128, 0, st, P, s, V.u, dt, G, F[0]);
     }
     {
         WEC_PROF("tank3_advect_faces", 1, sizeof(R) * (nc + 2.0 * nf[1]), st);
