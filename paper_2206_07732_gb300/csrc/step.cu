@@ -350,8 +350,8 @@ __global__ void k_heave(TankP P, StepScalars *S, const double *__restrict__ part
 // SM), so the arithmetic spends as few FP64 instructions as the formulas allow:
 // limiter decisions on the integer pipe (limiters.cuh), face quantities formed
 // once, the viscous operator as a weighted sum.  At 1024x256 in FP64 the step's
-// stencils went from 1.15 to 0.58 ms: advection 243 -> 81 us, a reinitialisation
-// stage 51 -> 34, the momentum system 246 -> 147 (with the face quantities), a
+// stencils went from 1.15 to 0.43 ms: advection 243 -> 63 us, a reinitialisation
+// stage 51 -> 26, the momentum system 246 -> 106 (with the face quantities), a
 // Jacobi sweep 69 -> 18.
 constexpr int TX = 128;  // threads along a row
 inline dim3 row_grid(int nx, int rows) { return dim3(rows, (nx + TX - 1) / TX); }
@@ -359,7 +359,7 @@ inline dim3 row_grid(int nx, int rows) { return dim3(rows, (nx + TX - 1) / TX); 
 // The PPM value of sigma on every x-face (block rows 0 .. ny-1) and y-face (the
 // ny+1 rows after them), time-centred and upwind: a face value depends on the
 // face alone and is read by the two cells beside it.  Formed by each cell for its
-// four faces, advection took 243 us at 1024x256 in FP64; the two kernels take 81.
+// four faces, advection took 243 us at 1024x256 in FP64; the two kernels take 63.
 template <typename R>
 __global__ void __launch_bounds__(TX) k_ppm_faces(TankP P, const R *__restrict__ s, const R *__restrict__ u,
                                                   const R *__restrict__ v, const double *__restrict__ eta0,
@@ -416,6 +416,7 @@ __global__ void __launch_bounds__(TX) k_reinit(TankP P, const R *__restrict__ f,
 {
     pdl_entry();
     const int nx = P.nx, ny = P.ny, i = blockIdx.y * TX + threadIdx.x, j = blockIdx.x;
+    const bool inner = warp_inside(i >= 2 && i < nx - 2 && j >= 2 && j < ny - 2, i < nx);
     if (i >= nx) return;
     const int c0 = j * nx + i;
     const R ih = cst<R>(P).ih, h = cst<R>(P).h, c = f[c0];
@@ -424,7 +425,7 @@ __global__ void __launch_bounds__(TX) k_reinit(TankP P, const R *__restrict__ f,
         sgn[c0] = S = c / sqrt(c * c + h * h);
     else
         S = sgn[c0];
-    const bool pos = positive(S), inner = i >= 2 && i < nx - 2 && j >= 2 && j < ny - 2;
+    const bool pos = positive(S);
     R g2 = R(0.0);
 #pragma unroll
     for (int d = 0; d < 2; ++d) {
@@ -522,9 +523,10 @@ __global__ void __launch_bounds__(TX) k_faces(TankP P, const R *__restrict__ rho
 }
 
 // One face of a momentum control volume of component C (0: u-face, 1: v-face) at
-// (i, j), in direction d, side s (0 lower, 1 upper): the mass flux m = U r and the
-// momentum flux f = m q, r and q the Koren-limited upwind face density and velocity
-// -- rho-breve and the convection share the mass flux.  Side 1 of a CV is side 0 of
+// (i, j), in direction d, side s (0 lower, 1 upper): twice the mass flux, m = U r
+// with U the sum of two d-velocities, and twice the momentum flux, f = m q (the halves
+// are taken once, from the sums over the CV's faces); r and q the Koren-limited upwind
+// face density and velocity -- rho-breve and the convection share the mass flux.  Side 1 of a CV is side 0 of
 // the next one along d, the same values.
 template <bool IN, int C, typename R>
 __device__ __forceinline__ void cv_face(const TankP &P, const R *__restrict__ rf, const R *__restrict__ u,
@@ -539,7 +541,6 @@ __device__ __forceinline__ void cv_face(const TankP &P, const R *__restrict__ rf
     else
         U = d == 0 ? uq2<IN>(P, u, i + s, j - 1) + uq2<IN>(P, u, i + s, j)
                    : vq2<IN>(P, v, vin, i, j + o) + vq2<IN>(P, v, vin, i, j + o + 1);
-    U = R(0.5) * U;
     const int di = d == 0, dj = d;
     R rr[4], qq[4];
 #pragma unroll
@@ -636,8 +637,8 @@ __device__ __forceinline__ void momentum_row(const TankP &P, const MomArgs<R> &M
     const TankC<R> &K = cst<R>(P);
     const R dt = R(M.inp[0]), idt = R(1.0) / dt, ih = K.ih, hi2 = R(0.5) * ih * ih;
     const R r0 = rf[f], w = (C == 0 ? M.u : M.v)[f];
-    const R rb = r0 - dt * ih * ((m1 - m0) + (my[1] - my[0]));
-    const R Cv = ((f1 - f0) + (fy[1] - fy[0])) * ih;
+    const R rb = r0 - R(0.5) * (dt * ih) * ((m1 - m0) + (my[1] - my[0]));
+    const R Cv = ((f1 - f0) + (fy[1] - fy[0])) * (R(0.5) * ih);
     const R chi = R(0.5) * (M.chi_1[cm] + M.chi_1[c]), rbdt = rb * idt;
     const R al = C == 0 ? M.tb.alpha_u[i] : M.tb.alpha_c[i];
     const R D = rbdt + chi * K.ikp + al * rbdt + vort_damp<R>(P, C == 0 ? M.tb.vort_c[j] : M.tb.vort_v[j], idt);

@@ -309,19 +309,16 @@ __global__ void __launch_bounds__(128) k3t_advect(Tank3P P, const R *__restrict_
 // S(sigma0) (|grad f| - 1) at a cell; S = sigma0 / sqrt(sigma0^2 + h^2), formed
 // once per reinitialisation (k3t_reinit_sign).  The one-sided ENO-2 slopes are
 // taken in units of 1/h (a_h = h a) and the Godunov Hamiltonian's squares
-// summed before the single scaling by 1/h^2; max(max(a, 0)^2, min(b, 0)^2) for
+// summed before the single scaling by 1/h; max(max(a, 0)^2, min(b, 0)^2) for
 // S > 0 (mirrored for S <= 0) is the square of the largest of a, -b and 0.
 template <typename R>
 __device__ __forceinline__ R reinit_rhs3(const Tank3P &P, const R *__restrict__ f, const R *__restrict__ sg,
-                                         const Cell3 &q, const Ghost3 &G)
+                                         const Cell3 &q, bool inner, const Ghost3 &G)
 {
     const Tank3C<R> &K = cst3<R>(P);
     const R c = f[q.c];
     const R S = sg[q.c];
     const bool pos = positive(S);
-    // cells two or more from every boundary read their neighbours at fixed
-    // offsets (no ghosts, 32-bit indices); the others through sig3
-    const bool inner = q.i >= 2 && q.i < P.nx - 2 && q.j >= 2 && q.j < P.ny - 2 && q.k >= 2 && q.k < P.nz - 2;
     const int c32 = (int)q.c, st3[3] = {1, P.nx, P.nx * P.ny};
     R g2 = R(0);
 #pragma unroll
@@ -340,24 +337,14 @@ __device__ __forceinline__ R reinit_rhs3(const Tank3P &P, const R *__restrict__ 
             p1 = sig3<R>(P, f, q.i + di, q.j + dj, q.k + dk, G);
             p2 = sig3<R>(P, f, q.i + 2 * di, q.j + 2 * dj, q.k + 2 * dk, G);
         }
-        R a, nb;  // nb = -b
-        if constexpr (is_df<R>) {
-            // float pairs: the second differences from the four first differences
-            // (seven pair subtractions instead of nine operations and two
-            // scalings; the same values to the pairs' rounding)
-            const R em = m1 - m2, e0 = c - m1, e1 = p1 - c, ep = p2 - p1;
-            const R dm = e0 - em, d0 = e1 - e0, dp = ep - e1;
-            a = e0 + scl2<R>(0.5f, mm3(dm, d0));
-            nb = scl2<R>(0.5f, mm3(d0, dp)) - e1;
-        } else {
-            const R dm = m2 - scl2<R>(2.f, m1) + c, d0 = m1 - scl2<R>(2.f, c) + p1, dp = c - scl2<R>(2.f, p1) + p2;
-            a = (c - m1) + scl2<R>(0.5f, mm3(dm, d0));
-            nb = (c - p1) + scl2<R>(0.5f, mm3(d0, dp));
-        }
+        // the three second differences from the four first ones
+        const R em = m1 - m2, e0 = c - m1, e1 = p1 - c, ep = p2 - p1;
+        const R dm = e0 - em, d0 = e1 - e0, dp = ep - e1;
+        const R a = e0 + scl2<R>(0.5f, mm3(dm, d0)), nb = scl2<R>(0.5f, mm3(d0, dp)) - e1;  // nb = -b
         const R m = godunov_max(a, nb, pos);
         g2 += m * m;
     }
-    return S * (sqrt(g2 * K.ih * K.ih) - R(1));
+    return S * (K.ih * sqrt(g2) - R(1));
 }
 
 // S(sigma0) = sigma0 / sqrt(sigma0^2 + h^2) of the field s into s0
@@ -379,8 +366,13 @@ __global__ void __launch_bounds__(128) k3t_reinit_stage(Tank3P P, const R *__res
 {
     pdl_entry();
     Cell3 q;
-    if (!cell_of(P, q)) return;
-    const R y = f[q.c] - dtau * reinit_rhs3<R>(P, f, sg, q, G);
+    const bool use = cell_of(P, q);
+    // cells two or more from every boundary read their neighbours at fixed
+    // offsets (no ghosts, 32-bit indices); the others through sig3
+    bool inner = q.i >= 2 && q.i < P.nx - 2 && q.j >= 2 && q.j < P.ny - 2 && q.k >= 2 && q.k < P.nz - 2;
+    inner = warp_inside(inner, use);
+    if (!use) return;
+    const R y = f[q.c] - dtau * reinit_rhs3<R>(P, f, sg, q, inner, G);
     out[q.c] = stage == 1 ? y : scl2<R>(0.5f, out[q.c] + y);
 }
 
@@ -495,9 +487,10 @@ __device__ __forceinline__ R frq(const Tank3P &P, const R *__restrict__ a, int c
 }
 
 // One face of a momentum control volume -- direction d, side s (0 lower, 1
-// upper) -- of comp's CV at face (i, j, k): its mass flux m = U r and momentum
-// flux f = m q, with U the d-velocity at the CV face and r, q the upwind values of
-// the face density and the velocity.  A CV face is shared by the two CVs beside
+// upper) -- of comp's CV at face (i, j, k): twice its mass flux, m = U r, and twice
+// its momentum flux, f = m q, with U twice the d-velocity at the CV face (a sum of
+// two; the halves are taken once, from the sums over the CV's faces) and r, q the
+// upwind values of the face density and the velocity.  A CV face is shared by the two CVs beside
 // it along d and depends on it alone: side 1 of (i, j, k) is side 0 of the next
 // CV along d, the same values.
 template <bool IN, typename R>
@@ -508,20 +501,20 @@ __device__ __forceinline__ void tface(const Tank3P &P, const R *__restrict__ rfc
     R U;
     if (d == comp) {  // CV faces at the cell centres on either side
         const int o = s - 1;
-        U = comp == 0   ? scl2<R>(0.5f, uq<IN>(P, V.u, i + o, j, k) + uq<IN>(P, V.u, i + o + 1, j, k))
-            : comp == 1 ? scl2<R>(0.5f, vq<IN>(P, V.v, i, j + o, k) + vq<IN>(P, V.v, i, j + o + 1, k))
-                        : scl2<R>(0.5f, wq<IN>(P, V.w, V.win, i, j, k + o) + wq<IN>(P, V.w, V.win, i, j, k + o + 1));
+        U = comp == 0   ? uq<IN>(P, V.u, i + o, j, k) + uq<IN>(P, V.u, i + o + 1, j, k)
+            : comp == 1 ? vq<IN>(P, V.v, i, j + o, k) + vq<IN>(P, V.v, i, j + o + 1, k)
+                        : wq<IN>(P, V.w, V.win, i, j, k + o) + wq<IN>(P, V.w, V.win, i, j, k + o + 1);
     } else {  // CV faces on the edges: the d-velocity averaged over the comp direction
         const int e = s;
         if (d == 0)
-            U = comp == 1 ? scl2<R>(0.5f, uq<IN>(P, V.u, i + e, j - 1, k) + uq<IN>(P, V.u, i + e, j, k))
-                          : scl2<R>(0.5f, uq<IN>(P, V.u, i + e, j, k - 1) + uq<IN>(P, V.u, i + e, j, k));
+            U = comp == 1 ? uq<IN>(P, V.u, i + e, j - 1, k) + uq<IN>(P, V.u, i + e, j, k)
+                          : uq<IN>(P, V.u, i + e, j, k - 1) + uq<IN>(P, V.u, i + e, j, k);
         else if (d == 1)
-            U = comp == 0 ? scl2<R>(0.5f, vq<IN>(P, V.v, i - 1, j + e, k) + vq<IN>(P, V.v, i, j + e, k))
-                          : scl2<R>(0.5f, vq<IN>(P, V.v, i, j + e, k - 1) + vq<IN>(P, V.v, i, j + e, k));
+            U = comp == 0 ? vq<IN>(P, V.v, i - 1, j + e, k) + vq<IN>(P, V.v, i, j + e, k)
+                          : vq<IN>(P, V.v, i, j + e, k - 1) + vq<IN>(P, V.v, i, j + e, k);
         else
-            U = comp == 0 ? scl2<R>(0.5f, wq<IN>(P, V.w, V.win, i - 1, j, k + e) + wq<IN>(P, V.w, V.win, i, j, k + e))
-                          : scl2<R>(0.5f, wq<IN>(P, V.w, V.win, i, j - 1, k + e) + wq<IN>(P, V.w, V.win, i, j, k + e));
+            U = comp == 0 ? wq<IN>(P, V.w, V.win, i - 1, j, k + e) + wq<IN>(P, V.w, V.win, i, j, k + e)
+                          : wq<IN>(P, V.w, V.win, i, j - 1, k + e) + wq<IN>(P, V.w, V.win, i, j, k + e);
     }
     const int a0 = s - 1;  // the stencil runs over (base + a0 - 1 .. base + a0 + 2) along d
     const int di = d == 0, dj = d == 1, dk = d == 2;
@@ -546,14 +539,14 @@ template <bool IN, typename R>
 __device__ __forceinline__ void transport3(const Tank3P &P, const R *__restrict__ rfc, const Vel3<R> &V, int comp,
                                            int i, int j, int k, R dtih, R &rb, R &C)
 {
-    const R ih = cst3<R>(P).ih;
+    const R hih = scl2<R>(0.5f, cst3<R>(P).ih);
     R m[6], f[6];
 #pragma unroll
     for (int d = 0; d < 3; ++d)
 #pragma unroll
         for (int s = 0; s < 2; ++s) tface<IN, R>(P, rfc, V, comp, i, j, k, d, s, m[2 * d + s], f[2 * d + s]);
-    rb = frq<IN>(P, rfc, comp, i, j, k) - dtih * (((m[1] - m[0]) + (m[3] - m[2])) + (m[5] - m[4]));
-    C = (((f[1] - f[0]) + (f[3] - f[2])) + (f[5] - f[4])) * ih;
+    rb = frq<IN>(P, rfc, comp, i, j, k) - scl2<R>(0.5f, dtih) * (((m[1] - m[0]) + (m[3] - m[2])) + (m[5] - m[4]));
+    C = (((f[1] - f[0]) + (f[3] - f[2])) + (f[5] - f[4])) * hih;
 }
 
 // The viscous operator div[mu (grad u + grad u^T)] of component comp at a face,
@@ -802,8 +795,8 @@ __global__ void __launch_bounds__(128, 8) k3t_transport(Tank3P P, MomIn<R> M, R 
     const long long fi = COMP == 0   ? ((long long)k * P.ny + j) * (P.nx + 1) + i
                          : COMP == 1 ? ((long long)k * (P.ny + 1) + j) * P.nx + i
                                      : ((long long)k * P.ny + j) * P.nx + i;
-    Dout[fi] = r0 - M.dtih * (((m1 - m0) + (m[1] - m[0])) + (m[3] - m[2]));
-    Rout[fi] = (((f1 - f0) + (f[1] - f[0])) + (f[3] - f[2])) * cst3<R>(P).ih;
+    Dout[fi] = r0 - scl2<R>(0.5f, M.dtih) * (((m1 - m0) + (m[1] - m[0])) + (m[3] - m[2]));
+    Rout[fi] = (((f1 - f0) + (f[1] - f[0])) + (f[3] - f[2])) * scl2<R>(0.5f, cst3<R>(P).ih);
 }
 template <int COMP, typename R>
 __global__ void __launch_bounds__(128) k3t_momentum_finish(Tank3P P, MomIn<R> M, R *__restrict__ Dout,
