@@ -8,8 +8,8 @@
 // BF16 tensors ([rows][C / 8][W][8]).  The forward convolutions (3x3, nearest
 // upsampling + 3x3, 2x2 stride 2) and the 3x3 input gradients (the 3x3
 // convolution of the output gradient with the flipped, transposed weights) run
-// in the halo kernels (k_conv_rows for the two finest levels, k_conv_halo persistent
-// and warp-specialised, k_conv_halo1 one tile per CTA): a stage holds one input row of
+// in the halo kernels (k_conv_rows where its weights fit, k_conv_halo persistent and
+// warp-specialised, k_conv_halo1 one tile per CTA): a stage holds one input row of
 // one channel chunk, staged by bulk copy, and every horizontal tap reads it through a
 // shifted descriptor; the weights arrive pre-packed by bulk copy.  The stride-2
 // layer's input gradient is one GEMM for all four sub-pixels (k_down_dx).  Weight
@@ -70,7 +70,7 @@ inline size_t round_up_z(size_t a, size_t b) { return (a + b - 1) / b * b; }
 // ----------------------------------------------------------- tile constants --
 constexpr int kBM = 128;     // GEMM rows (pixels, or weight rows in k_wgrad_tc) per CTA
 
-enum EpiKind { E_FWD = 0, E_DX = 1, E_F32 = 2, E_DOWNDX = 3, E_POOL = 4 };
+enum EpiKind { E_FWD = 0, E_DX = 1, E_DOWNDX = 2, E_POOL = 3 };
 
 // The input tensors of a layer and its output grid: channel c < c0 comes from in0,
 // the rest from in1 (concatenation).
@@ -84,7 +84,7 @@ struct Gat {
 
 // Fused epilogue.  E_FWD: out0 = bf16(relu(acc + bias)).  E_DX: input gradient;
 // columns < nsplit: out0 = bf16(acc * (mask0 > 0)), the rest: out1 = bf16(acc).
-// E_F32: outf = acc.  E_DOWNDX: the stride-2 layer's input gradient, column z ld0 + c
+// E_DOWNDX: the stride-2 layer's input gradient, column z ld0 + c
 // channel c at sub-pixel z of each half-grid pixel's 2x2 block:
 // out0 = bf16((acc + add) * (mask0 > 0)).
 // E_POOL (row-block tiles): an upsampling layer's input gradient on the half grid,
@@ -97,7 +97,6 @@ struct Epi {
     int ld0;
     bf16 *out1;
     int ld1, nsplit;
-    float *outf;
     const bf16 *add;
 };
 
@@ -205,14 +204,6 @@ __device__ __forceinline__ void tc_epilogue(const Epi &e, const Gat &g, unsigned
         asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
         if (p >= M) continue;
         const int col = n0 + c0;
-        if (e.kind == E_F32) {
-            float4 *d = reinterpret_cast<float4 *>(e.outf + (size_t)p * e.ld0 + col);
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                d[q] = make_float4(__uint_as_float(v[4 * q]), __uint_as_float(v[4 * q + 1]), __uint_as_float(v[4 * q + 2]),
-                                   __uint_as_float(v[4 * q + 3]));
-            continue;
-        }
 #pragma unroll
         for (int hh = 0; hh < 2; ++hh) {  // two 8-channel chunks
             const int cc = col + 8 * hh;
@@ -684,7 +675,7 @@ __device__ __forceinline__ void pool_epilogue(const Epi &e, unsigned t0, unsigne
     }
 }
 
-// Stride-1 and upsampling convolutions of the two finest levels: a CTA's tile is
+// Stride-1 and upsampling convolutions of the finer levels (rows_bn): a CTA's tile is
 // 128 pixels of R consecutive image rows, with an accumulator per row (two for the
 // column parities of the up mode), and the weights of all taps stay in shared
 // memory.  An input row is staged once and feeds the (up to three) output rows
@@ -1457,29 +1448,6 @@ __global__ void __launch_bounds__(kT) k_head_final(const float *__restrict__ par
         *loss = sh[0] * inv_m;
 }
 
-// Input gradient of an upsampling layer: G(n, i, j, c) = bf16(sum of the 2x2
-// block of tmp (full grid, NHWC FP32) * (low > 0)), low the half-grid input
-// tensor; G and low chunk-planar, the thread index running in their order.
-__global__ void k_up_pool(const float *__restrict__ tmp, const bf16 *__restrict__ low, int N, int h, int w, int C,
-                          bf16 *__restrict__ G)
-{
-    pdl_entry();
-    const long long k = blockIdx.x * (long long)kT + threadIdx.x;
-    const long long total = (long long)N * h * w * C;
-    if (k >= total) return;
-    const int c8 = (int)(k & 7);
-    const long long t = k >> 3;
-    const int j = (int)(t % w);
-    const long long t2 = t / w;
-    const int q = (int)(t2 % (C / 8));
-    const long long row = t2 / (C / 8);
-    const int i = (int)(row % h), n = (int)(row / h), c = 8 * q + c8;
-    const size_t W2 = 2 * (size_t)w;
-    const size_t o = (((size_t)n * 2 * h + 2 * i) * W2 + 2 * j) * C + c;
-    const float s = (tmp[o] + tmp[o + C]) + (tmp[o + W2 * C] + tmp[o + W2 * C + C]);
-    G[k] = __float2bfloat16_rn(__bfloat162float(low[k]) > 0.0f ? s : 0.0f);
-}
-
 // Column sums of a chunk-planar G [rows][C / 8][W][8] (bias gradient): block (q, b)
 // sums chunk q over rows [b rpb, (b + 1) rpb) into part[b][8 q ..], 16 bytes a load.
 __global__ void __launch_bounds__(kT) k_colsum(const bf16 *__restrict__ G, int rows, int W, int C, int rpb,
@@ -1736,7 +1704,6 @@ struct wec_net {
     bf16 *act[wec::kNumLayers] = {};          // layer outputs
     float *out = nullptr;                     // [maxb][H][W]
     bf16 *gA[4] = {}, *gB[4] = {}, *skip[3] = {};  // gradients per level
-    float *tmpf = nullptr;                    // input gradient of the coarsest upsampling layer (its output grid)
     float *part = nullptr;                    // split-K partials of the weight gradients
     size_t part_n = 0;
     float *cpart = nullptr;                   // column-sum / head partials
@@ -1906,15 +1873,16 @@ int launch_halo_cs(int CS, bool down, cudaStream_t st, long long ntiles, const H
 }
 
 // Column-tile width of the row-block kernel (k_conv_rows), or 0 where it does not
-// apply: the two finest levels (below them the weights of all taps do not fit beside
-// a second CTA), the widest tile whose weights take at most 76 KB, and at most 64
-// output columns: 64 -> 128 channels took 49 us against 46 with the one-row tiles,
-// four images of 256 x 512, but with E_POOL, which replaces two passes over an FP32
-// full grid, 27 against 55 + 30.  The up mode only with three stages: with two,
-// 128 -> 64 channels took 25 us against 22.
+// apply: above the coarsest level, the widest tile whose weights take at most 76 KB
+// (beside the staged rows of a second CTA), and as many columns as the layers of the
+// level have outputs -- twice as many lose: 64 -> 128 channels at level 1 took 49 us
+// against 46 with the one-row tiles, four images of 256 x 512.  At level 2,
+// 128 -> 128 channels take 26 us (30).  E_POOL always (level 1: 27 us; an FP32 full
+// grid and a pooling pass took 55 + 30).  The up mode only with three stages: with
+// two, 128 -> 64 channels took 25 us against 22.
 int rows_bn(int mode, int level, int cin, int ncols, bool pool = false)
 {
-    if (mode == H_DOWN2 || level > 1 || (ncols > 64 && !pool)) return 0;
+    if (mode == H_DOWN2 || level > 2 || (ncols > std::max(64, chans(level)) && !pool)) return 0;
     if (mode == H_UP3) return cin == 64 && ncols == 32 ? 32 : 0;
     for (int bn : {64, 32})
         if (ncols % bn == 0 && 9 * cin * bn * 2 <= 76 * 1024) return bn;
@@ -2163,7 +2131,6 @@ int forward(wec_net *N, int batch, const float *x, float *out, const float *targ
 
 int backward(wec_net *N, int batch)
 {
-    cudaStream_t st = N->st;
     for (int l = 0; l < 3; ++l) {  // decoder, last level first; G of dec(l) is in gA[l]
         const int C = chans(l);
         if (int r = wgrad(N, dec(l), batch, N->gA[l])) return r;
@@ -2181,24 +2148,12 @@ int backward(wec_net *N, int batch)
         e.ld1 = C;
         if (int r = dx_conv(N, cat(l), batch, N->gB[l], e)) return r;
         if (int r = wgrad(N, up(l), batch, N->gA[l])) return r;
-        const bf16 *low = l == 2 ? N->act[enc_b(3)] : N->act[dec(l + 1)];
         Epi f{};
         f.ld0 = 2 * C;
-        if (rows_bn(H_CONV3, l, C, 2 * C, true)) {  // the 2x2 sums in the epilogue
-            f.kind = E_POOL;
-            f.out0 = N->gA[l + 1];
-            f.mask0 = low;
-            if (int r = dx_conv(N, up(l), batch, N->gA[l], f)) return r;
-            continue;
-        }
-        f.kind = E_F32;
-        f.outf = N->tmpf;
+        f.kind = E_POOL;  // the 2x2 sums in the epilogue
+        f.out0 = N->gA[l + 1];
+        f.mask0 = l == 2 ? N->act[enc_b(3)] : N->act[dec(l + 1)];
         if (int r = dx_conv(N, up(l), batch, N->gA[l], f)) return r;
-        const int h = level_h(N, l + 1), w = level_w(N, l + 1);
-        const long long n = (long long)batch * h * w * 2 * C;
-        WEC_PROF("net_up_pool", -1, 16.0 * n + 4.0 * n, st);
-        WEC_CK(launch_k(k_up_pool, nblk(n, kT), kT, 0, st, (const float *)N->tmpf, low, batch, h, w, 2 * C,
-                        N->gA[l + 1]));
     }
     for (int l = 3; l >= 0; --l) {  // encoder; G of down(l)'s output is in gA[l + 1]
         const int C = chans(l);
@@ -2376,7 +2331,6 @@ int wec_net_create(int H, int W, int max_batch, void *cuda_stream, wec_net **out
         A((void **)&N->gB[l], 2 * pix(l) * chans(l));
         if (l < 3) A((void **)&N->skip[l], 2 * pix(l) * chans(l));
     }
-    A((void **)&N->tmpf, 4 * pix(2) * 2 * chans(2));
     A((void **)&N->part, 4 * part_n);
     A((void **)&N->cpart, 4 * (size_t)std::max(kCsumBlocks * 8, nblk((long long)P0, kT) * kHeadVals));
     A((void **)&N->xb, 4 * P0 * kInCh);
