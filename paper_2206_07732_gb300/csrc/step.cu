@@ -162,18 +162,45 @@ __device__ __forceinline__ R warp_sum_d(R v)
 }
 
 // eta at x = 0 (for the inflow profile) and at the three ghost columns, at t^n
-// and t^{n+1}: one warp per value, lanes over the wave components.
-__global__ void k_bc_eta(TankP P, const StepScalars *S, const double *__restrict__ inp, Bc bc)
+// and t^{n+1}: one block per value, threads over the wave components.  The blocks of
+// x = 0 also form what the components' velocities share over the rows (bc.comp): FP64
+// transcendentals are some 50 to 80 instructions of a pipe that issues one per 16
+// clocks, so every row of k_bc_rows evaluating them for itself bound that kernel.
+// With these the two kernels went from 53 to 28 us at 1024x256 and from 37 to 24 at
+// 128x64 (64 components, launch gaps included).
+constexpr int kEtaT = 128;
+__global__ void __launch_bounds__(kEtaT) k_bc_eta(TankP P, const StepScalars *S, const double *__restrict__ inp, Bc bc)
 {
     pdl_entry();
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;  // 8 warps: (time, position)
+    __shared__ double sh[kEtaT / 32];
+    const int w = blockIdx.x, lane = threadIdx.x & 31;          // 8 blocks: (time, position)
     const double t = (w & 1) ? S->t + inp[0] : S->t;
     const int pos = w >> 1;                                    // 0: x = 0; 1..3: ghost columns
     const double x = pos == 0 ? 0.0 : (-pos + 0.5) * P.h;
     double e = 0.0;
-    for (int c = lane; c < P.ncomp; c += 32) e += P.amp[c] * cos(P.kw[c] * x - P.omega[c] * t + P.phase[c]);
+    for (int c = threadIdx.x; c < P.ncomp; c += kEtaT) {
+        const double a = P.amp[c], ph = P.kw[c] * x - P.omega[c] * t + P.phase[c];
+        if (pos == 0) {
+            double sn, cs;
+            sincos(ph, &sn, &cs);
+            e += a * cs;
+            const double f = a * P.omega[c] / sinh(P.kw[c] * P.depth);
+            if (w & 1) {
+                bc.comp[c] = f * cs;
+                bc.comp[2 * P.ncomp + c] = f * sn;
+            } else {
+                bc.comp[P.ncomp + c] = f * sn;
+            }
+        } else {
+            e += a * cos(ph);
+        }
+    }
     e = warp_sum_d(e);
-    if (lane) return;
+    if (lane == 0) sh[threadIdx.x >> 5] = e;
+    __syncthreads();
+    if (threadIdx.x) return;
+    e = 0.0;
+    for (int q = 0; q < kEtaT / 32; ++q) e += sh[q];
     if (pos == 0)
         bc.eta_in[w & 1] = e;
     else
@@ -181,49 +208,43 @@ __global__ void k_bc_eta(TankP P, const StepScalars *S, const double *__restrict
 }
 
 // Inflow at x = 0: u_in(y_{j+1/2}, t^{n+1}) and v_in(y_j, t^n), v_in(y_j, t^{n+1}),
-// Airy velocities with Wheeler stretching, blended to zero in the air.  One warp
-// per row j, lanes over the components.
+// Airy velocities with Wheeler stretching, blended to zero in the air.  A block per
+// row j, a warp for each of the three, lanes over the components.
 template <typename R>
-__global__ void k_bc_rows(TankP P, const StepScalars *S, const double *__restrict__ inp, Bc bc)
+__global__ void __launch_bounds__(96) k_bc_rows(TankP P, const StepScalars *S, const double *__restrict__ inp, Bc bc)
 {
     pdl_entry();
-    const int j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (j > P.ny) return;
-    const R t0 = R(S->t), t1 = R(S->t) + R(inp[0]), d = cst<R>(P).depth;
-    R out[3];
-    for (int q = 0; q < 3; ++q) {
-        const R t = q == 1 ? t0 : t1;
-        const R y = q == 0 ? (j + R(0.5)) * cst<R>(P).h : j * cst<R>(P).h;
-        const R e = R(bc.eta_in[q == 1 ? 0 : 1]);
-        const R ys = y < d + e ? y : d + e;
-        const R yp = d * ys / (d + e);
-        R acc = R(0.0);
+    const int j = blockIdx.x, q = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (q == 0 && j == P.ny) return;
+    const R d = cst<R>(P).depth;
+    const R y = q == 0 ? (j + R(0.5)) * cst<R>(P).h : j * cst<R>(P).h;
+    const R e = R(bc.eta_in[q == 1 ? 0 : 1]);
+    const R ys = y < d + e ? y : d + e;
+    const R yp = d * ys / (d + e);
+    R acc = R(0.0);
+    if constexpr (sizeof(R) == 4) {
+        const R t = q == 1 ? R(S->t) : R(S->t) + R(inp[0]);
         for (int c = lane; c < P.ncomp; c += 32) {
             R k = R(P.kw[c]), w = R(P.omega[c]);
             R ph = -w * t + R(P.phase[c]);
-            R ch, sh;  // cosh(k y') / sinh(k d) and sinh(k y') / sinh(k d)
-            if constexpr (sizeof(R) == 4) {
-                // overflow-free in FP32 (k d reaches ~120 for short components)
-                R e1 = exp(k * (yp - d)), e2 = exp(-k * (yp + d)), den = R(1.0) - exp(R(-2.0) * k * d);
-                ch = (e1 + e2) / den;
-                sh = (e1 - e2) / den;
-            } else {
-                R sk = sinh(k * d);
-                ch = cosh(k * yp) / sk;
-                sh = sinh(k * yp) / sk;
-            }
+            // cosh(k y') / sinh(k d) and sinh(k y') / sinh(k d), overflow-free in FP32
+            // (k d reaches ~120 for short components)
+            R e1 = exp(k * (yp - d)), e2 = exp(-k * (yp + d)), den = R(1.0) - exp(R(-2.0) * k * d);
             if (q == 0)
-                acc += R(P.amp[c]) * w * ch * cos(ph);
+                acc += R(P.amp[c]) * w * ((e1 + e2) / den) * cos(ph);
             else
-                acc += R(P.amp[c]) * w * sh * sin(ph);
+                acc += R(P.amp[c]) * w * ((e1 - e2) / den) * sin(ph);
         }
-        acc = warp_sum_d<R>(acc);
-        out[q] = (R(1.0) - heav<R>(y - d - e, cst<R>(P).h)) * acc;
+    } else {
+        const double *f = bc.comp + q * P.ncomp;
+        for (int c = lane; c < P.ncomp; c += 32) {
+            const R ky = P.kw[c] * yp;
+            acc += f[c] * (q == 0 ? cosh(ky) : sinh(ky));
+        }
     }
+    acc = warp_sum_d<R>(acc);
     if (lane) return;
-    if (j < P.ny) bc.uin1[j] = out[0];
-    bc.vin0[j] = out[1];
-    bc.vin1[j] = out[2];
+    (q == 0 ? bc.uin1 : q == 1 ? bc.vin0 : bc.vin1)[j] = (R(1.0) - heav<R>(y - d - e, cst<R>(P).h)) * acc;
 }
 
 // Cell materials from sigma and the body at yc (which = 0: y_c^n, 1: y_c^{n+1}).
@@ -968,7 +989,7 @@ int tank_alloc_and_init(wec_tank *T)
         WEC_CK(cudaMalloc(q, nv * 8));
         WEC_CK(cudaMemset(*q, 0, nv * 8));
     }
-    size_t nbc = (size_t)P.ny + 2 * (P.ny + 1) + 8;
+    size_t nbc = (size_t)P.ny + 2 * (P.ny + 1) + 8 + 3 * (size_t)P.ncomp;
     WEC_CK(cudaMalloc(&T->bcbuf, nbc * 8));
     T->bc.uin1 = T->bcbuf;
     T->bc.vin0 = T->bc.uin1 + P.ny;
@@ -976,6 +997,7 @@ int tank_alloc_and_init(wec_tank *T)
     T->bc.eta0 = T->bc.vin1 + P.ny + 1;
     T->bc.eta1 = T->bc.eta0 + 3;
     T->bc.eta_in = T->bc.eta1 + 3;
+    T->bc.comp = T->bc.eta_in + 2;
     WEC_CK(cudaMalloc(&T->part, kRedBlocks * 8));
     WEC_CK(cudaMalloc(&T->tabs, (size_t)(2 * P.nx + 1 + 2 * P.ny + 1) * 8));
     if (T->opts.precision == WEC_PREC_MIXED) WEC_CK(cudaMalloc(&T->tabs32, (size_t)(2 * P.nx + 1 + 2 * P.ny + 1) * 4));
@@ -1051,11 +1073,11 @@ void enqueue_front_t(wec_tank *T, const Work<R> &W, cudaStream_t st)
     // (1) inflow / ghost data at t^n and t^{n+1}
     {
         WEC_PROF("bc", -1, fb * 8.0, st);
-        launch_k(k_bc_eta, 1, 256, 0, st, P, T->S, T->inp, T->bc);
+        launch_k(k_bc_eta, 8, kEtaT, 0, st, P, T->S, T->inp, T->bc);
     }
     {
         WEC_PROF("bc", -1, fb * (3.0 * P.ny + 2), st);
-        launch_k(k_bc_rows<R>, nblk(P.ny + 1, 2), 64, 0, st, P, T->S, T->inp, T->bc);
+        launch_k(k_bc_rows<R>, P.ny + 1, 96, 0, st, P, T->S, T->inp, T->bc);
     }
     // (2) materials at n, force from p^{n-1/2}, u^n (Eq. int_fh), heave (Eq. newton_u)
     {

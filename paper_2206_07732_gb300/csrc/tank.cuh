@@ -43,6 +43,7 @@ struct Bc {
     double *eta0;  // [3]    eta(-(g+1/2) h, t^n)
     double *eta1;  // [3]    eta(-(g+1/2) h, t^{n+1})
     double *eta_in;  // [2]  eta(0, t^n), eta(0, t^{n+1})
+    double *comp;    // [3][ncomp] a_c omega_c / sinh(k_c d) times cos(ph_c(t^{n+1})), sin(ph_c(t^n)), sin(ph_c(t^{n+1}))
 };
 
 }  // namespace wec

@@ -1173,46 +1173,68 @@ __global__ void k3t_hydrostatic(Tank3P P, const double *__restrict__ rf, double 
 // half-width h (the arithmetic of airy_host) -- u_in(t1) at the cell layers,
 // w_in(t0), w_in(t1) and their mean at the face heights -- into bc (FP64; the
 // host has written the vorticity-damping entries), and all entries narrowed
-// into bcr (nullable).  One warp per layer: rows 0..nz-1 the cells, nz..2nz the
-// faces (both times); the components are split over the lanes.  Evaluated on
-// the host, these ~6 x 10^5 transcendentals per step kept the GPU idle for
-// several milliseconds at the start of every step.
+// into bcr (nullable).  First k3t_inflow_comp, a block per time (t0, t1): eta at
+// x = 0 and what the components' velocities share over the layers, a_c omega_c /
+// sinh(k_c d) times cos and sin of the phase, into comp ([2] eta, then [2][2][ncomp]).
+// Then a block per row (0..nz-1 the cells, nz..2nz the faces), a warp per time, the
+// components over the lanes.  (One kernel with a warp per row evaluated all of it in
+// every row, four rows to an SM: it was bound by the FP64 pipe, and a step at 64x32x32
+// took 20 us more.)
 __device__ __forceinline__ double warp_sum_d(double v)
 {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
-template <typename R>
-__global__ void __launch_bounds__(128) k3t_inflow(Tank3P P, double t0, double t1, double *__restrict__ bc, R *bcr)
+__global__ void __launch_bounds__(128) k3t_inflow_comp(Tank3P P, double t0, double t1, double *__restrict__ comp)
 {
     pdl_entry();
-    const int nz = P.nz, lane = threadIdx.x & 31, row = blockIdx.x * 4 + (threadIdx.x >> 5);
-    if (row > 2 * nz) return;
+    __shared__ double sh[4];
+    const int tt = blockIdx.x;
+    const double t = tt ? t1 : t0;
+    double *cs = comp + 2 + 2 * tt * P.ncomp, *sn = cs + P.ncomp;
+    double e = 0.0;
+    for (int c = threadIdx.x; c < P.ncomp; c += 128) {
+        double s0, c0;
+        sincos(P.phase[c] - P.omega[c] * t, &s0, &c0);
+        const double f = P.amp[c] * P.omega[c] / sinh(P.kw[c] * P.depth);
+        e += P.amp[c] * c0;
+        cs[c] = f * c0;
+        sn[c] = f * s0;
+    }
+    e = warp_sum_d(e);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = e;
+    __syncthreads();
+    if (threadIdx.x == 0) comp[tt] = (sh[0] + sh[1]) + (sh[2] + sh[3]);
+}
+template <typename R>
+__global__ void __launch_bounds__(64) k3t_inflow(Tank3P P, const double *__restrict__ comp, double *__restrict__ bc, R *bcr)
+{
+    pdl_entry();
+    __shared__ double out[2];
+    const int nz = P.nz, lane = threadIdx.x & 31, tt = threadIdx.x >> 5, row = blockIdx.x;
     double *uin1 = bc, *win0 = uin1 + nz, *win1 = win0 + nz + 1, *vc = win1 + nz + 1, *vf = vc + nz,
            *wmean = vf + nz + 1;
     const bool cell = row < nz;
     const int k = cell ? row : row - nz;
     const double z = cell ? (k + 0.5) * P.h : k * P.h, d = P.depth;
-    double out[2] = {0.0, 0.0};
-    for (int tt = 0; tt < (cell ? 1 : 2); ++tt) {
-        const double t = cell || tt == 1 ? t1 : t0;
-        double e = 0.0;  // eta at x = 0
-        for (int c = lane; c < P.ncomp; c += 32) e += P.amp[c] * cos(P.kw[c] * 0.0 - P.omega[c] * t + P.phase[c]);
-        e = warp_sum_d(e);
-        const double zs = z < d + e ? z : d + e, zp = d * zs / (d + e), phi = z - d - e;
+    if (!cell || tt == 1) {  // (the cells at t1 alone)
+        const double e = comp[tt], zs = z < d + e ? z : d + e, zp = d * zs / (d + e), phi = z - d - e;
         const double blend = 1.0 - (phi < -P.h ? 0.0 : phi > P.h ? 1.0
                                     : 0.5 * (1.0 + phi / P.h + sin(kPi3 * phi / P.h) / kPi3));
+        const double *f = comp + 2 + (2 * tt + (cell ? 0 : 1)) * P.ncomp;
         double s = 0.0;
         for (int c = lane; c < P.ncomp; c += 32) {
-            const double kk = P.kw[c], om = P.omega[c], ph = kk * 0.0 - om * t + P.phase[c], sk = sinh(kk * d);
-            s += cell ? P.amp[c] * om * cosh(kk * zp) / sk * cos(ph) : P.amp[c] * om * sinh(kk * zp) / sk * sin(ph);
+            const double kz = P.kw[c] * zp;
+            s += f[c] * (cell ? cosh(kz) : sinh(kz));
         }
-        out[tt] = blend * warp_sum_d(s);
+        s = warp_sum_d(s);
+        if (lane == 0) out[tt] = blend * s;
     }
-    if (lane != 0) return;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
     if (cell) {
-        uin1[k] = out[0];
-        if (bcr) bcr[k] = R(out[0]);
+        uin1[k] = out[1];
+        if (bcr) bcr[k] = R(out[1]);
     } else {
         const double m = 0.5 * (out[0] + out[1]);
         win0[k] = out[0];
@@ -1390,7 +1412,9 @@ static int tank3_step_impl(wec_tank3 *T, Work3<R> &W, double dt, double pto_forc
     for (int k = 0; k < nz; ++k) vc[k] = vort((k + 0.5) * h);
     for (int k = 0; k <= nz; ++k) vf[k] = vort(k * h);
     WEC_CK(cudaMemcpyAsync(T->bc, hb.data(), hb.size() * 8, cudaMemcpyHostToDevice, st));
-    launch_k(k3t_inflow<R>, nblk(2 * nz + 1, 4), 128, 0, st, P, t0, t1, T->bc, f32 ? W.bc : (R *)nullptr);
+    double *const comp = T->bc + 6 * nz + 4;
+    launch_k(k3t_inflow_comp, 2, 128, 0, st, P, t0, t1, comp);
+    launch_k(k3t_inflow<R>, 2 * nz + 1, 64, 0, st, P, (const double *)comp, T->bc, f32 ? W.bc : (R *)nullptr);
     const double *d_win0 = T->bc + nz, *d_win1 = d_win0 + nz + 1;
     const R *r_uin1 = W.bc, *r_win0 = r_uin1 + nz, *r_win1 = r_win0 + nz + 1, *r_vc = r_win1 + nz + 1,
             *r_vf = r_vc + nz;
@@ -1827,7 +1851,7 @@ int wec_tank3_create(const wec_grid3 *grid, const wec_fluids *fl, const wec_wave
                     if (e == cudaSuccess) e = cudaMalloc(&T->uh[c], nf[c] * 8);
             }
         }
-        if (e == cudaSuccess) e = cudaMalloc(&T->bc, (size_t)(6 * nz + 4) * 8);
+        if (e == cudaSuccess) e = cudaMalloc(&T->bc, (size_t)(6 * nz + 4 + 2 + 4 * P.ncomp) * 8);
         if (e == cudaSuccess) e = cudaMalloc(&T->tabs, (size_t)(nx + 1) * 8);
         if (e == cudaSuccess) e = cudaMalloc(&T->part, (size_t)(3 * nz + 1024 + 8) * 8);
         if (e != cudaSuccess) {
