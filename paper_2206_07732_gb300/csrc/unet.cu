@@ -807,7 +807,7 @@ __global__ void __maxnreg__(80)
                 int n, i0, rv, x0;
                 decode(t, n, i0, rv, x0);
                 for (int cc = 0; cc < ncc && ok; ++cc)
-                    for (int q = 0; q < row_count(rv); ++q, ++g) {
+                    for (int q = 0; q < row_count(rv) && ok; ++q, ++g) {
                         const int s = g % NS; // input row first_row + q
                         ok = mbar_wait(full0 + 8 * s, (unsigned)((g / NS) & 1));
                         if (!ok) break;
