@@ -434,7 +434,7 @@ __global__ void __launch_bounds__(kPThreads, 1) k_conv_halo(Halo h, const bf16 *
 
     if (tid == 0) {
         for (int s = 0; s < NS; ++s) {
-            mbar_init(full0 + 8 * s, 129);  // 128 producers + the bulk copies' expect_tx arrival
+            mbar_init(full0 + 8 * s, DOWN ? 129 : 5);  // producers (or their warps) + the bulk copies' expect_tx arrival
             mbar_init(empty0 + 8 * s, 1);
         }
         for (int b = 0; b < 2; ++b) {
@@ -466,6 +466,11 @@ __global__ void __launch_bounds__(kPThreads, 1) k_conv_halo(Halo h, const bf16 *
     if (warp < 4) {
         // ---- producers ----
         long long g = 0, sig = 0;  // stages staged / signalled by this thread
+        // Stages whose slots outside the row are zero for the column tile zx.  (One thread
+        // issuing all of a stage's copies, the zero slots stored again for every stage and
+        // 128 arrivals took 3 % of the network's time.)
+        unsigned zeroed = 0;
+        int zx = -1;
         for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
             int nt, rowid, x0;
             decode(t, nt, rowid, x0);
@@ -473,7 +478,8 @@ __global__ void __launch_bounds__(kPThreads, 1) k_conv_halo(Halo h, const bf16 *
             const bf16 *Bt = Bp + (size_t)nt * h.nst * TH * BN * CS;
             for (int kt = 0; kt < KT && ok; ++kt, ++g) {
                 const int s = (int)(g % NS);
-                if (g >= NS) ok = mbar_wait(empty0 + 8 * s, (unsigned)(((g / NS) - 1) & 1));
+                if (g >= NS)  // (the warp goes on or stops as one)
+                    ok = __all_sync(0xffffffffu, mbar_wait(empty0 + 8 * s, (unsigned)(((g / NS) - 1) & 1)));
                 if (!ok) break;
                 unsigned char *As = smem + s * S::kStage, *Bs = As + S::kA;
                 const int cc = kt / TV, ta = kt - TV * cc, cb = cc * CS;
@@ -498,24 +504,31 @@ __global__ void __launch_bounds__(kPThreads, 1) k_conv_halo(Halo h, const bf16 *
                     // segment of its plane), the others are zero
                     const int xs = max(x0 - 1, 0), xe = min(x0 - 1 + S::kSlots, h.Wi), s0 = xs - (x0 - 1);
                     if (tid == 0) {
-                        const unsigned abytes = row_ok ? (unsigned)(xe - xs) * 16u * CH : 0u;
-                        mbar_expect_tx(full0 + 8 * s, S::kB + abytes);
+                        mbar_expect_tx(full0 + 8 * s, S::kB + (row_ok ? (unsigned)(xe - xs) * 16u * CH : 0u));
                         bulk_g2s(smem_u32(Bs), Bt + (size_t)kt * TH * BN * CS, S::kB, full0 + 8 * s);
-                        if (row_ok)
-                            for (int q = 0; q < CH; ++q)
-                                bulk_g2s(smem_u32(As + q * S::kLBO + s0 * 16),
-                                         tbase + cofs(trow, xs, coff + 8 * q, tC, h.Wi), (unsigned)(xe - xs) * 16u,
-                                         full0 + 8 * s);
                     }
-                    for (int idx = tid; idx < S::kSlots * CH; idx += 128) {
-                        const int q = idx % CH, sl = idx / CH;
-                        if (!(row_ok && sl >= s0 && sl < s0 + (xe - xs)))
-                            *reinterpret_cast<uint4 *>(As + q * S::kLBO + sl * 16) = make_uint4(0u, 0u, 0u, 0u);
+                    if (row_ok && tid >= 32 && tid < 32 + CH) {
+                        const int q = tid - 32;
+                        bulk_g2s(smem_u32(As + q * S::kLBO + s0 * 16), tbase + cofs(trow, xs, coff + 8 * q, tC, h.Wi),
+                                 (unsigned)(xe - xs) * 16u, full0 + 8 * s);
                     }
-                    // only bulk copies (tracked by the byte count) and this thread's
-                    // zero stores: signal at once
-                    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-                    mbar_arrive(full0 + 8 * s);
+                    if (x0 != zx) {
+                        zx = x0;
+                        zeroed = 0;
+                    }
+                    if (!row_ok || !(zeroed >> s & 1)) {
+                        for (int idx = tid; idx < S::kSlots * CH; idx += 128) {
+                            const int q = idx % CH, sl = idx / CH;
+                            if (!(row_ok && sl >= s0 && sl < s0 + (xe - xs)))
+                                *reinterpret_cast<uint4 *>(As + q * S::kLBO + sl * 16) = make_uint4(0u, 0u, 0u, 0u);
+                        }
+                        zeroed |= 1u << s;
+                        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+                    }
+                    // only bulk copies (tracked by the byte count) and the warp's zero
+                    // stores: signal at once
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(full0 + 8 * s);
                     sig = g + 1;
                 } else {
                     if (tid == 0) {
@@ -718,7 +731,7 @@ __global__ void __maxnreg__(80)
 
     if (tid == 0) {
         for (int s = 0; s < NS; ++s) {
-            mbar_init(full0 + 8 * s, 129);  // 128 producers + the bulk copies' expect_tx arrival
+            mbar_init(full0 + 8 * s, 5);  // the producers' warps + the bulk copies' expect_tx arrival
             mbar_init(empty0 + 8 * s, 1);
         }
         for (int q = 0; q < RM; ++q) {  // per output row: accumulator full, and read
@@ -759,10 +772,16 @@ __global__ void __maxnreg__(80)
             mbar_expect_tx(wfull, (unsigned)wbytes);
             bulk_g2s(smem_u32(smem), Bp + (size_t)nt * h.nst * 3 * BN * CS, (unsigned)wbytes, wfull);
         }
+        unsigned zeroed = 0;  // stages whose slots outside the row are zero for the column tile zx
+        int zx = -1;
         int g = 0;
         for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
             int n, i0, rv, x0;
             decode(t, n, i0, rv, x0);
+            if (x0 != zx) {
+                zx = x0;
+                zeroed = 0;
+            }
             const int xs = max(x0 - 1, 0), xe = min(x0 - 1 + 136, h.Wi), s0 = xs - (x0 - 1);
             for (int cc = 0; cc < ncc && ok; ++cc) {
                 const int cb = cc * CS;
@@ -770,26 +789,29 @@ __global__ void __maxnreg__(80)
                 const int tC = cb < h.c0 ? h.c0 : h.c1, coff = cb < h.c0 ? cb : cb - h.c0;
                 for (int q = 0; q < row_count(rv); ++q, ++g) {
                     const int s = g % NS, y = first_row(i0) + q;
-                    if (g >= NS) ok = mbar_wait(empty0 + 8 * s, (unsigned)((g / NS - 1) & 1));
+                    if (g >= NS)  // (the warp goes on or stops as one)
+                        ok = __all_sync(0xffffffffu, mbar_wait(empty0 + 8 * s, (unsigned)((g / NS - 1) & 1)));
                     if (!ok) break;
                     unsigned char *const As = ring + s * S::kStage;
                     const bool row_ok = y >= 0 && y < h.Hi;
-                    if (tid == 0) {
-                        mbar_expect_tx(full0 + 8 * s, row_ok ? (unsigned)(xe - xs) * 16u * CH : 0u);
-                        if (row_ok)
-                            for (int c = 0; c < CH; ++c)
-                                bulk_g2s(smem_u32(As + c * S::kLBO + s0 * 16),
-                                         tbase + cofs((size_t)n * h.Hi + y, xs, coff + 8 * c, tC, h.Wi),
-                                         (unsigned)(xe - xs) * 16u, full0 + 8 * s);
+                    if (tid == 0) mbar_expect_tx(full0 + 8 * s, row_ok ? (unsigned)(xe - xs) * 16u * CH : 0u);
+                    if (row_ok && tid >= 32 && tid < 32 + CH) {
+                        const int c = tid - 32;
+                        bulk_g2s(smem_u32(As + c * S::kLBO + s0 * 16),
+                                 tbase + cofs((size_t)n * h.Hi + y, xs, coff + 8 * c, tC, h.Wi), (unsigned)(xe - xs) * 16u,
+                                 full0 + 8 * s);
                     }
-                    if (!row_ok || s0 > 0 || xe - xs < 136)
+                    if (!row_ok || !(zeroed >> s & 1)) {
                         for (int idx = tid; idx < 136 * CH; idx += 128) {
                             const int c = idx % CH, sl = idx / CH;
                             if (!(row_ok && sl >= s0 && sl < s0 + (xe - xs)))
                                 *reinterpret_cast<uint4 *>(As + c * S::kLBO + sl * 16) = make_uint4(0u, 0u, 0u, 0u);
                         }
-                    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-                    mbar_arrive(full0 + 8 * s);
+                        zeroed |= 1u << s;
+                        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+                    }
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(full0 + 8 * s);
                 }
             }
         }
