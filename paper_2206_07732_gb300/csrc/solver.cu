@@ -728,7 +728,7 @@ __device__ __forceinline__ void block_orth_k(VT *V, long long n, int nk, const V
 // full basis), advances j otherwise, and sets the IF condition.
 // Bound by the FP64 pipe (FP64) or HBM (float pairs over HBM-sized vectors).  Two
 // kernels, one per pass, read the basis twice: 531 us together at 512x256x256 in
-// float pairs where this one takes 318.
+// float pairs where this one takes 330.
 template <int KB, typename VT = double>
 __global__ void __cluster_dims__(kCl, 1, 1)
     __launch_bounds__(KT, KB <= 4 ? (std::is_same<VT, double>::value ? 4 : 5) : KB <= 8 ? 3 : 2)
