@@ -107,6 +107,14 @@ __device__ __forceinline__ void cl_expect(unsigned long long *b, unsigned bytes)
                  "r"(bytes)
                  : "memory");
 }
+// The two halves of a cluster barrier, for the end of the kernel: a CTA's shared memory
+// has to stay until every CTA has made its last access to it.  The halo exchange does
+// not order that: it reaches one CTA further per pass, 2 nu2 - 1 in all on the first
+// level, where the owner of a coarse layer can be half the cluster away (a slab has two
+// layers at least, so a level of two per CTA lies above one on half the CTAs).
+// Arriving before the last pass and waiting behind it hides the barrier.
+__device__ __forceinline__ void cl_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cl_depart() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 // waits for the phase of the given parity, at most about 0.1 s; false if that runs out
 __device__ __forceinline__ bool cl_wait(unsigned long long *b, unsigned parity)
 {
@@ -164,7 +172,7 @@ __global__ void __launch_bounds__(kClThreads, 1)
     auto arm = [&](const ClLevel<T> &v) {
         const unsigned bytes = (unsigned)sizeof(T) * ((v.nx * v.nm) >> 1);
         const int k0 = rank * v.t;
-        if (tid != 0 || v.nct == 1 || k0 >= v.ns) return;
+        if (tid != 0 || v.nct == 1 || k0 >= v.ns || bad) return;  // (no second arrival in an incomplete phase)
         if (rank > 0) cl_expect(hbar, bytes);
         if (k0 + v.t < v.ns) cl_expect(hbar + 1, bytes);
     };
@@ -335,6 +343,7 @@ __global__ void __launch_bounds__(kClThreads, 1)
 #pragma unroll
             for (int col = 0; col < 2; ++col) {
                 const bool fin = !down && q == 0 && s == nu - 1 && col == 1;
+                if (fin && C > 1) cl_arrive();  // (no access to another CTA follows)
 #pragma unroll
                 for (int u = 0; u < K; ++u) {
                     if (m[u].fl < 0) break;
@@ -425,6 +434,15 @@ __global__ void __launch_bounds__(kClThreads, 1)
     }
     if (last == 0 && rank == 0)
         for (int c = tid; c < M.n; c += nt) o[c] = widen_out<OT>(sm[M.oxl + c]);
+    if (C > 1) {
+        const bool last_pass = last > 0 && nu2 > 0 && (M.v[0].nct > 1 || rank == 0);
+        if (!last_pass) cl_arrive();
+        cl_depart();
+        // after an expired wait: the layers still on their way to this CTA (every
+        // CTA has sent its last one; the others have waited for theirs)
+        if (bad)
+            for (int it = 0; it < 100; ++it) __nanosleep(1000);
+    }
 }
 
 int g_cluster_max = 8;  // CTAs per cluster this GPU takes (16 where the occupancy query allows it)
