@@ -357,7 +357,8 @@ int wec_poisson_apply(wec_poisson *P, const double *x, double *y);
  * object's precision (FP32 arithmetic for WEC_PREC_MIXED, FP64 values in/out). */
 int wec_poisson_vcycle(wec_poisson *P, const double *b, double *x);
 /* FGMRES(restart) right-preconditioned by the V-cycle; x: device, guess in,
- * solution out.  Converged when ||b - A x||_2 <= rtol ||b||_2 (true residual). */
+ * solution out.  Converged when ||b - A x||_2 <= rtol ||b||_2 (true residual).
+ * Returns when its work on the stream is complete, as the calls above do. */
 int wec_poisson_solve(wec_poisson *P, const double *b, double *x, double rtol, int max_iters,
                       int *iters, double *final_rel_residual);
 

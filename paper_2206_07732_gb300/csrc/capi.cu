@@ -267,6 +267,7 @@ int wec_pressure_solve(wec_tank *T, const double *rhs, double *p, double rtol, i
     int rc = poisson_solve(&T->solver, rhs, p, rtol, T->opts.max_iters, iters, relres);
     WEC_CK(cudaEventRecord(T->ev_out, T->gst));
     WEC_CK(cudaStreamWaitEvent(T->st, T->ev_out, 0));
+    WEC_CK(cudaStreamSynchronize(T->st));  // (the solve returns at the state its last kernel publishes)
     return rc;
 }
 
@@ -462,7 +463,9 @@ int wec_poisson_solve(wec_poisson *P, const double *b, double *x, double rtol, i
     if (!P || !b || !x) return fail(WEC_ERR_INVALID, "NULL argument");
     if (!P->have_coef) return fail(WEC_ERR_INVALID, "set the coefficients first");
     if (!(rtol > 0.0) || max_iters < 1) return fail(WEC_ERR_INVALID, "rtol must be > 0, max_iters >= 1");
-    return poisson_solve(P, b, x, rtol, max_iters, iters, relres);
+    const int rc = poisson_solve(P, b, x, rtol, max_iters, iters, relres);
+    WEC_CK(cudaStreamSynchronize(P->st));  // (the solve returns at the state its last kernel publishes)
+    return rc;
 }
 
 double wec_wave_number(double omega, double depth, double g) { return wave_number(omega, depth, g); }

@@ -161,7 +161,8 @@ void poisson_free(wec_poisson *P);
 // Level-0 coefficients already in P->L64[0].bu / bv (/ bw in 3D) (device): build coarse levels,
 // FP32 copies, the coarsest inverse and the dense level's matrix (enqueued on st).
 int poisson_build(wec_poisson *P, cudaStream_t st);
-// Host-polled FGMRES solve on P->st.
+// Host-polled FGMRES solve on P->st.  Returns once the deciding kernel has published
+// its state, which that kernel outlives by a moment: x is final in stream order.
 int poisson_solve(wec_poisson *P, const double *b, double *x, double rtol, int maxit, int *iters,
                   double *relres);
 // Record the same solve into the graph being captured on st (conditional nodes).

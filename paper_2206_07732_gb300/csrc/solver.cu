@@ -1784,7 +1784,9 @@ int poisson_solve(wec_poisson *P, const double *b, double *x, double rtol, int m
             if (int e = read_state(P, st)) return e;
         }
     }
-    return solve_result(P, iters, relres);
+    const int rc = solve_result(P, iters, relres);
+    if (rc != WEC_OK && rc != WEC_ERR_NOT_CONVERGED) WEC_CK(cudaStreamSynchronize(st));  // (a step ends here)
+    return rc;
 }
 
 int solve_result(wec_poisson *P, int *iters, double *relres)
