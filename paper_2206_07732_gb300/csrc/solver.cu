@@ -469,11 +469,7 @@ struct KPub {
 __device__ __forceinline__ void publish(const KState *ks, KPub k)
 {
     if (!k.pub) return;
-    static_assert(sizeof(KState) % 8 == 0, "copied in 8-byte words");
-    const unsigned long long *s = reinterpret_cast<const unsigned long long *>(ks);
-    volatile unsigned long long *d = reinterpret_cast<volatile unsigned long long *>(k.pub);
-#pragma unroll
-    for (int q = 0; q < (int)(sizeof(KState) / 8); ++q) d[q] = s[q];
+    *k.pub = *ks;
     __threadfence_system();
     *reinterpret_cast<volatile unsigned *>(k.pub + 1) = k.seq;
 }
