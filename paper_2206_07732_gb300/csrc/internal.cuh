@@ -149,6 +149,7 @@ struct wec_poisson {
     wec::KState *ksh = nullptr; // pinned host mirror
     volatile unsigned *kseq = nullptr;  // pinned, behind it: number of the last state a kernel published there
     unsigned seq = 0;           // number of the state a host-polled solve waits for
+    unsigned sched = 0;         // the process's scheduling flag (cudaDeviceSchedule...)
     size_t bytes = 0;
 };
 

@@ -18,6 +18,7 @@
 #include <cstring>
 #include <map>
 #include <mutex>
+#include <thread>
 #include <tuple>
 
 #include <cooperative_groups.h>
@@ -1353,11 +1354,19 @@ void enqueue_close(wec_poisson *P, const double *b, double *x, unsigned long lon
 
 // Waits for the state the last enqueued deciding kernel publishes (P->seq).  The
 // stream is asked now and then: a launch or device error ends the wait, and a
-// stream that has drained without publishing is an error too.
+// stream that has drained without publishing is an error too.  The process's
+// scheduling flag holds here as it does for a synchronisation: a process that asked
+// to sleep (cudaDeviceScheduleBlockingSync) sleeps until the stream has drained, and
+// only one that asked to spin (cudaDeviceScheduleSpin) never gives its core up.
 int read_state(wec_poisson *P, cudaStream_t st)
 {
+    if (P->sched == cudaDeviceScheduleBlockingSync) {
+        const cudaError_t e = cudaStreamSynchronize(st);
+        if (e != cudaSuccess) return cuda_fail(e, "pressure solve");
+    }
     for (unsigned it = 1; *P->kseq != P->seq; ++it) {
         if (it % 4096) continue;
+        if (P->sched != cudaDeviceScheduleSpin) std::this_thread::yield();
         const cudaError_t e = cudaStreamQuery(st);
         if (e == cudaErrorNotReady) continue;
         if (e != cudaSuccess) return cuda_fail(e, "pressure solve");
@@ -1527,6 +1536,8 @@ int poisson_init(wec_poisson *P, int nx, int ny, int prec, int restart, int nu1,
     WEC_CK(cudaMallocHost(&P->ksh, sizeof(KState) + 8));
     std::memset(P->ksh, 0, sizeof(KState) + 8);
     P->kseq = reinterpret_cast<volatile unsigned *>(P->ksh + 1);
+    WEC_CK(cudaGetDeviceFlags(&P->sched));
+    P->sched &= cudaDeviceScheduleMask;
     P->bytes += ((m + 1) * n + n) * 8 + m * n * 8;
     if (d3) return WEC_OK;  // the 3D V-cycle has no tile shapes to tune
     return poisson_autotune(P, st);

@@ -1,5 +1,8 @@
 """What a host-polled pressure solve leaves behind when it returns."""
 import ctypes as C
+import os
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -55,3 +58,33 @@ def test_stream_has_drained_after_a_tank_solve():
         early += not s.query()
     assert early == 0
     t.close()
+
+
+SLEEPS = """
+import ctypes as C, time
+cu, d = C.CDLL("libcuda.so.1"), C.c_int()
+assert cu.cuInit(0) == 0 and cu.cuDeviceGet(C.byref(d), 0) == 0
+assert cu.cuDevicePrimaryCtxSetFlags_v2(d, 4) == 0  # CU_CTX_SCHED_BLOCKING_SYNC, this process's context
+import torch
+from paper_2206_07732_gb300 import synth, wec
+n = (256, 128, 128)
+b = torch.randn(n[::-1], dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(0))
+P, x = wec.Poisson3(*n), torch.zeros_like(b)
+P.set_coefficients(*[torch.from_numpy(a).cuda() for a in synth.random_coefficients3(*n, seed=1, contrast=10.0)])
+P.solve(b, x, rtol=1e-8)
+w, c = time.perf_counter(), time.thread_time()
+for _ in range(10):
+    x.zero_()
+    P.solve(b, x, rtol=1e-10)
+print((time.thread_time() - c) / (time.perf_counter() - w))
+"""
+
+
+def test_a_process_that_asked_to_sleep_sleeps():
+    # an Arnoldi step of this grid is some 0.8 ms of GPU time and a few dozen launches of
+    # a few us each: a host that sleeps meanwhile uses well under half of its core, one
+    # that spins all of it
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", SLEEPS], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr
+    assert float(r.stdout) < 0.5
