@@ -528,8 +528,8 @@ int wec_jonswap(double Hs, double Tp, double gamma, int ncomp, double *amp, doub
  * rounding.  "mg_autotune" (default 1): when a solver is created, time the fused
  * kernels' tile shapes (64x16, 32x16, 32x8, 16x8) on each level above the cluster's
  * and keep the fastest; 0 uses 64x16 everywhere.  Tuning results are kept per (grid,
- * precision, mg_pre, mg_post) for the life of the process: later solvers of the
- * same shape reuse them (a tile's shape does not change the bits).
+ * precision, mg_pre, mg_post, the cluster's first level) for the life of the process:
+ * later solvers of the same shape reuse them (a tile's shape does not change the bits).
  * "mg_bottom_shift" (default -1, as 0): start the cluster kernel this many levels
  * below the first that fits (0..8, capped at the coarsest).
  * "mg3_bottom" (default 1): the 3D V-cycle runs its coarse levels in one

@@ -1022,7 +1022,7 @@ void vcycle_fused(wec_poisson *P, Level<T> *L, const T *b0, TO *x0, const int *b
 }
 
 bool g_mg_autotune = true;     // wec_set_option "mg_autotune"
-int g_mg_bottom_shift = -1;    // wec_set_option "mg_bottom_shift" (-1: the smallest admissible level)
+int g_mg_bottom_shift = -1;    // wec_set_option "mg_bottom_shift" (-1: as 0)
 
 // Autotuner of the fused level kernels: on each level above the cluster kernel's, time the
 // pre + post pair of every tile shape (3 runs each, CUDA events on the solver's
@@ -1080,14 +1080,14 @@ __global__ void k_fill(long long n, T *a, T v)
     if (c < n) a[c] = v;
 }
 
-// Tuning results per (nx, ny, precision, nu1, nu2), shared by every solver of
-// the process: the first solver of a shape times the candidates, later ones
-// reuse its choices.
+// Tuning results per (nx, ny, precision, nu1, nu2, first level of the cluster kernel),
+// shared by every solver of the process: the first solver of a shape times the
+// candidates, later ones reuse its choices.
 struct TuneResult {
     int tile[kMaxLevels];
 };
 std::mutex g_tune_mu;
-std::map<std::tuple<int, int, int, int, int>, TuneResult> g_tune_cache;
+std::map<std::tuple<int, int, int, int, int, int>, TuneResult> g_tune_cache;
 
 int poisson_autotune(wec_poisson *P, cudaStream_t st)
 {
@@ -1102,7 +1102,7 @@ int poisson_autotune(wec_poisson *P, cudaStream_t st)
     }
     if (!g_mg_autotune || P->bottom_level < 1) return WEC_OK;
     std::lock_guard<std::mutex> lk(g_tune_mu);
-    const auto key = std::make_tuple(P->nx, P->ny, P->prec, P->nu1, P->nu2);
+    const auto key = std::make_tuple(P->nx, P->ny, P->prec, P->nu1, P->nu2, P->bottom_level);
     int *tiles = P->prec == WEC_PREC_FP64 ? P->tile64 : P->tile32;
     auto hit = g_tune_cache.find(key);
     if (hit != g_tune_cache.end()) {

@@ -43,3 +43,22 @@ def test_poisson3_tuner_candidates_all_converge():
     assert len(table) == len(tune.CANDIDATES_3D)
     assert best in tune.CANDIDATES_3D
     assert all(r["iters"] > 0 for r in table)
+
+
+@pytest.mark.parametrize("prec", [wec.PREC_FP64, wec.PREC_MIXED])
+def test_levels_given_back_by_the_cluster_kernel_are_tuned(prec):
+    # a solver whose cluster starts further down has more tile levels than the one of
+    # the same shape before it: they are timed (launches at its creation), once
+    def launches(shift):
+        wec.set_option("mg_bottom_shift", shift)
+        n = wec.launch_count()
+        wec.Poisson(1280, 320, precision=prec).close()
+        return wec.launch_count() - n
+
+    try:
+        first, again = launches(-1), launches(-1)
+        lower, lower_again, back = launches(2), launches(2), launches(-1)
+    finally:
+        wec.set_option("mg_bottom_shift", -1)
+    assert first > 0 and again == 0 and back == 0
+    assert lower > first and lower_again == 0
