@@ -713,12 +713,21 @@ __device__ __forceinline__ void block_orth_k(VT *V, long long n, int nk, const V
     }
 }
 
-// Classical Gram-Schmidt, twice, in one pass over the basis.  With h1_k = v_k . w
-// the second pass's coefficients v_k . (w - sum_l h1_l v_l) are h1_k - sum_l G_kl
-// h1_l, G_kl = v_k . v_l the basis's Gram matrix: every earlier call measured its
-// new column (the dot products below, of the vector as it was stored), so the
-// second pass's dot products need no pass of their own.  w -= sum_k (h1_k + h2_k)
-// v_k leaves u_{j+1} in column j+1 (and its FP32 copy b32 for the next mixed
+// Classical Gram-Schmidt in one pass over the basis, corrected for the basis's own
+// loss of orthogonality.  With h1_k = v_k . w the coefficients of two passes together
+// are, in exact arithmetic, h1_k - sum_{l != k} G_kl h1_l, G_kl = v_k . v_l the basis's
+// Gram matrix: every earlier call measured its new column (the dot products below, of
+// the vector as it was stored), so they need no pass of their own.  What a measured
+// second pass would also take out, and this does not, is the rounding of the first:
+// the new column keeps components of order eps ||w|| / ||u|| along the basis, where
+// two measured passes leave eps.  They are not inherited -- the next column is
+// corrected for them -- and the recurrence A Z = V H does not rest on them; the
+// Givens estimate moves by that relative amount, and a cycle's end forms the true
+// residual.  Columns of the tanks' and of random operators up to a contrast of 1e8
+// have ||w|| / ||u|| of 3 to 40 and orthogonality to 1e-14; with a preconditioner
+// that is the inverse to FP32 it is 1e7, and orthogonality 1e-9: the same number of
+// steps and the same residuals as two measured passes in every case.
+// w -= sum_k h_k v_k leaves u_{j+1} in column j+1 (and its FP32 copy b32 for the next mixed
 // V-cycle), h_{j+1,j} = ||w||, s_{j+1} = 1 / h_{j+1,j}, and column j+1 of G.  The
 // last cluster applies the Givens rotations to column j, counts the iteration,
 // decides whether the cycle ends (converged estimate, iteration cap, breakdown, or
@@ -736,7 +745,7 @@ __global__ void __cluster_dims__(kCl, 1, 1)
     __shared__ double sh[KT / 32][KMAXV];
     __shared__ double bsm[KMAXV];
     __shared__ VT hs[KMAXV];
-    __shared__ double hh[KMAXV];  // h1 + h2, then the rotated column
+    __shared__ double hh[KMAXV];  // the corrected coefficients, then the rotated column
     const int j = ks->j, nk = j + 1, lane = threadIdx.x & 31;
     // a warp per row of G
     for (int k = threadIdx.x >> 5; k < nk; k += KT / 32) {
