@@ -723,10 +723,10 @@ __device__ __forceinline__ void block_orth_k(VT *V, long long n, int nk, const V
 // two measured passes leave eps.  They are not inherited -- the next column is
 // corrected for them -- and the recurrence A Z = V H does not rest on them; the
 // Givens estimate moves by that relative amount, and a cycle's end forms the true
-// residual.  Columns of the tanks' and of random operators up to a contrast of 1e8
-// have ||w|| / ||u|| of 3 to 40 and orthogonality to 1e-14; with a preconditioner
-// that is the inverse to FP32 it is 1e7, and orthogonality 1e-9: the same number of
-// steps and the same residuals as two measured passes in every case.
+// residual.  Random operators up to a contrast of 1e8 have ||w|| / ||u|| of 3 to 40
+// and orthogonality to 1e-14; with a preconditioner that is the inverse to FP32 it is
+// 1e7, and orthogonality 1e-9: the same number of steps and the same residuals as two
+// measured passes wherever the tolerance lies above the attainable residual.
 // w -= sum_k h_k v_k leaves u_{j+1} in column j+1 (and its FP32 copy b32 for the next mixed
 // V-cycle), h_{j+1,j} = ||w||, s_{j+1} = 1 / h_{j+1,j}, and column j+1 of G.  The
 // last cluster applies the Givens rotations to column j, counts the iteration,
