@@ -574,26 +574,32 @@ __device__ __forceinline__ void cv_face(const TankP &P, const R *__restrict__ rf
     f = m * upw3(qq[0], qq[1], qq[2], qq[3], U);
 }
 
-// The viscous operator div[mu (grad u + grad u^T)] of component C at a face:
-// h^2 L_mu(u) = S - Lc u_f, S the sum over the face's neighbours (its own component
-// and the cross terms; nd: node viscosities), Lc the sum of the coefficients (the
+// The viscous operator div[mu (grad u + grad u^T)] of component C at a face, times h^2,
+// in two forms with the same instruction count: as a sum of differences (DIFF: the
+// explicit half, whose rounding then scales with the differences), and as S of
+// h^2 L_mu(u) = S - Lc u_f, the sum over the face's neighbours (its own component and
+// the cross terms; nd: node viscosities), Lc the sum of the coefficients (the
 // diagonal, which the Jacobi splitting moves to the left).
-template <bool IN, int C, typename R>
-__device__ __forceinline__ R visc_off(const TankP &P, const R *__restrict__ mu, const R *__restrict__ nd,
+template <bool IN, int C, bool DIFF, typename R>
+__device__ __forceinline__ R visc_sum(const TankP &P, const R *__restrict__ mu, const R *__restrict__ nd,
                                       const R *__restrict__ u, const R *__restrict__ v, const double *__restrict__ vin,
                                       int i, int j)
 {
     const int nn = P.nx + 1;
     if (C == 0) {
+        const R c = DIFF ? uq2<IN>(P, u, i, j) : R(0.0);
+        auto at = [&](int a, int b) { return DIFF ? uq2<IN>(P, u, a, b) - c : uq2<IN>(P, u, a, b); };
         const R m1 = mu[j * P.nx + i], m0 = mu[j * P.nx + i - 1], n1 = nd[(j + 1) * nn + i], n0 = nd[j * nn + i];
-        return R(2.0) * (m1 * uq2<IN>(P, u, i + 1, j) + m0 * uq2<IN>(P, u, i - 1, j)) +
-               (n1 * ((uq2<IN>(P, u, i, j + 1) + vq2<IN>(P, v, vin, i, j + 1)) - vq2<IN>(P, v, vin, i - 1, j + 1)) +
-                n0 * ((uq2<IN>(P, u, i, j - 1) - vq2<IN>(P, v, vin, i, j)) + vq2<IN>(P, v, vin, i - 1, j)));
+        return R(2.0) * (m1 * at(i + 1, j) + m0 * at(i - 1, j)) +
+               (n1 * (at(i, j + 1) + (vq2<IN>(P, v, vin, i, j + 1) - vq2<IN>(P, v, vin, i - 1, j + 1))) +
+                n0 * (at(i, j - 1) - (vq2<IN>(P, v, vin, i, j) - vq2<IN>(P, v, vin, i - 1, j))));
     }
+    const R c = DIFF ? vq2<IN>(P, v, vin, i, j) : R(0.0);
+    auto at = [&](int a, int b) { return DIFF ? vq2<IN>(P, v, vin, a, b) - c : vq2<IN>(P, v, vin, a, b); };
     const R m1 = mu[min(j, P.ny - 1) * P.nx + i], m0 = mu[(j - 1) * P.nx + i], n1 = nd[j * nn + i + 1], n0 = nd[j * nn + i];
-    return R(2.0) * (m1 * vq2<IN>(P, v, vin, i, j + 1) + m0 * vq2<IN>(P, v, vin, i, j - 1)) +
-           (n1 * ((vq2<IN>(P, v, vin, i + 1, j) + uq2<IN>(P, u, i + 1, j)) - uq2<IN>(P, u, i + 1, j - 1)) +
-            n0 * ((vq2<IN>(P, v, vin, i - 1, j) - uq2<IN>(P, u, i, j)) + uq2<IN>(P, u, i, j - 1)));
+    return R(2.0) * (m1 * at(i, j + 1) + m0 * at(i, j - 1)) +
+           (n1 * (at(i + 1, j) + (uq2<IN>(P, u, i + 1, j) - uq2<IN>(P, u, i + 1, j - 1))) +
+            n0 * (at(i - 1, j) - (uq2<IN>(P, u, i, j) - uq2<IN>(P, u, i, j - 1))));
 }
 template <int C, typename R>
 __device__ __forceinline__ R visc_diag(const TankP &P, const R *__restrict__ mu, const R *__restrict__ nd, int i, int j)
@@ -648,11 +654,11 @@ __device__ __forceinline__ void momentum_row(const TankP &P, const MomArgs<R> &M
     if (in) {
 #pragma unroll
         for (int s = 0; s < 2; ++s) cv_face<true, C, R>(P, rf, M.u, M.v, vin, i, j, 1, s, my[s], fy[s]);
-        S = visc_off<true, C, R>(P, M.mu_n, M.nd_n, M.u, M.v, vin, i, j);
+        S = visc_sum<true, C, true, R>(P, M.mu_n, M.nd_n, M.u, M.v, vin, i, j);
     } else {
 #pragma unroll
         for (int s = 0; s < 2; ++s) cv_face<false, C, R>(P, rf, M.u, M.v, vin, i, j, 1, s, my[s], fy[s]);
-        S = visc_off<false, C, R>(P, M.mu_n, M.nd_n, M.u, M.v, vin, i, j);
+        S = visc_sum<false, C, true, R>(P, M.mu_n, M.nd_n, M.u, M.v, vin, i, j);
     }
     const int f = C == 0 ? j * (nx + 1) + i : j * nx + i, c = min(j, ny - 1) * nx + i, cm = C == 0 ? c - 1 : (j - 1) * nx + i;
     const TankC<R> &K = cst<R>(P);
@@ -663,7 +669,7 @@ __device__ __forceinline__ void momentum_row(const TankP &P, const MomArgs<R> &M
     const R chi = R(0.5) * (M.chi_1[cm] + M.chi_1[c]), rbdt = rb * idt;
     const R al = C == 0 ? M.tb.alpha_u[i] : M.tb.alpha_c[i];
     const R D = rbdt + chi * K.ikp + al * rbdt + vort_damp<R>(P, C == 0 ? M.tb.vort_c[j] : M.tb.vort_v[j], idt);
-    R rhs = r0 * w * idt - Cv + hi2 * (S - visc_diag<C, R>(P, M.mu_n, M.nd_n, i, j) * w);
+    R rhs = r0 * w * idt - Cv + hi2 * S;
     if (C == 0) {
         rhs -= R(M.p[c] - M.p[c - 1]) * ih;
     } else {
@@ -742,8 +748,8 @@ __global__ void __launch_bounds__(TX) k_jacobi(TankP P, const R *__restrict__ mu
             ub[f] = ua[f];
             return;
         }
-        const R S = in ? visc_off<true, 0, R>(P, mu_1, nd_1, ua, va, vin1, i, j)
-                       : visc_off<false, 0, R>(P, mu_1, nd_1, ua, va, vin1, i, j);
+        const R S = in ? visc_sum<true, 0, false, R>(P, mu_1, nd_1, ua, va, vin1, i, j)
+                       : visc_sum<false, 0, false, R>(P, mu_1, nd_1, ua, va, vin1, i, j);
         ub[f] = Ru[f] + Qu[f] * S;
     } else {
         const int j = blockIdx.x - ny, f = j * nx + i;
@@ -753,8 +759,8 @@ __global__ void __launch_bounds__(TX) k_jacobi(TankP P, const R *__restrict__ mu
             vb[f] = va[f];
             return;
         }
-        const R S = in ? visc_off<true, 1, R>(P, mu_1, nd_1, ua, va, vin1, i, j)
-                       : visc_off<false, 1, R>(P, mu_1, nd_1, ua, va, vin1, i, j);
+        const R S = in ? visc_sum<true, 1, false, R>(P, mu_1, nd_1, ua, va, vin1, i, j)
+                       : visc_sum<false, 1, false, R>(P, mu_1, nd_1, ua, va, vin1, i, j);
         vb[f] = Rv[f] + Qv[f] * S;
     }
 }

@@ -50,3 +50,32 @@ def test_one_step_matches_oracle(nx, ny):
     for name, fo, floor in FIELDS:
         a, b = g.get(name), o.get(fo)
         assert np.max(np.abs(a - b)) < 1e-10 * max(np.max(np.abs(b)), floor), name
+
+
+# FP32 stencils where the viscous terms carry the step (mu dt / (rho h^2) from 1e-1 to
+# 1e3; the tanks' is 1e-6): u* = R / D' + Q S is then a weighted mean of neighbouring
+# velocities in some ten FP32 roundings (the mirror of u, four products and their sums,
+# the reciprocal and the two factors, the last sum), 2^-24 of the value each -- the
+# explicit half among them, as long as its rounding scales with the velocity's
+# differences or is no larger than these.
+@pytest.mark.parametrize("n_jacobi", [1, 3])
+@pytest.mark.parametrize("mu", [1e2, 1e4, 1e6])
+def test_fp32_stencils_at_large_viscosity(mu, n_jacobi):
+    nx, ny = 128, 64
+    cfg = synth.tank_small(seed=0)
+    cfg["body"] = None
+    cfg["solver"]["n_jacobi"] = n_jacobi
+    cfg["mu_w"] = cfg["mu_a"] = mu
+    g, o = wec.Tank(cfg, precision=wec.PREC_MIXED), O.OracleTank(cfg)
+    x, y = np.linspace(0.0, 6.0, nx + 1), np.linspace(0.0, 5.0, ny + 1)[:, None]
+    u, v = 0.37 + 0.01 * np.sin(x + y[:-1]), 0.21 + 0.01 * np.cos(y - x[:-1])
+    u[:, -1] = 0.0
+    v[0, :] = 0.0
+    g.set("u", u)
+    o.set(O.F_U, u)
+    g.set("v", v)
+    o.set(O.F_V, v)
+    g.step(cfg["dt"], 0.0)
+    o.step(cfg["dt"], 0.0)
+    a, b = g.get("ustar")[8:-8, 8:-8], o.get(O.F_USTAR)[8:-8, 8:-8]
+    assert np.max(np.abs(a - b)) < 10 * 2.0 ** -24 * np.max(np.abs(b))
