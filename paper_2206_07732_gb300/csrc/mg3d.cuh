@@ -395,6 +395,7 @@ bool vcycle3_unfused(wec_poisson *P, Level<T> *L, const T *b0, T *x0, const int 
                     launch_cluster<T, 3, OT>(M, smem, 1, b, bs, xout, osel, st);
                     return true;
                 }
+                launch_cluster<T, 3, T>(M, smem, 1, b, bs, x, xs, st);
             } else {
                 launch_cluster<T, 3, T>(M, smem, 1, b, bs, x, xs, st);
             }
