@@ -8,10 +8,10 @@
 // BF16 tensors ([rows][C / 8][W][8]).  The forward convolutions (3x3, nearest
 // upsampling + 3x3, 2x2 stride 2) and the 3x3 input gradients (the 3x3
 // convolution of the output gradient with the flipped, transposed weights) run
-// in the halo kernels (k_conv_rows where its weights fit, k_conv_halo persistent and
-// warp-specialised, k_conv_halo1 one tile per CTA): a stage holds one input row of
-// one channel chunk, staged by bulk copy, and every horizontal tap reads it through a
-// shifted descriptor; the weights arrive pre-packed by bulk copy.  The stride-2
+// in the halo kernels (k_conv_rows where its weights fit, else k_conv_halo; both
+// persistent and warp-specialised): a stage holds one input row of one channel chunk,
+// staged by bulk copy, and every horizontal tap reads it through a shifted descriptor;
+// the weights arrive pre-packed by bulk copy.  The stride-2
 // layer's input gradient is one GEMM for all four sub-pixels (k_down_dx).  Weight
 // gradients reduce over pixels, split
 // across CTAs (k_wgrad_tc); their partial tiles are summed in a fixed order, so
@@ -933,202 +933,6 @@ __global__ void __maxnreg__(80)
     }
 }
 
-// One tile per CTA (the schedule for the full-resolution layers with at most 32
-// input channels per tensor, where many short tiles favour more resident CTAs
-// over the persistent kernel's overlap): warps 0-3 stage and then run the
-// epilogue, one thread of warp 4 issues the MMAs.
-template <int BN, int CS, bool DOWN>
-struct HaloSmem1 {
-    using P = HaloSmem<BN, CS, DOWN>;
-    static constexpr int kSlots = P::kSlots, kLBO = P::kLBO, kTH = P::kTH, kA = P::kA, kB = P::kB, kStage = P::kStage;
-    static constexpr int kStages = kStage <= 40 * 1024 ? 4 : 3;
-    static constexpr int kBytes = kStages * kStage + 256;
-};
-
-template <int BN, int CS, bool DOWN>
-__global__ void __launch_bounds__(kTcThreads, 1) k_conv_halo1(Halo h, const bf16 *__restrict__ Bp, Epi e, int *err)
-{
-    pdl_entry();
-    extern __shared__ __align__(1024) unsigned char smem[];
-    using S = HaloSmem1<BN, CS, DOWN>;
-    constexpr int TH = S::kTH, TV = DOWN ? 2 : 3;
-    // cp.async stages a producer keeps in flight before signalling: one stage of
-    // slack between the MMA being waited for and the one being fed
-    constexpr int LAG = S::kStages - 2;
-    constexpr int NS = S::kStages;
-    constexpr int CH = CS / 8;  // 16-byte chunks per halo pixel
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    unsigned char *bar_base = smem + NS * S::kStage;
-    const unsigned full0 = smem_u32(bar_base), empty0 = full0 + 8 * NS, done = empty0 + 8 * NS;
-    unsigned *tmem_slot = reinterpret_cast<unsigned *>(bar_base + 8 * (2 * NS + 1));
-    // The tile: 128 columns from x0 of output row i -- of the input row for the up
-    // mode, whose two accumulators hold the output columns 2 (x0 + r) + b, b = 0, 1
-    // (each tap of either parity reads the half-resolution row one slot apart).
-    const bool up = !DOWN && h.mode == H_UP3;
-    const int xt = blockIdx.x % h.xtiles, rowid = blockIdx.x / h.xtiles;
-    const int i = rowid % h.H, n = rowid / h.H, x0 = xt * kBM;
-    const int nvalid = min(kBM, (up ? h.Wi : h.W) - x0);  // valid tile rows
-    const int n0 = blockIdx.y * BN;
-    const bf16 *Bt = Bp + (size_t)blockIdx.y * h.nst * TH * BN * CS;
-    constexpr int kCols = DOWN ? (BN < 32 ? 32 : BN) : 2 * BN;  // the up mode's two accumulators
-
-    if (tid == 0) {
-        for (int s = 0; s < NS; ++s) {
-            mbar_init(full0 + 8 * s, 129);  // 128 producers + the bulk copy's expect_tx arrival
-            mbar_init(empty0 + 8 * s, 1);
-        }
-        mbar_init(done, 1);
-        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-    }
-    if (warp == 4) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tmem_slot)),
-                     "r"(kCols)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    const unsigned tmem = *tmem_slot;
-    bool ok = true;
-    const int KT = h.nst;
-
-    if (warp < 4) {
-        // ---- producers: the halo row of the stage (8 consecutive threads read one
-        // pixel's CS channels, 16 bytes each); thread 0 also issues the B bulk copy ----
-        int signalled = 0;
-        for (int kt = 0; kt < KT && ok; ++kt) {
-            const int s = kt % NS;
-            if (kt >= NS) ok = mbar_wait(empty0 + 8 * s, ((kt / NS) - 1) & 1);
-            if (!ok) break;
-            unsigned char *As = smem + s * S::kStage, *Bs = As + S::kA;
-            const int cc = kt / TV, ta = kt - TV * cc, cb = cc * CS;
-            int y = DOWN ? 2 * i + ta : i + ta - 1;  // input row (output grid for the up mode)
-            const bool row_ok = y >= 0 && y < (DOWN ? h.Hi : h.H);
-            if (h.mode == H_UP3) y >>= 1;
-            const bf16 *tbase;
-            int tC, coff;
-            if (cb < h.c0) {
-                tbase = h.in0;
-                tC = h.c0;
-                coff = cb;
-            } else {
-                tbase = h.in1;
-                tC = h.c1;
-                coff = cb - h.c0;
-            }
-            const size_t trow = (size_t)n * h.Hi + (row_ok ? y : 0);
-            if (!DOWN) {
-                // slots x0 - 1 + sl of the input row: the columns inside [0, Wi) arrive
-                // by one bulk copy per channel chunk (a contiguous row segment of its
-                // plane), the others are zero
-                const int xs = max(x0 - 1, 0), xe = min(x0 - 1 + S::kSlots, h.Wi), s0 = xs - (x0 - 1);
-                if (tid == 0) {
-                    const unsigned abytes = row_ok ? (unsigned)(xe - xs) * 16u * CH : 0u;
-                    mbar_expect_tx(full0 + 8 * s, S::kB + abytes);
-                    bulk_g2s(smem_u32(Bs), Bt + (size_t)kt * TH * BN * CS, S::kB, full0 + 8 * s);
-                    if (row_ok)
-                        for (int q = 0; q < CH; ++q)
-                            bulk_g2s(smem_u32(As + q * S::kLBO + s0 * 16), tbase + cofs(trow, xs, coff + 8 * q, tC, h.Wi),
-                                     (unsigned)(xe - xs) * 16u, full0 + 8 * s);
-                }
-                for (int idx = tid; idx < S::kSlots * CH; idx += 128) {
-                    const int q = idx % CH, sl = idx / CH;
-                    if (!(row_ok && sl >= s0 && sl < s0 + (xe - xs)))
-                        *reinterpret_cast<uint4 *>(As + q * S::kLBO + sl * 16) = make_uint4(0u, 0u, 0u, 0u);
-                }
-            } else {
-                if (tid == 0) {
-                    mbar_expect_tx(full0 + 8 * s, S::kB);
-                    bulk_g2s(smem_u32(Bs), Bt + (size_t)kt * TH * BN * CS, S::kB, full0 + 8 * s);
-                }
-                for (int idx = tid; idx < S::kSlots * CH; idx += 128) {
-                    const int q = idx % CH, sl = idx / CH;
-                    const int r = sl & (kBM - 1), x = 2 * (x0 + r) + (sl >> 7);  // even / odd input pixels
-                    const bool v = row_ok && x0 + r < h.W;
-                    cp16(As + q * S::kLBO + sl * 16, v ? tbase + cofs(trow, x, coff + 8 * q, tC, h.Wi) : h.in0,
-                         v ? 16 : 0);
-                }
-            }
-            if (!DOWN) {
-                // only bulk copies (tracked by the barrier's byte count) and zero
-                // stores of this thread: signal at once
-                asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-                mbar_arrive(full0 + 8 * s);
-                signalled = kt + 1;
-            } else {
-                cp_commit();
-                if (kt >= LAG) {
-                    cp_wait<LAG>();
-                    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-                    mbar_arrive(full0 + 8 * ((kt - LAG) % NS));
-                    signalled = kt - LAG + 1;
-                }
-            }
-        }
-        cp_wait<0>();
-        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-        if (ok)
-            for (int kt = signalled; kt < KT; ++kt) mbar_arrive(full0 + 8 * (kt % NS));
-    } else if (lane == 0) {
-        // ---- MMA issuer: per stage TH taps x CS / 16 K-steps ----
-        constexpr unsigned idesc = umma_idesc<BN>();
-        for (int kt = 0; kt < KT && ok; ++kt) {
-            const int s = kt % NS;
-            ok = mbar_wait(full0 + 8 * s, (kt / NS) & 1);
-            if (!ok) break;
-            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-            const unsigned a0 = smem_u32(smem + s * S::kStage), b0 = a0 + S::kA;
-            for (int b = 0; b < (up ? 2 : 1); ++b)
-#pragma unroll
-                for (int tb = 0; tb < TH; ++tb) {
-                    // slot offset of the tap: tb (3x3), the even / odd input array (down),
-                    // (b + tb + 1) / 2 (up: output column 2 (x0 + r) + b reads input x0 + r + that - 1)
-                    const int so = DOWN ? tb * kBM : (up ? (b + tb + 1) >> 1 : tb);
-#pragma unroll
-                    for (int kk = 0; kk < CS / 16; ++kk) {
-                        const uint64_t ad = umma_desc_s(a0 + 2 * kk * S::kLBO + so * 16, S::kLBO, 128);
-                        const uint64_t bd = umma_desc_s(b0 + tb * (BN * CS * 2) + 2 * kk * 128, 128, CH * 128);
-                        const unsigned acc = (kt > 0 || tb > 0 || kk > 0) ? 1u : 0u;
-                        asm volatile(
-                            "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-                            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem + b * BN),
-                            "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
-                            : "memory");
-                    }
-                }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
-                             empty0 + 8 * s)
-                         : "memory");
-        }
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(done)
-                     : "memory");
-        if (!mbar_wait(done, 0)) ok = false;  // no MMA in flight past this point
-    }
-
-    if (warp < 4) {
-        if (ok) ok = mbar_wait(done, 0);
-        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-        Gat g{};  // the epilogue needs only the output grid
-        g.N = h.N;
-        g.H = h.H;
-        g.W = h.W;
-        const bool go = __all_sync(0xffffffffu, ok);
-        for (int b = 0; b < (up ? 2 : 1); ++b) {
-            const int ps = up ? 2 : 1, m0 = rowid * h.W + ps * x0 + b;
-            tc_epilogue<BN>(e, g, tmem + b * BN, m0, n0, m0 + ps * nvalid, warp, lane, go, ps);
-        }
-    }
-    if (!ok) atomicExch(err, 1);
-    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-    __syncthreads();
-    if (warp == 4) {
-        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(kCols) : "memory");
-    }
-}
-
-
 // Weight gradient on tcgen05: part[z][k][n] = sum over the pixels of split z of
 // A(p, k) G[p][n], A the layer's forward gather.  The reduction runs over pixels,
 // and a chunk-planar row holds 8 channels of consecutive pixels 16 bytes apart:
@@ -1859,37 +1663,17 @@ int launch_halo_t(cudaStream_t st, long long ntiles, const Halo &h, const bf16 *
     return WEC_OK;
 }
 
-// One tile per CTA (k_conv_halo1): grid (image rows x column tiles of 128, column tiles of BN).
-template <int BN, int CS>
-int launch_halo1_t(cudaStream_t st, const Halo &h, const bf16 *B, const Epi &e, int *err)
-{
-    using S = HaloSmem1<BN, CS, false>;
-    static bool attr = false;  // dynamic shared memory above 48 KB, set once per instantiation
-    if (!attr) {
-        WEC_CK(cudaFuncSetAttribute(k_conv_halo1<BN, CS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    S::kBytes));
-        attr = true;
-    }
-    dim3 grid((unsigned)(h.N * h.H * h.xtiles), (unsigned)(h.ncols / BN));
-    WEC_CK(launch_k(k_conv_halo1<BN, CS, false>, grid, kTcThreads, S::kBytes, st, h, B, e, err));
-    return WEC_OK;
-}
-
 template <int BN>
 int launch_halo_cs(int CS, bool down, cudaStream_t st, long long ntiles, const Halo &h, const bf16 *B, const Epi &e,
                    int *err)
 {
-    // schedule: layers with at most 32 input channels per tensor (full resolution:
-    // many short tiles) one tile per CTA; the others persistent
-    if (!down && CS == 32) return launch_halo1_t<BN, 32>(st, h, B, e, err);
-    if (!down && CS == 16) return launch_halo1_t<BN, 16>(st, h, B, e, err);
+    // (stride-1 and upsampling layers of at most 32 channels per tensor are the
+    // row-block kernel's, rows_bn)
     if (down) {
         if (CS == 64) return launch_halo_t<BN, 64, true>(st, ntiles, h, B, e, err);
         if (CS == 32) return launch_halo_t<BN, 32, true>(st, ntiles, h, B, e, err);
-    } else {
-        if (CS == 64) return launch_halo_t<BN, 64, false>(st, ntiles, h, B, e, err);
-        if (CS == 32) return launch_halo_t<BN, 32, false>(st, ntiles, h, B, e, err);
-        if (CS == 16) return launch_halo_t<BN, 16, false>(st, ntiles, h, B, e, err);
+    } else if (CS == 64) {
+        return launch_halo_t<BN, 64, false>(st, ntiles, h, B, e, err);
     }
     return fail(WEC_ERR_INVALID, "net: unsupported channels per stage");
 }
