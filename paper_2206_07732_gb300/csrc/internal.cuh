@@ -32,6 +32,19 @@ int cuda_fail(cudaError_t e, const char *what);
 
 inline int nblk(long long n, int t) { return (int)((n + t - 1) / t); }
 
+// SMs of the device the process computes on (152 on a whole GB300), asked once
+inline int sm_count()
+{
+    static const int n = [] {
+        int dev = 0, v = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v < 1)
+            v = 152;
+        return v;
+    }();
+    return n;
+}
+
 // Programmatic dependent launch.  Every kernel of the library starts with
 // pdl_entry(), which waits until the previous kernel on the stream has
 // completed and its writes are visible -- the same ordering as plain stream

@@ -1229,7 +1229,7 @@ int set_kgrid_max()
 // final reduction.
 int kgrid(long long n, int gmax)
 {
-    if (n <= (1ll << 20)) gmax = std::min(gmax, 2 * 152);
+    if (n <= (1ll << 20)) gmax = std::min(gmax, 2 * sm_count());
     const long long g = std::min<long long>(nblk(n, KT), gmax);
     return (int)((g + kCl - 1) / kCl * kCl);
 }

@@ -1263,7 +1263,7 @@ dim3 gridf(const Tank3P &P, int comp)
 int march_layers(dim3 &g)
 {
     int nk = 8;
-    while (nk > 1 && (long long)g.x * g.y * ((g.z + nk - 1) / nk) < 152 * 16) nk /= 2;
+    while (nk > 1 && (long long)g.x * g.y * ((g.z + nk - 1) / nk) < sm_count() * 16) nk /= 2;
     g.z = (g.z + nk - 1) / nk;
     return nk;
 }

@@ -1651,12 +1651,10 @@ int launch_halo_t(cudaStream_t st, long long ntiles, const Halo &h, const bf16 *
     if (!ctas) {
         WEC_CK(cudaFuncSetAttribute(k_conv_halo<BN, CS, DOWN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     S::kBytes));
-        int dev = 0, sms = 0, occ = 0;
-        WEC_CK(cudaGetDevice(&dev));
-        WEC_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        int occ = 0;
         WEC_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_conv_halo<BN, CS, DOWN>, kPThreads, S::kBytes));
         const int cols = DOWN ? 2 * BN : 4 * BN;
-        ctas = sms * std::max(1, std::min(occ, 512 / cols));
+        ctas = sm_count() * std::max(1, std::min(occ, 512 / cols));
     }
     const unsigned grid = (unsigned)std::min<long long>(ntiles, ctas);
     WEC_CK(launch_k(k_conv_halo<BN, CS, DOWN>, grid, kPThreads, S::kBytes, st, h, B, e, err));
@@ -1706,7 +1704,7 @@ int launch_rows_t(cudaStream_t st, const Halo &h, const bf16 *B, const Epi &e, i
         WEC_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 113 * 1024));
         attr = true;
     }
-    const int ntn = h.ncols / BN, slots = 2 * 152 / ntn;
+    const int ntn = h.ncols / BN, slots = std::max(1, 2 * sm_count() / ntn);
     // rows per tile: as many as the accumulators hold, fewer where the tiles would not fill the GPU
     int R = S::kRows;
     auto tiles = [&](int r) { return (long long)h.N * ((h.H + r - 1) / r) * h.xtiles; };
@@ -1776,7 +1774,7 @@ int wgrad_max_splits(long long units, int L)
 {
     const WgShape w = wgrad_shape(L);
     const int tiles = (w.rows + 127) / 128 * (kLayers[L].co / w.bn);
-    return (int)std::min<long long>(std::max(1, 152 * w.occ / tiles), units);
+    return (int)std::min<long long>(std::max(1, sm_count() * w.occ / tiles), units);
 }
 int wgrad_splits(long long units, int L, int *ups)
 {
