@@ -1629,13 +1629,19 @@ inline bool halo_bwd(int L) { return L != enc_a(0) && (kLayers[L].kind == L_CONV
 inline int halo_kin(int L, bool bwd) { return bwd ? kLayers[L].co : cin_pad(kLayers[L].ci); }
 inline int halo_mode(int kind) { return kind == L_UP3 ? H_UP3 : (kind == L_DOWN2 ? H_DOWN2 : H_CONV3); }
 
+// one-row tiles of an image; the up mode tiles the half-resolution row
+long long halo_tiles(const wec_net *N, int level, bool up)
+{
+    const int w = up ? level_w(N, level) / 2 : level_w(N, level);
+    return (long long)level_h(N, level) * ((w + kBM - 1) / kBM);
+}
+
 // Column-tile width: the widest of 128 / 64 dividing ncols that still gives >= 128
 // tiles for one image (measured: wider tiles beat more, narrower ones down to
 // about one tile per SM), else 32.  The up mode tiles the half-resolution row.
 int halo_bn(const wec_net *N, int level, int ncols, bool up = false)
 {
-    const int w = up ? level_w(N, level) / 2 : level_w(N, level);
-    const long long tiles = (long long)level_h(N, level) * ((w + kBM - 1) / kBM);
+    const long long tiles = halo_tiles(N, level, up);
     for (int c : {128, 64})
         if (ncols % c == 0 && tiles * (ncols / c) >= 128) return c;
     return 32;
@@ -1665,13 +1671,13 @@ template <int BN>
 int launch_halo_cs(int CS, bool down, cudaStream_t st, long long ntiles, const Halo &h, const bf16 *B, const Epi &e,
                    int *err)
 {
-    // (stride-1 and upsampling layers of at most 32 channels per tensor are the
-    // row-block kernel's, rows_bn)
     if (down) {
         if (CS == 64) return launch_halo_t<BN, 64, true>(st, ntiles, h, B, e, err);
         if (CS == 32) return launch_halo_t<BN, 32, true>(st, ntiles, h, B, e, err);
-    } else if (CS == 64) {
-        return launch_halo_t<BN, 64, false>(st, ntiles, h, B, e, err);
+    } else {
+        if (CS == 64) return launch_halo_t<BN, 64, false>(st, ntiles, h, B, e, err);
+        if (CS == 32) return launch_halo_t<BN, 32, false>(st, ntiles, h, B, e, err);
+        if (CS == 16) return launch_halo_t<BN, 16, false>(st, ntiles, h, B, e, err);
     }
     return fail(WEC_ERR_INVALID, "net: unsupported channels per stage");
 }
@@ -1683,10 +1689,16 @@ int launch_halo_cs(int CS, bool down, cudaStream_t st, long long ntiles, const H
 // against 46 with the one-row tiles, four images of 256 x 512.  At level 2,
 // 128 -> 128 channels take 26 us (30).  E_POOL always (level 1: 27 us; an FP32 full
 // grid and a pooling pass took 55 + 30).  The up mode only with three stages: with
-// two, 128 -> 64 channels took 25 us against 22.
-int rows_bn(int mode, int level, int cin, int ncols, bool pool = false)
+// two, 128 -> 64 channels took 25 us against 22.  And only where the one-row tiles of
+// the largest batch are more than the SMs: up to there each has a CTA of its own, and
+// half as many CTAs with twice the work lose -- 64 -> 64 channels at 32 x 64 to 64 x
+// 128 pixels 13 us against 10, 128 -> 128 at 16 x 32 15 against 12, a forward pass at
+// 64 x 128 200 against 170 (E_POOL has the row blocks alone).
+int rows_bn(const wec_net *N, int mode, int level, int cin, int ncols, bool pool = false)
 {
     if (mode == H_DOWN2 || level > 2 || (ncols > std::max(64, chans(level)) && !pool)) return 0;
+    const bool up = mode == H_UP3;
+    if (!pool && N->maxb * halo_tiles(N, level, up) * (ncols / halo_bn(N, level, ncols, up)) <= sm_count()) return 0;
     if (mode == H_UP3) return cin == 64 && ncols == 32 ? 32 : 0;
     for (int bn : {64, 32})
         if (ncols % bn == 0 && 9 * cin * bn * 2 <= 76 * 1024) return bn;
@@ -1749,7 +1761,7 @@ int conv_halo(wec_net *N, cudaStream_t st, int tag, int mode, int batch, int lev
     const long long ntiles = (long long)batch * h.H * h.xtiles * (ncols / BN);
     const double M = (double)batch * h.H * h.W;
     WEC_PROF("net_conv", tag, 2.0 * M * ((double)(h.c0 + h.c1) + ncols) + 2.0 * tv * tv * (h.c0 + h.c1) * ncols, st);
-    if (rows_bn(mode, level, h.c0 + h.c1, ncols, e.kind == E_POOL)) return launch_rows(BN, CS, st, h, B, e, N->err);
+    if (rows_bn(N, mode, level, h.c0 + h.c1, ncols, e.kind == E_POOL)) return launch_rows(BN, CS, st, h, B, e, N->err);
     switch (BN) {
     case 128: return launch_halo_cs<128>(CS, mode == H_DOWN2, st, ntiles, h, B, e, N->err);
     case 64: return launch_halo_cs<64>(CS, mode == H_DOWN2, st, ntiles, h, B, e, N->err);
@@ -2098,13 +2110,13 @@ int wec_net_create(int H, int W, int max_batch, void *cuda_stream, wec_net **out
             nw = round_up_z(nw + weight_count(L), 64);
         }
         if (halo_fwd(L)) {
-            N->bnf[L] = rows_bn(halo_mode(d.kind), d.level, cin_pad(d.ci), d.co);
+            N->bnf[L] = rows_bn(N, halo_mode(d.kind), d.level, cin_pad(d.ci), d.co);
             if (!N->bnf[L]) N->bnf[L] = halo_bn(N, d.level, d.co, d.kind == L_UP3);
             N->hf[L] = nw;
             nw = round_up_z(nw + (size_t)taps(d.kind) * halo_kin(L, false) * d.co, 64);
         }
         if (halo_bwd(L)) {
-            N->bnb[L] = rows_bn(H_CONV3, d.level, d.co, d.ci, d.kind == L_UP3);
+            N->bnb[L] = rows_bn(N, H_CONV3, d.level, d.co, d.ci, d.kind == L_UP3);
             if (!N->bnb[L]) N->bnb[L] = halo_bn(N, d.level, d.ci);
             N->hb[L] = nw;
             nw = round_up_z(nw + 9 * (size_t)halo_kin(L, true) * d.ci, 64);
