@@ -7,7 +7,8 @@
 // axis (z in 3D, y in 2D), one CTA each, with one halo layer on either side; a
 // colour pass updates the CTA's own cells and stores those of its first and last
 // layer into the neighbour's halo through distributed shared memory, and waits
-// for theirs.  Slabs have an even number of layers, so the children
+// for theirs -- which orders a CTA with its neighbours alone, so the kernel ends in a
+// cluster barrier (cl_arrive).  Slabs have an even number of layers, so the children
 // of a coarse cell lie in one CTA, which restricts them into the b of the CTA
 // that owns the coarse layer; the prolongation reads the coarse iterate from its
 // owner.  FP32 levels of at most kClSingle cells run in CTA 0 alone, with block

@@ -33,7 +33,7 @@ __device__ __forceinline__ T offsum_at(const T *bu, const T *bv, const TX *x, in
 }
 
 // a * b + c rounded once, written out: the 3D multigrid forms the same terms in
-// its per-level kernels and in its one-CTA coarse levels, and left to the
+// its per-level kernels and in its coarse levels' cluster, and left to the
 // compiler the contraction of a product into a sum differs between them
 template <typename T>
 __device__ __forceinline__ T fma3(T a, T b, T c)

@@ -11,7 +11,7 @@
 //   Eqs. ls_flow, ls_solid, Hflow, Hbody .. materials (k_materials)
 //   Eq. c_discrete_momentum .. consistent mass/momentum transport, Crank-Nicolson
 //                           viscosity, flow-density gravity, implicit Brinkman term
-//                           (Eq. bp_discrete) (k_mom_u, k_mom_v, k_jacobi)
+//                           (Eq. bp_discrete) (k_momentum, k_jacobi)
 //   Eq. spongelayer ....... vorticity damping over the top four cells
 //   Section "Numerical wave tank" .. Airy inflow at x = 0, wave damping zone
 //   Eq. c_discrete_continuity .. incremental projection (k_proj_rhs, solver, k_project)
@@ -370,7 +370,7 @@ __global__ void k_heave(TankP P, StepScalars *S, const double *__restrict__ part
 // FP64 every one of them is bound by the FP64 pipe (two operations per clock and
 // SM), so the arithmetic spends as few FP64 instructions as the formulas allow:
 // limiter decisions on the integer pipe (limiters.cuh), face quantities formed
-// once, the viscous operator as a weighted sum.  At 1024x256 in FP64 the step's
+// once, the viscous coefficients shared by its two forms.  At 1024x256 in FP64 the step's
 // stencils went from 1.15 to 0.43 ms: advection 243 -> 63 us, a reinitialisation
 // stage 51 -> 26, the momentum system 246 -> 106 (with the face quantities), a
 // Jacobi sweep 69 -> 18.

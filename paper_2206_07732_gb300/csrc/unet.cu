@@ -8,8 +8,8 @@
 // BF16 tensors ([rows][C / 8][W][8]).  The forward convolutions (3x3, nearest
 // upsampling + 3x3, 2x2 stride 2) and the 3x3 input gradients (the 3x3
 // convolution of the output gradient with the flipped, transposed weights) run
-// in the halo kernels (k_conv_rows where its weights fit, else k_conv_halo; both
-// persistent and warp-specialised): a stage holds one input row of one channel chunk,
+// in the halo kernels (k_conv_rows where its weights fit and the image fills the GPU,
+// else k_conv_halo; both persistent and warp-specialised): a stage holds one input row of one channel chunk,
 // staged by bulk copy, and every horizontal tap reads it through a shifted descriptor;
 // the weights arrive pre-packed by bulk copy.  The stride-2
 // layer's input gradient is one GEMM for all four sub-pixels (k_down_dx).  Weight
